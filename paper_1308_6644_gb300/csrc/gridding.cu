@@ -1772,16 +1772,16 @@ nuasm_status run_binning_lattice(nuasm_plan_s* P, const LatticeSpec& lat, cudaSt
     const Geometry& g = P->g;
     const BinArgs a{g.n, g.W, g.T, g.ntx, g.w, g.h, P->p.pitch, P->m};
     const int nt = g.ntiles, ntx = g.ntx, nx = lat.nx, ny = lat.ny;
-    // scratch: l0x, l0y (int), fx, fy (double), rx, ry (int4)
+    // scratch: rx, ry (int4, first: 16-byte aligned whatever nx + ny), fx, fy (double), l0x, l0y (int)
     const size_t bi = sizeof(int) * (size_t(nx) + ny), bd = sizeof(double) * (size_t(nx) + ny),
                  br = sizeof(int4) * 2 * size_t(ntx);
     char* scratch = nullptr;
     cudaError_t e = xmalloc_async(reinterpret_cast<void**>(&scratch), bd + br + bi, st);
     if (e != cudaSuccess) return cuda_status(e);
-    double* dfx = reinterpret_cast<double*>(scratch);
-    double* dfy = dfx + nx;
-    int4* drx = reinterpret_cast<int4*>(scratch + bd);
+    int4* drx = reinterpret_cast<int4*>(scratch);
     int4* dry = drx + ntx;
+    double* dfx = reinterpret_cast<double*>(scratch + br);
+    double* dfy = dfx + nx;
     int* dl0x = reinterpret_cast<int*>(scratch + bd + br);
     int* dl0y = dl0x + nx;
     auto fail = [&](cudaError_t err) {

@@ -221,3 +221,30 @@ def test_lattice_outside_window_is_rejected(P):
     with pytest.raises(P.NuasmError) as ei:
         P.nuasm_plan_lattice(P.make_params(32, 10e-6, 633e-9, 0.01), 40, 40, 10e-6, -200e-6, -200e-6)
     assert ei.value.code == 2
+
+
+@pytest.mark.parametrize("prec,nx,ny", [("f32", 119, 120), ("f64", 61, 64), ("f32", 1, 2)])
+def test_lattice_with_an_odd_sum_of_sides(P, prec, nx, ny):
+    """nx + ny odd: the plan's scratch arrays (int4 ranges beside nx + ny
+    doubles) stay 16-byte aligned, and the lattice equals its points given one
+    by one."""
+    import torch
+    n, pitch, p2 = 64, 10e-6, 4e-6
+    x0, y0 = -0.5 * nx * p2, -0.5 * ny * p2
+    params = P.make_params(n, pitch, 633e-9, 0.05, prec=prec)
+    yy, xx = np.meshgrid(y0 + np.arange(ny) * p2, x0 + np.arange(nx) * p2, indexing="ij")
+    lat = P.nuasm_plan_lattice(params, nx, ny, p2, x0, y0)
+    pts = P.nuasm_plan(params, _dev(xx.ravel()), _dev(yy.ravel()))
+    try:
+        assert P.nuasm_plan_info(lat)["records"] == P.nuasm_plan_info(pts)["records"]
+        rng = np.random.default_rng(45)
+        u1 = _dev((rng.normal(size=n * n) + 1j * rng.normal(size=n * n)).astype(CDT[prec]))
+        va, vb = (torch.zeros(nx * ny, dtype=torch.complex64 if prec == "f32" else torch.complex128, device="cuda")
+                  for _ in range(2))
+        P.nuasm2_execute(lat, u1, va)
+        P.nuasm2_execute(pts, u1, vb)
+        torch.cuda.synchronize()
+        assert O.rel_l2(va.cpu().numpy(), vb.cpu().numpy()) < (1e-6 if prec == "f32" else 1e-13)
+    finally:
+        lat.destroy()
+        pts.destroy()
