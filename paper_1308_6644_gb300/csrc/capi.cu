@@ -184,10 +184,11 @@ cudaError_t upload_tables(nuasm_plan_s* P, const HostTables& t, cudaStream_t st)
     if (P->f64) {
         const double* tw = reinterpret_cast<const double*>(host.data() + tw_off);
         float* out = reinterpret_cast<float*>(host.data() + bytes);
-        for (size_t i = 0; i < df_bytes / sizeof(double); ++i) {
+        for (size_t i = 0; i < df_bytes / sizeof(double); ++i) {   // a complex entry: both hi parts, then both lo
             const float hi = float(tw[i]);
-            out[2 * i] = hi;
-            out[2 * i + 1] = float(tw[i] - double(hi));
+            float* q = out + 4 * (i / 2) + (i & 1);
+            q[0] = hi;
+            q[2] = float(tw[i] - double(hi));
         }
     }
     e = cudaMemcpyAsync(base, host.data(), bytes + df_bytes, cudaMemcpyHostToDevice, st);

@@ -12,7 +12,8 @@ namespace nuasm {
 // A real hi + lo of two floats (about 47 significant bits) and a complex of
 // two of them, for FFT passes of FP64 plans on the FP32 pipe.  Sums use the
 // two-sum of the high parts with the low parts added to its error term, and
-// products the FMA error of the high parts; both renormalise once.
+// products the FMA errors of the high parts; both renormalise once (a complex
+// product once per component, after the sum of its two real products).
 struct dfr {
     float hi, lo;
     dfr() = default;
@@ -20,43 +21,110 @@ struct dfr {
     __host__ __device__ constexpr explicit dfr(double d) : hi(float(d)), lo(float(d - double(float(d)))) {}
 };
 __host__ __device__ constexpr dfr operator-(dfr a) { return dfr(-a.hi, -a.lo); }
-__device__ __forceinline__ dfr operator+(dfr a, dfr b) {
-    const float s = a.hi + b.hi;
-    const float bb = s - a.hi;
-    const float e = ((a.hi - (s - bb)) + (b.hi - bb)) + (a.lo + b.lo);
-    const float h = s + e;
-    return dfr(h, e - (h - s));
+// ---------------------------------------------------------------- packed FP32 pairs
+// One f32x2 instruction does both halves of a register pair.  Its peak rate is
+// the scalar one (measured: 126 against 121 lane operations per cycle and SM)
+// at half the issue slots and half the code, and the double-float row passes
+// were short of both, not of the FP32 pipe (42% busy; instruction fetch their
+// top stall): N' = 4096 row_t1 1.56 -> 1.17 ms, row_t2 1.49 -> 1.11 ms.
+// The packing stays inside each asm statement: as 64-bit shifts and ors in C++
+// it multiplied the compile time of the passes by ten.
+#define NUASM_F2_OP2(name, op)                                                                       \
+    __device__ __forceinline__ float2 name(float2 a, float2 b) {                                      \
+        float2 r;                                                                                     \
+        asm("{\n.reg .b64 a, b, r;\nmov.b64 a, {%2, %3};\nmov.b64 b, {%4, %5};\n" op                 \
+            " r, a, b;\nmov.b64 {%0, %1}, r;\n}"                                                      \
+            : "=f"(r.x), "=f"(r.y)                                                                    \
+            : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));                                                \
+        return r;                                                                                     \
+    }
+NUASM_F2_OP2(add2, "add.rn.f32x2")
+NUASM_F2_OP2(sub2, "sub.rn.f32x2")
+NUASM_F2_OP2(mul2, "mul.rn.f32x2")
+#undef NUASM_F2_OP2
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    float2 r;
+    asm("{\n.reg .b64 a, b, c, r;\nmov.b64 a, {%2, %3};\nmov.b64 b, {%4, %5};\nmov.b64 c, {%6, %7};\n"
+        "fma.rn.f32x2 r, a, b, c;\nmov.b64 {%0, %1}, r;\n}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return r;
 }
-__device__ __forceinline__ dfr operator-(dfr a, dfr b) { return a + (-b); }
-__device__ __forceinline__ dfr operator*(dfr a, dfr b) {
-    const float p = a.hi * b.hi;
-    const float e = fmaf(a.hi, b.hi, -p) + fmaf(a.hi, b.lo, a.lo * b.hi);
-    const float h = p + e;
-    return dfr(h, e - (h - p));
-}
-// k a for a small integer k (the FFT engine's direction signs)
-__device__ __forceinline__ dfr operator*(int k, dfr a) {
-    return k == 1 ? a : k == -1 ? -a : dfr(float(k), 0.f) * a;
-}
+__device__ __forceinline__ float2 f2_swap(float2 a) { return make_float2(a.y, a.x); }
+__device__ __forceinline__ float2 f2_dup(float a) { return make_float2(a, a); }
+
+// A complex of two double-floats, the high parts (re, im) and the low parts
+// (re, im) each a register pair, so that a complex sum is one packed sequence.
 struct __align__(16) dfc {
-    dfr x, y;
+    float2 h, l;
+    __device__ __forceinline__ dfr x() const { return dfr(h.x, l.x); }
+    __device__ __forceinline__ dfr y() const { return dfr(h.y, l.y); }
 };
-__device__ __forceinline__ dfc cadd(dfc a, dfc b) { return dfc{a.x + b.x, a.y + b.y}; }
-__device__ __forceinline__ dfc csub(dfc a, dfc b) { return dfc{a.x - b.x, a.y - b.y}; }
-__device__ __forceinline__ dfc cmul(dfc a, dfc b) { return dfc{a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x}; }
-__device__ __forceinline__ dfc cconj(dfc a) { return dfc{a.x, -a.y}; }
+// s + e renormalised (|e| small against |s|)
+__device__ __forceinline__ dfc dfc_renorm(float2 s, float2 e) {
+    const float2 h = add2(s, e);
+    return dfc{h, sub2(e, sub2(h, s))};
+}
+__device__ __forceinline__ dfc cadd(dfc a, dfc b) {
+    const float2 s = add2(a.h, b.h), bb = sub2(s, a.h);
+    const float2 e = add2(sub2(a.h, sub2(s, bb)), sub2(b.h, bb));
+    return dfc_renorm(s, add2(e, add2(a.l, b.l)));
+}
+__device__ __forceinline__ dfc csub(dfc a, dfc b) {
+    const float2 s = sub2(a.h, b.h), bb = sub2(s, a.h);
+    const float2 e = sub2(sub2(a.h, sub2(s, bb)), add2(b.h, bb));
+    return dfc_renorm(s, add2(e, sub2(a.l, b.l)));
+}
+// a + DIR i b: the products by +-1 are exact, so the multiplication by i costs
+// only the swap
+template <int DIR> __device__ __forceinline__ dfc cadd_i(dfc a, dfc b) {
+    const float2 sg = DIR > 0 ? make_float2(-1.f, 1.f) : make_float2(1.f, -1.f);
+    const float2 bh = f2_swap(b.h), bl = f2_swap(b.l);
+    const float2 s = fma2(bh, sg, a.h), nb = sub2(a.h, s);
+    const float2 e = add2(sub2(a.h, add2(s, nb)), fma2(bh, sg, nb));
+    return dfc_renorm(s, add2(e, fma2(bl, sg, a.l)));
+}
+// a r for a real constant r (the product and its error in scalar FMAs: the
+// packed fma of a, r and the packed product of a and -r came back as zero)
+__device__ __forceinline__ dfc cscale(dfc a, dfr r) {
+    const float2 p = make_float2(a.h.x * r.hi, a.h.y * r.hi);
+    float2 e = make_float2(fmaf(a.h.x, r.hi, -p.x), fmaf(a.h.y, r.hi, -p.y));
+    e = fma2(a.h, f2_dup(r.lo), e);
+    return dfc_renorm(p, fma2(a.l, f2_dup(r.hi), e));
+}
+// the four products and their errors one by one (a packed form would need
+// every factor in both halves of a pair), their sums packed
+__device__ __forceinline__ dfc cmul(dfc a, dfc b) {
+    const float2 p = make_float2(a.h.x * b.h.x, a.h.x * b.h.y);
+    const float2 q = make_float2(-a.h.y * b.h.y, a.h.y * b.h.x);
+    float2 ep = make_float2(fmaf(a.h.x, b.h.x, -p.x), fmaf(a.h.x, b.h.y, -p.y));
+    float2 eq = make_float2(fmaf(-a.h.y, b.h.y, -q.x), fmaf(a.h.y, b.h.x, -q.y));
+    ep = make_float2(fmaf(a.h.x, b.l.x, ep.x), fmaf(a.h.x, b.l.y, ep.y));
+    eq = make_float2(fmaf(-a.h.y, b.l.y, eq.x), fmaf(a.h.y, b.l.x, eq.y));
+    ep = make_float2(fmaf(a.l.x, b.h.x, ep.x), fmaf(a.l.x, b.h.y, ep.y));
+    eq = make_float2(fmaf(-a.l.y, b.h.y, eq.x), fmaf(a.l.y, b.h.x, eq.y));
+    const float2 s = add2(p, q), bb = sub2(s, p);
+    const float2 e = add2(sub2(p, sub2(s, bb)), sub2(q, bb));
+    return dfc_renorm(s, add2(e, add2(ep, eq)));
+}
+__device__ __forceinline__ dfc cconj(dfc a) {
+    return dfc{make_float2(a.h.x, -a.h.y), make_float2(a.l.x, -a.l.y)};
+}
+__device__ __forceinline__ dfc cneg(dfc a) {
+    return dfc{make_float2(-a.h.x, -a.h.y), make_float2(-a.l.x, -a.l.y)};
+}
 template <> struct CTraits<dfc> {
     using real = dfr;
     static constexpr int pad_shift = 3;   // 16-byte elements, as complex128
-    __device__ static dfc zero() { return dfc{dfr(0.f, 0.f), dfr(0.f, 0.f)}; }
-    __device__ static dfc make(dfr a, dfr b) { return dfc{a, b}; }
+    __device__ static dfc zero() { return dfc{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
+    __device__ static dfc make(dfr a, dfr b) { return dfc{make_float2(a.hi, b.hi), make_float2(a.lo, b.lo)}; }
 };
 
 // read-only cached load of a table entry (complex types of 8 or 16 bytes, reals)
 template <typename T> __device__ __forceinline__ T ldgv(const T* p) { return __ldg(p); }
 template <> __device__ __forceinline__ dfc ldgv<dfc>(const dfc* p) {
     const float4 q = __ldg(reinterpret_cast<const float4*>(p));
-    return dfc{dfr(q.x, q.y), dfr(q.z, q.w)};
+    return dfc{make_float2(q.x, q.y), make_float2(q.z, q.w)};
 }
 
 // 2^k as a double for k in [-1022, 1023]

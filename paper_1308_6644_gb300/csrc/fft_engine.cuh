@@ -119,6 +119,38 @@ template <int DIR, typename V> struct Dft<16, DIR, V> {
     }
 };
 
+// Double-float: the multiplications by +-i go into the sums (cadd_i), which
+// leaves the swaps of their factors as the only cost.
+template <int DIR> struct Dft<4, DIR, dfc> {
+    __device__ __forceinline__ static void run(dfc* v) {
+        const dfc t0 = cadd(v[0], v[2]), t1 = csub(v[0], v[2]);
+        const dfc t2 = cadd(v[1], v[3]), t3 = csub(v[1], v[3]);
+        v[0] = cadd(t0, t2);
+        v[2] = csub(t0, t2);
+        v[1] = cadd_i<DIR>(t1, t3);
+        v[3] = cadd_i<-DIR>(t1, t3);
+    }
+};
+template <int DIR> struct Dft<8, DIR, dfc> {
+    __device__ __forceinline__ static void run(dfc* v) {
+        const dfr r = dfr(0.70710678118654752440);
+        dfc e[4] = {v[0], v[2], v[4], v[6]};
+        dfc o[4] = {v[1], v[3], v[5], v[7]};
+        Dft<4, DIR, dfc>::run(e);
+        Dft<4, DIR, dfc>::run(o);
+        const dfc o1 = cscale(cadd_i<DIR>(o[1], o[1]), r);   // o[1] exp(DIR 2 pi i / 8)
+        const dfc o3 = cscale(cadd_i<DIR>(o[3], o[3]), r);   // o[3] exp(DIR 2 pi i 3 / 8) = DIR i o3
+        v[0] = cadd(e[0], o[0]);
+        v[4] = csub(e[0], o[0]);
+        v[1] = cadd(e[1], o1);
+        v[5] = csub(e[1], o1);
+        v[2] = cadd_i<DIR>(e[2], o[2]);
+        v[6] = cadd_i<-DIR>(e[2], o[2]);
+        v[3] = cadd_i<DIR>(e[3], o3);
+        v[7] = cadd_i<-DIR>(e[3], o3);
+    }
+};
+
 template <int R> struct Log2 { static constexpr int v = R <= 1 ? 0 : 1 + Log2<R / 2>::v; };
 template <> struct Log2<1> { static constexpr int v = 0; };
 

@@ -150,14 +150,14 @@ template <typename V> struct Mem {
 template <> struct Mem<dfc> {
     using type = double2;
     static constexpr bool scaled = true;
-    __device__ static dfc ld(double2 x, int sc) { return dfc{dfr_split(x.x, sc), dfr_split(x.y, sc)}; }
-    __device__ static double2 st(dfc v, int sc) { return make_double2(dfr_to_double(v.x, sc), dfr_to_double(v.y, sc)); }
+    __device__ static dfc ld(double2 x, int sc) { return CTraits<dfc>::make(dfr_split(x.x, sc), dfr_split(x.y, sc)); }
+    __device__ static double2 st(dfc v, int sc) { return make_double2(dfr_to_double(v.x(), sc), dfr_to_double(v.y(), sc)); }
 };
 template <typename V> using MemT = typename Mem<V>::type;
 
 __device__ __forceinline__ bool nonzero(float2 v) { return v.x != 0.f || v.y != 0.f; }
 __device__ __forceinline__ bool nonzero(double2 v) { return v.x != 0.0 || v.y != 0.0; }
-__device__ __forceinline__ bool nonzero(dfc v) { return v.x.hi != 0.f || v.y.hi != 0.f; }
+__device__ __forceinline__ bool nonzero(dfc v) { return v.h.x != 0.f || v.h.y != 0.f; }
 
 // exponent k with 2^k <= |x| < 2^(k+1) (-1023 for zeros and subnormals)
 __device__ __forceinline__ int dexp2(double x) {
@@ -437,7 +437,7 @@ __global__ void __launch_bounds__(RowCfg<V, LOGNP>::P, RowCfg<V, LOGNP>::MINB)
         const V y = NUASM_IN_RANGE(row * NP + q, ROWS * NP, dbg::kRowModes) ? M[row * NP + q] : zero;
         if (sgn == 0) return y;
         const V f = half_bin<V, +1, LOGNP, R0I>(tw, q);
-        return cmul(y, q < HALF ? f : CTraits<V>::make(-f.x, -f.y));
+        return cmul(y, q < HALF ? f : cneg(f));
     };
     auto put = [&](int row, int k, int sgn, V v) {
         const int u = 2 * k + sgn;
@@ -498,7 +498,7 @@ __global__ void __launch_bounds__(RowCfg<V, LOGNP>::P, RowCfg<V, LOGNP>::MINB)
         const V y = NUASM_IN_RANGE(row * NP + q, ROWS * NP, dbg::kRowModes) ? M[row * NP + q] : zero;
         if (sgn == 0) return y;
         const V f = half_bin<V, +1, LOGNP, R0>(tw, q);
-        return cmul(y, q < HALF ? f : CTraits<V>::make(-f.x, -f.y));
+        return cmul(y, q < HALF ? f : cneg(f));
     };
     auto put_row = [&](int row, int k, int sgn, V v) {
         const int u = 2 * k + sgn;
@@ -602,7 +602,7 @@ __global__ void __launch_bounds__(ColCfg<V, LOGNP, MODE>::P, ColCfg<V, LOGNP, MO
                 const V y = ld(q * Wp + col);
                 if (sgn == 0) return y;
                 const V f = half_bin<V, +1, LOGNP, Cf::E>(tw, q);
-                return cmul(y, q < HALF ? f : CTraits<V>::make(-f.x, -f.y));
+                return cmul(y, q < HALF ? f : cneg(f));
             },
             [&](int k, int c, V v) {
                 const int col = col0 + c;
