@@ -389,7 +389,7 @@ nuasm_status nuasm::plan_create(nuasm_plan_s** out, const nuasm_params_t* p, int
     P->poly = ht.poly;
     if (P->f64) {
         fit_kernel_poly64(P->g, &P->poly64);
-        split_kernel_poly64(P->poly64, &P->poly64df);
+        split_kernel_poly64(P->poly64, P->g.w, &P->poly64df);
     }
     P->nonsep_mode = choose_nonsep_mode(rp, ht.rmax);
     cudaError_t e = upload_tables(P, ht, st);

@@ -895,65 +895,126 @@ __device__ __forceinline__ int dexp(double x) {
     return (int(static_cast<unsigned long long>(__double_as_longlong(x)) >> 52) & 0x7ff) - 1023;
 }
 
-// a b + c; the sum is kept as hi + lo without renormalisation (lo collects
-// the rounding errors of the products and of the hi sums exactly or to 2^-24
-// of its own size)
-__device__ __forceinline__ df df_fma(df a, df b, df c) {
-    const float p = a.hi * b.hi;
-    float e = fmaf(a.hi, b.hi, -p);
-    e = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, e));
-    const df t = df_two_sum(p, c.hi);
-    return {t.hi, t.lo + (e + c.lo)};
+// Two double-floats side by side, their high and their low parts each a
+// register pair (f32x2 operands).
+struct dfp { float2 h, l; };
+
+// s + e as a normalised pair of sums
+__device__ __forceinline__ dfp dfp_renorm(float2 s, float2 e) {
+    const float2 h = add2(s, e);
+    return {h, sub2(e, sub2(h, s))};
+}
+// p + c with the rounding errors of p (e) and of the sum kept in the low part,
+// without renormalisation (the low part collects them exactly or to 2^-24 of
+// its own size)
+__device__ __forceinline__ dfp dfp_add(float2 p, float2 e, dfp c) {
+    const float2 s = add2(p, c.h), bb = sub2(s, p);
+    const float2 t = add2(sub2(p, sub2(s, bb)), sub2(c.h, bb));
+    return {s, add2(t, add2(e, c.l))};
+}
+// a b for one double-float b: the high parts' products (returned) and their
+// errors with the cross terms (*e)
+__device__ __forceinline__ float2 dfp_prod(dfp a, float bh, float bl, float2* e) {
+    const float2 p = make_float2(a.h.x * bh, a.h.y * bh);
+    const float2 r = make_float2(fmaf(a.h.x, bh, -p.x), fmaf(a.h.y, bh, -p.y));
+    *e = make_float2(fmaf(a.h.x, bl, fmaf(a.l.x, bh, r.x)), fmaf(a.h.y, bl, fmaf(a.l.y, bh, r.y)));
+    return p;
 }
 
-// Tap weights of one axis in double-float: Horner's rule on the FP64
-// polynomials, the degrees from kDfTail up in FP32 (the coefficients' hi
-// parts; their sum is below 3.1e-7 for the ES kernel at w = 11 and 13 and
-// 1.1e-7 for the Gaussian at w = 15, 21 and 25, so this adds below 2e-14 to
-// a weight) and the rest in double-float.
-constexpr int kDfTail = 9;
-static_assert(kPoly64Deg >= kDfTail, "FP64 tap degree");
-// c: the kPoly64Deg + 1 coefficients of one tap (parameter or shared memory)
-__device__ __forceinline__ df tap_weight_df(const float2* c, df x) {
-    float t = c[kPoly64Deg].x;
-#pragma unroll
-    for (int k = kPoly64Deg - 1; k >= kDfTail; --k) t = fmaf(t, x.hi, c[k].x);
-    df acc = {t, 0.f};
-#pragma unroll
-    for (int k = kDfTail - 1; k >= 0; --k) acc = df_fma(acc, x, df{c[k].x, c[k].y});
-    return df_two_sum(acc.hi, acc.lo);
+// One axis's argument of the tap polynomials: x = 2f - 1 as a double-float, and
+// x^2 in both halves of register pairs.
+struct TapArg {
+    float xh, xl;
+    float2 sh, sl;
+};
+__device__ __forceinline__ TapArg tap_arg(double f) {
+    const df v = df_split(f, 0);
+    const df x = df_two_sum(2.f * v.hi, -1.f);   // 2 v.hi is exact
+    const df n = df_fast_two_sum(x.hi, fmaf(2.f, v.lo, x.lo));
+    const df s = df_mul(n, n);
+    return {n.hi, n.lo, f2_dup(s.hi), f2_dup(s.lo)};
 }
-constexpr int kDfCoef = kPoly64Deg + 1;
 
-// x weights from the parameter copy of the coefficients (unrolled), y
-// weights one row at a time from the CTA's shared copy cs (rolled row loop)
+// The weights of taps i and w - 1 - i (x and y of the pairs) in double-float:
+// E and O of KernelPolyDF by Horner's rule in x^2, both at once in packed
+// arithmetic, then E + x O and E - x O.  Degrees 10 and up are summed in FP32
+// (below 3.1e-7 for the ES kernel at w = 11 and 13 and 1.1e-7 for the Gaussian
+// at w = 15, 21 and 25, so this adds below 2e-14 to a weight), the others in
+// double-float.  c: the tap pair's coefficients (shared memory).  Against one
+// polynomial of degree 13 per tap this is half the steps, two of them to an
+// instruction.
+constexpr int kDfTailStep = 5;   // coefficients 10 .. kPoly64Deg
+static_assert(KernelPolyDF::kSteps > kDfTailStep, "FP64 tap degree");
+__device__ __forceinline__ dfp tap_pair_df(const float4* c, const TapArg& a) {
+    constexpr int K = KernelPolyDF::kSteps;
+    float2 t = make_float2(c[K - 1].x, c[K - 1].y);
+#pragma unroll
+    for (int k = K - 2; k >= kDfTailStep; --k) t = fma2(t, a.sh, make_float2(c[k].x, c[k].y));
+    dfp acc = {t, make_float2(0.f, 0.f)};
+#pragma unroll
+    for (int k = kDfTailStep - 1; k >= 0; --k) {
+        const float4 q = c[k];
+        const float2 p = mul2(acc.h, a.sh);
+        float2 e = make_float2(fmaf(acc.h.x, a.sh.x, -p.x), fmaf(acc.h.y, a.sh.y, -p.y));
+        e = fma2(acc.h, a.sl, fma2(acc.l, a.sh, e));
+        acc = dfp_add(p, e, dfp{make_float2(q.x, q.y), make_float2(q.z, q.w)});
+    }
+    const float p = acc.h.y * a.xh;
+    const float e = fmaf(acc.h.y, a.xl, fmaf(acc.l.y, a.xh, fmaf(acc.h.y, a.xh, -p)));
+    const dfp r = dfp_add(make_float2(p, -p), make_float2(e, -e), dfp{f2_dup(acc.h.x), f2_dup(acc.l.x)});
+    return dfp_renorm(r.h, r.l);
+}
+constexpr int kDfSteps = KernelPolyDF::kSteps;
+// the coefficients of the kernel's tap pairs to shared memory
+template <int WMAX> __device__ __forceinline__ void load_tap_coefs(const KernelPolyDF& kp, float4* cs) {
+    for (int i = threadIdx.x; i < (WMAX + 1) / 2 * kDfSteps; i += blockDim.x) cs[i] = kp.c[i / kDfSteps][i % kDfSteps];
+}
+template <int WMAX> __device__ __forceinline__ void tap_weights_df(const float4* cs, const TapArg& a, df* w) {
+#pragma unroll
+    for (int i = 0; i <= (WMAX - 1) / 2; ++i) {
+        const dfp q = tap_pair_df(cs + i * kDfSteps, a);
+        w[i] = df{q.h.x, q.l.x};
+        w[WMAX - 1 - i] = df{q.h.y, q.l.y};   // an odd WMAX's middle tap: O = 0, both are E
+    }
+}
+
+// x weights in registers, y weights a mirrored pair of rows at a time (rolled loop)
 template <int WMAX>
 __device__ __forceinline__ void interp_point_df(const RecD& r, const float4* __restrict__ tl, int THP, int x0, int y0,
-                                                const KernelPolyDF& kp, const float2* cs, double scale,
-                                                double2* __restrict__ v, [[maybe_unused]] int tl_n,
-                                                [[maybe_unused]] long long m) {
+                                                const float4* cs, double scale, double2* __restrict__ v,
+                                                [[maybe_unused]] int tl_n, [[maybe_unused]] long long m) {
     const int lx = int(r.cell & 0xffffu) - x0, ly = int(r.cell >> 16) - y0;
     df wx[WMAX];
-    const df xv = df_split(fma(2.0, r.fx, -1.0), 0), yv = df_split(fma(2.0, r.fy, -1.0), 0);
-#pragma unroll
-    for (int q = 0; q < WMAX; ++q) wx[q] = tap_weight_df(kp.c[q], xv);
-    df ar = {0.f, 0.f}, ai = {0.f, 0.f};
+    tap_weights_df<WMAX>(cs, tap_arg(r.fx), wx);
+    const TapArg ya = tap_arg(r.fy);
+    const float2 zero = make_float2(0.f, 0.f);
+    dfp acc = {zero, zero};
 #pragma unroll 1
-    for (int qy = 0; qy < WMAX; ++qy) {
-        const df wyq = tap_weight_df(cs + qy * kDfCoef, yv);
-        const float4* row = tl + (ly + qy) * THP + lx;
-        df rr = {0.f, 0.f}, ri = {0.f, 0.f};
+    for (int iy = 0; iy <= (WMAX - 1) / 2; ++iy) {
+        dfp wy = tap_pair_df(cs + iy * kDfSteps, ya);
+        int qy = iy;
+#pragma unroll 1
+        for (int k = iy == WMAX - 1 - iy ? 1 : 0; k < 2; ++k) {
+            const float4* row = tl + (ly + qy) * THP + lx;
+            dfp s = {zero, zero};
 #pragma unroll
-        for (int qx = 0; qx < WMAX; ++qx) {
-            if (!NUASM_IN_RANGE((ly + qy) * THP + lx + qx, tl_n, dbg::kInterpTile)) continue;
-            const float4 g = row[qx];
-            rr = df_fma(df{g.x, g.y}, wx[qx], rr);
-            ri = df_fma(df{g.z, g.w}, wx[qx], ri);
+            for (int qx = 0; qx < WMAX; ++qx) {
+                if (!NUASM_IN_RANGE((ly + qy) * THP + lx + qx, tl_n, dbg::kInterpTile)) continue;
+                const float4 g = row[qx];
+                float2 e;
+                const float2 p = dfp_prod(dfp{make_float2(g.x, g.y), make_float2(g.z, g.w)}, wx[qx].hi, wx[qx].lo, &e);
+                s = dfp_add(p, e, s);
+            }
+            s = dfp_renorm(s.h, s.l);
+            float2 e;
+            const float2 p = dfp_prod(s, wy.h.x, wy.l.x, &e);
+            acc = dfp_add(p, e, acc);
+            wy = {f2_swap(wy.h), f2_swap(wy.l)};   // then the mirrored row
+            qy = WMAX - 1 - iy;
         }
-        ar = df_fma(df_two_sum(rr.hi, rr.lo), wyq, ar);
-        ai = df_fma(df_two_sum(ri.hi, ri.lo), wyq, ai);
     }
-    const double2 out = make_double2((double(ar.hi) + double(ar.lo)) * scale, (double(ai.hi) + double(ai.lo)) * scale);
+    const double2 out = make_double2((double(acc.h.x) + double(acc.l.x)) * scale,
+                                     (double(acc.h.y) + double(acc.l.y)) * scale);
     if (NUASM_IN_RANGE(r.j, m, dbg::kInterpOut)) v[r.j] = out;
 }
 
@@ -982,42 +1043,47 @@ constexpr int kDfBatch = 512;
 // clustered FP64 points: 3.04 ms at 2, 2.85 ms at 3)
 #define NUASM_DF_SPREAD_MINB 3
 #endif
-// a b without renormalisation (the low part is the product's exact error
-// plus the cross terms)
-__device__ __forceinline__ df df_prod(df a, df b) {
-    const float p = a.hi * b.hi;
-    float e = fmaf(a.hi, b.hi, -p);
-    e = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, e));
-    return {p, e};
-}
-// n_h, n_l of p (|p| < 1) by round-to-nearest additions of "magic" constants
-// on the FP32 pipe instead of conversion instructions (whose pipe runs at a
-// quarter of the FP32 rate): t = p.hi 2^30 is rounded to a multiple of 256 by
-// adding 3 2^30 (the sum lies in [2^31, 2^32), whose float spacing is 256),
-// the exact remainder plus p.lo 2^30 (|.| <= 192) to an integer by adding
-// 1.5 2^23 (spacing 1), and what is left (|.| <= 1/2 + 2^-17), times 2^22,
-// likewise; a sum's bits minus the constant's bits are the rounded value in
-// units of the spacing.
-__device__ __forceinline__ void df_quant_add(df p, int cell, int* ph, int* pl) {
+// n_h, n_l of both components of p + e (in units of 2^-30, |p| < 2^30, |e| <
+// 2^6) by round-to-nearest additions of "magic" constants on the FP32 pipe
+// instead of conversion instructions (whose pipe runs at an eighth of the FP32
+// rate): p is rounded to a multiple of 256 by adding 3 2^30 (the sum lies in
+// [2^31, 2^32), whose float spacing is 256), the exact remainder plus e (|.| <=
+// 192) to an integer by adding 1.5 2^23 (spacing 1), and what is left (|.| <=
+// 1/2 + 2^-17), times 2^22, likewise; a sum's bits minus the constant's bits
+// are the rounded value in units of the spacing.
+__device__ __forceinline__ void df_quant_add(float2 p, float2 e, int cell, int* rh, int* rl, int* ih, int* il) {
     constexpr float M1 = 3221225472.f, M2 = 12582912.f;   // 3 2^30, 1.5 2^23
-    const float t = p.hi * 1073741824.f;                    // 2^30: exact; |t| < 2^30
-    const float tl = p.lo * 1073741824.f;                   // |tl| < 2^6
-    const float s1 = t + M1;
-    const float r1 = t - (s1 - M1);                         // exact, |r1| <= 128
-    const float s2 = (r1 + tl) + M2;
-    const float d = (r1 - (s2 - M2)) + tl;                  // r1 - (s2 - M2) exact; |d| <= 1/2 + 2^-17
-    const float s3 = fmaf(d, 4194304.f, M2);                // d 2^22 rounded (|d 2^22| <= 2^21 + 32)
-    const int nh = ((__float_as_int(s1) - __float_as_int(M1)) << 8) + (__float_as_int(s2) - __float_as_int(M2));
-    const int nl = __float_as_int(s3) - __float_as_int(M2);
-    atomicAdd(&ph[cell], nh);
-    atomicAdd(&pl[cell], nl);
+    constexpr int B1 = 0x4f400000, B2 = 0x4b400000;        // their bits
+    const float2 m1 = f2_dup(M1), m2 = f2_dup(M2);
+    const float2 s1 = add2(p, m1);
+    const float2 r1 = sub2(p, sub2(s1, m1));                // exact, |r1| <= 128
+    const float2 s2 = add2(add2(r1, e), m2);
+    const float2 d = add2(sub2(r1, sub2(s2, m2)), e);       // r1 - (s2 - M2) exact; |d| <= 1/2 + 2^-17
+    const float2 s3 = fma2(d, f2_dup(4194304.f), m2);       // d 2^22 rounded (|d 2^22| <= 2^21 + 32)
+    atomicAdd(&rh[cell], ((__float_as_int(s1.x) - B1) << 8) + (__float_as_int(s2.x) - B2));
+    atomicAdd(&rl[cell], __float_as_int(s3.x) - B2);
+    atomicAdd(&ih[cell], ((__float_as_int(s1.y) - B1) << 8) + (__float_as_int(s2.y) - B2));
+    atomicAdd(&il[cell], __float_as_int(s3.y) - B2);
 }
 // 2^k as a double for k in [-1022, 1023]
 __device__ __forceinline__ double pow2d(int k) { return __longlong_as_double(static_cast<long long>(k + 1023) << 52); }
-// V 2^k for an integer |V| < 2^62 (two exact power-of-two factors when k is below the normal range)
+// V 2^k for an integer |V| < 2^62: rounded to 53 bits and assembled by integer
+// operations (an FP64 conversion and product hold the FP64 pipe for 128 cycles
+// a warp); results below the normal range go through two exact power-of-two
+// factors.
 __device__ __forceinline__ double scaled_int(long long V, int k) {
-    const double v = double(V);
-    return k >= -1022 ? v * pow2d(k) : (v * pow2d(k + 512)) * pow2d(-512);
+    if (V == 0) return 0.0;
+    unsigned long long m = V < 0 ? 0ull - static_cast<unsigned long long>(V) : static_cast<unsigned long long>(V);
+    const int lz = __clzll(m);
+    const int E = 63 - lz + k;   // exponent of the leading bit
+    if (E < -1022 || E > 1022) {
+        const double v = double(V);
+        return k >= -1022 ? v * pow2d(k) : (v * pow2d(k + 512)) * pow2d(-512);
+    }
+    m <<= lz;
+    m = (m >> 11) + ((m >> 10) & 1);   // at most 2^53: a carry moves into the exponent
+    const unsigned long long bits = (static_cast<unsigned long long>(E + 1022) << 52) + m;
+    return __longlong_as_double(static_cast<long long>(bits | (V < 0 ? 1ull << 63 : 0ull)));
 }
 
 template <int WMAX>
@@ -1029,7 +1095,7 @@ __global__ void __launch_bounds__(256, WMAX <= 13 ? NUASM_DF_SPREAD_MINB : 2) sp
                                                           const int4* __restrict__ items) {
     constexpr int NT = 256, RPB = kDfBatch / NT;
     extern __shared__ unsigned char smem_raw[];
-    __shared__ float2 cs[WMAX * kDfCoef];
+    __shared__ float4 cs[(WMAX + 1) / 2 * kDfSteps];
     __shared__ double red[NT / 32];
     __shared__ double bsum;
     int tile, b, e;
@@ -1051,7 +1117,7 @@ __global__ void __launch_bounds__(256, WMAX <= 13 ? NUASM_DF_SPREAD_MINB : 2) sp
     int* ih = rl + TT;
     int* il = ih + TT;
     pdl_allow_next();
-    for (int i = threadIdx.x; i < WMAX * kDfCoef; i += NT) cs[i] = kp.c[i / kDfCoef][i % kDfCoef];
+    load_tap_coefs<WMAX>(kp, cs);
     for (int i = threadIdx.x; i < TT; i += NT) {
         rh[i] = 0;
         rl[i] = 0;
@@ -1129,25 +1195,37 @@ __global__ void __launch_bounds__(256, WMAX <= 13 ? NUASM_DF_SPREAD_MINB : 2) sp
             const int i = i0 + threadIdx.x + k * NT;
             if (i >= e) continue;
             const int lx = int(r[k].cell & 0xffffu) - x0, ly = int(r[k].cell >> 16) - y0;
-            const df vr = df_split(val[k].x, Eb), vi = df_split(val[k].y, Eb);
-            const df xv = df_split(fma(2.0, r[k].fx, -1.0), 0), yv = df_split(fma(2.0, r[k].fy, -1.0), 0);
+            // the value in units of 2^(Eb - 30)
+            const df vr = df_split(val[k].x, Eb - 30), vi = df_split(val[k].y, Eb - 30);
+            const dfp vv = {make_float2(vr.hi, vi.hi), make_float2(vr.lo, vi.lo)};
             df wx[WMAX];
-#pragma unroll
-            for (int q = 0; q < WMAX; ++q) wx[q] = tap_weight_df(kp.c[q], xv);
+            tap_weights_df<WMAX>(cs, tap_arg(r[k].fx), wx);
+            const TapArg yt = tap_arg(r[k].fy);
             const int ya = max(0, -ly), yb = min(WMAX, T - ly);
             const int xa = max(0, -lx), xb = min(WMAX, T - lx);
 #pragma unroll 1
-            for (int qy = ya; qy < yb; ++qy) {
-                const df wyq = tap_weight_df(cs + qy * kDfCoef, yv);
-                const df pr = df_mul(vr, wyq), pi = df_mul(vi, wyq);
-                const int rowi = (ly + qy) * TS + lx;
+            for (int iy = 0; iy <= (WMAX - 1) / 2; ++iy) {
+                dfp wy = tap_pair_df(cs + iy * kDfSteps, yt);
+                int qy = iy;
+#pragma unroll 1
+                for (int h = iy == WMAX - 1 - iy ? 1 : 0; h < 2; ++h) {
+                    if (qy >= ya && qy < yb) {
+                        float2 e;
+                        const float2 p = dfp_prod(vv, wy.h.x, wy.l.x, &e);
+                        const dfp pw = dfp_renorm(p, e);
+                        const int rowi = (ly + qy) * TS + lx;
 #pragma unroll
-                for (int qx = 0; qx < WMAX; ++qx) {
-                    if (qx < xa || qx >= xb) continue;
-                    const int cell = rowi + qx;
-                    if (!NUASM_IN_RANGE(cell, TT, dbg::kSpreadPlane)) continue;
-                    df_quant_add(df_prod(pr, wx[qx]), cell, rh, rl);
-                    df_quant_add(df_prod(pi, wx[qx]), cell, ih, il);
+                        for (int qx = 0; qx < WMAX; ++qx) {
+                            if (qx < xa || qx >= xb) continue;
+                            const int cell = rowi + qx;
+                            if (!NUASM_IN_RANGE(cell, TT, dbg::kSpreadPlane)) continue;
+                            float2 te;
+                            const float2 tp = dfp_prod(pw, wx[qx].hi, wx[qx].lo, &te);
+                            df_quant_add(tp, te, cell, rh, rl, ih, il);
+                        }
+                    }
+                    wy = {f2_swap(wy.h), f2_swap(wy.l)};   // then the mirrored row
+                    qy = WMAX - 1 - iy;
                 }
             }
         }
@@ -1217,7 +1295,7 @@ __global__ void __launch_bounds__(256, WMAX <= 13 ? NUASM_DF_SPREAD_MINB : 2) sp
 // schedule (one CTA per tile or chunk, a ring of prefetched records); the
 // tile is staged in FP64, scaled by 2^-s, s the largest exponent among its
 // values (so no value leaves the float range), and split in place into
-// (re.hi, re.lo, im.hi, im.lo) cells of the same 16 bytes.
+// (re.hi, im.hi, re.lo, im.lo) cells of the same 16 bytes.
 template <int WMAX>
 __global__ void __launch_bounds__(kInterpThreads, 2) interp_df_kernel(const RecD* __restrict__ rec,
                                                                       const int* __restrict__ off,
@@ -1231,8 +1309,8 @@ __global__ void __launch_bounds__(kInterpThreads, 2) interp_df_kernel(const RecD
     double2* tld = reinterpret_cast<double2*>(smem_raw);
     float4* tl = reinterpret_cast<float4*>(smem_raw);
     __shared__ int emax;
-    __shared__ float2 cs[WMAX * kDfCoef];
-    for (int i = threadIdx.x; i < WMAX * kDfCoef; i += kInterpThreads) cs[i] = kp.c[i / kDfCoef][i % kDfCoef];
+    __shared__ float4 cs[(WMAX + 1) / 2 * kDfSteps];
+    load_tap_coefs<WMAX>(kp, cs);
     const int T = a.T, TH = T + WMAX - 1;
     int tile, b, e;
     if (items) {
@@ -1274,7 +1352,7 @@ __global__ void __launch_bounds__(kInterpThreads, 2) interp_df_kernel(const RecD
     for (int i = threadIdx.x; i < TH * THP; i += kInterpThreads) {   // each thread splits the cells it staged
         const double2 val = tld[i];
         const df re = df_split(val.x, sc), im = df_split(val.y, sc);
-        tl[i] = make_float4(re.hi, re.lo, im.hi, im.lo);
+        tl[i] = make_float4(re.hi, im.hi, re.lo, im.lo);
     }
     __syncthreads();
     const double scale = __longlong_as_double(static_cast<long long>(sc + 1023) << 52);   // 2^sc
@@ -1286,7 +1364,7 @@ __global__ void __launch_bounds__(kInterpThreads, 2) interp_df_kernel(const RecD
             if (i < e) {
                 const RecD r = pre[k];
                 if (i + AHEAD < e && NUASM_IN_RANGE(i + AHEAD, a.nrec, dbg::kInterpRec)) pre[k] = rec[i + AHEAD];
-                interp_point_df<WMAX>(r, tl, THP, x0, y0, kp, cs, scale, v, TH * THP, a.m);
+                interp_point_df<WMAX>(r, tl, THP, x0, y0, cs, scale, v, TH * THP, a.m);
             }
         }
     }

@@ -533,11 +533,16 @@ void fit_poly(const Geometry& g, int d, Poly* kp) {
 void fit_kernel_poly(const Geometry& g, KernelPoly* kp) { fit_poly<KernelPoly, float>(g, g.w + 1, kp); }
 void fit_kernel_poly64(const Geometry& g, KernelPoly64* kp) { fit_poly<KernelPoly64, double>(g, kPoly64Deg, kp); }
 
-void split_kernel_poly64(const KernelPoly64& kp, KernelPolyDF* out) {
-    for (int i = 0; i < kPolyMaxW; ++i)
-        for (int k = 0; k < kPolyMaxD; ++k) {
-            const float hi = float(kp.c[i][k]);
-            out->c[i][k] = float2{hi, float(kp.c[i][k] - double(hi))};
+void split_kernel_poly64(const KernelPoly64& kp, int w, KernelPolyDF* out) {
+    std::memset(out, 0, sizeof(*out));
+    for (int i = 0; i <= (w - 1) / 2; ++i)
+        for (int k = 0; k < KernelPolyDF::kSteps; ++k) {
+            // the two fits of a mirrored pair differ by rounding: their mean serves both
+            const double* a = kp.c[i];
+            const double* b = kp.c[w - 1 - i];
+            const double e = 0.5 * (a[2 * k] + b[2 * k]), o = 0.5 * (a[2 * k + 1] - b[2 * k + 1]);
+            const float eh = float(e), oh = float(o);
+            out->c[i][k] = float4{eh, oh, float(e - double(eh)), float(o - double(oh))};
         }
 }
 

@@ -41,12 +41,17 @@ struct KernelPoly64 {
     double c[kPolyMaxW][kPolyMaxD];
     int deg;
 };
-// The FP64 coefficients as pairs of floats (x: the coefficient rounded to
-// float, y: the rounded remainder), for FP64-mode gridding in double-float
-// arithmetic.
+// The FP64 coefficients for FP64-mode gridding in double-float arithmetic.
+// The kernel is even, so taps i and w - 1 - i have mirrored polynomials: with
+// tap i split as E(x^2) + x O(x^2), the mirrored one is E - x O.  c[i][k] holds
+// the coefficients 2k of tap i (for E) and 2k + 1 (for O), i <= (w - 1)/2, as
+// pairs of floats: x = E's value rounded to float, y = O's, z = E's remainder,
+// w = O's.
 struct KernelPolyDF {
-    float2 c[kPolyMaxW][kPolyMaxD];
+    static constexpr int kPairs = (kPolyMaxW + 1) / 2, kSteps = (kPoly64Deg + 1) / 2;
+    float4 c[kPairs][kSteps];
 };
+static_assert(kPoly64Deg % 2 == 1, "even and odd coefficients pair up");
 
 // Host tables in FP64 (complex as re/im pairs), natural N'-bin order.
 struct HostTables {
@@ -152,7 +157,7 @@ void twiddle(int i, int G, double* re, double* im);
 double nonsep_rmax(const nuasm_params_t& p, const Geometry& g);
 void fit_kernel_poly(const Geometry& g, KernelPoly* kp);
 void fit_kernel_poly64(const Geometry& g, KernelPoly64* kp);
-void split_kernel_poly64(const KernelPoly64& kp, KernelPolyDF* out);
+void split_kernel_poly64(const KernelPoly64& kp, int w, KernelPolyDF* out);
 nuasm_status validate(const nuasm_params_t& p, int64_t m, nuasm_params_t* resolved);
 bool kernel_shape(double tol, int prec, int kernel, int* w, double* beta);
 double kernel_value(const Geometry& g, double t);
