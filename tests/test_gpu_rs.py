@@ -152,3 +152,41 @@ def test_paper_nuasm2_against_rs_on_quadrant_pitch_destination(P):
     assert res[8e-3]["asm"] > 30                      # the paper's ~32 dB class
     assert res[8e-3]["asm"] > res[32e-3]["asm"] > res[128e-3]["asm"]
     assert res[8e-3]["fresnel"] < res[32e-3]["fresnel"] < res[128e-3]["fresnel"]
+
+
+@pytest.mark.parametrize("prec,tol", [("f32", 1e-5), ("f64", 1e-11)])
+@pytest.mark.parametrize("m1,m2", [(1, 1), (31, 65), (256, 32), (257, 33), (513, 64), (1025, 7), (2500, 130)])
+def test_rs_split_edges(P, prec, tol, m1, m2):
+    """Ragged source tiles and point sets, with one and with several CTAs a
+    set (the split starts above 512 sources)."""
+    rng = np.random.default_rng(61)
+    h = 120e-6
+    x1, y1 = rng.uniform(-h, h, m1), rng.uniform(-h, h, m1)
+    x2, y2 = rng.uniform(-h, h, m2), rng.uniform(-h, h, m2)
+    c = rng.normal(size=m1) + 1j * rng.normal(size=m1)
+    area = rng.uniform(0.5, 1.5, m1) * 1e-11
+    got = rs_gpu(P, prec, x1, y1, c, area, x2, y2, 500e-9, 8e-3, 20e-6, -10e-6)
+    cc = c.astype(np.complex64 if prec == "f32" else np.complex128)
+    assert O.rel_l2(got, O.rs_direct(x1, y1, cc, area, x2, y2, 500e-9, 8e-3, 20e-6, -10e-6)) < tol
+
+
+@pytest.mark.parametrize("prec,tol", [("f32", 1e-5), ("f64", 1e-11)])
+@pytest.mark.parametrize("unit", [2.0 ** -60, 2.0 ** 60])
+def test_rs_does_not_depend_on_the_unit_of_length(P, prec, tol, unit):
+    rng = np.random.default_rng(62)
+    m, h = 300, 100e-6
+    x1, y1, x2, y2 = (rng.uniform(-h, h, m) for _ in range(4))
+    c = rng.normal(size=m) + 1j * rng.normal(size=m)
+    area = rng.uniform(0.5, 1.5, m) * 1e-11
+    a = rs_gpu(P, prec, x1, y1, c, area, x2, y2, 500e-9, 8e-3)
+    b = rs_gpu(P, prec, x1 * unit, y1 * unit, c, area * unit ** 2, x2 * unit, y2 * unit, 500e-9 * unit, 8e-3 * unit)
+    assert O.rel_l2(b, a) < tol
+
+
+def test_rs_points_far_beyond_the_distance(P):
+    """rho / z = 1e16: the FP64 kernel's direct formulas."""
+    rng = np.random.default_rng(63)
+    x1, y1, x2, y2 = (rng.uniform(-1e7, 1e7, 70) for _ in range(4))
+    c, area = rng.normal(size=70) + 1j * rng.normal(size=70), rng.uniform(0.5, 1.5, 70)
+    got = rs_gpu(P, "f64", x1, y1, c, area, x2, y2, 1e9, 1e-9)
+    assert O.rel_l2(got, O.rs_direct(x1, y1, c, area, x2, y2, 1e9, 1e-9)) < 1e-11
