@@ -21,40 +21,11 @@ struct dfr {
     __host__ __device__ constexpr explicit dfr(double d) : hi(float(d)), lo(float(d - double(float(d)))) {}
 };
 __host__ __device__ constexpr dfr operator-(dfr a) { return dfr(-a.hi, -a.lo); }
-// ---------------------------------------------------------------- packed FP32 pairs
-// One f32x2 instruction does both halves of a register pair.  Its peak rate is
-// the scalar one (measured: 126 against 121 lane operations per cycle and SM)
-// at half the issue slots and half the code, and the double-float row passes
-// were short of both, not of the FP32 pipe (42% busy; instruction fetch their
-// top stall): N' = 4096 row_t1 1.56 -> 1.17 ms, row_t2 1.49 -> 1.11 ms.
-// The packing stays inside each asm statement: as 64-bit shifts and ors in C++
-// it multiplied the compile time of the passes by ten.
-#define NUASM_F2_OP2(name, op)                                                                       \
-    __device__ __forceinline__ float2 name(float2 a, float2 b) {                                      \
-        float2 r;                                                                                     \
-        asm("{\n.reg .b64 a, b, r;\nmov.b64 a, {%2, %3};\nmov.b64 b, {%4, %5};\n" op                 \
-            " r, a, b;\nmov.b64 {%0, %1}, r;\n}"                                                      \
-            : "=f"(r.x), "=f"(r.y)                                                                    \
-            : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));                                                \
-        return r;                                                                                     \
-    }
-NUASM_F2_OP2(add2, "add.rn.f32x2")
-NUASM_F2_OP2(sub2, "sub.rn.f32x2")
-NUASM_F2_OP2(mul2, "mul.rn.f32x2")
-#undef NUASM_F2_OP2
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
-    float2 r;
-    asm("{\n.reg .b64 a, b, c, r;\nmov.b64 a, {%2, %3};\nmov.b64 b, {%4, %5};\nmov.b64 c, {%6, %7};\n"
-        "fma.rn.f32x2 r, a, b, c;\nmov.b64 {%0, %1}, r;\n}"
-        : "=f"(r.x), "=f"(r.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
-    return r;
-}
-__device__ __forceinline__ float2 f2_swap(float2 a) { return make_float2(a.y, a.x); }
-__device__ __forceinline__ float2 f2_dup(float a) { return make_float2(a, a); }
-
 // A complex of two double-floats, the high parts (re, im) and the low parts
 // (re, im) each a register pair, so that a complex sum is one packed sequence.
+// The double-float row passes were short of issue slots and instruction fetch,
+// not of the FP32 pipe (42% busy): N' = 4096 row_t1 1.56 -> 1.17 ms, row_t2
+// 1.49 -> 1.11 ms against scalar operations.
 struct __align__(16) dfc {
     float2 h, l;
     __device__ __forceinline__ dfr x() const { return dfr(h.x, l.x); }
@@ -115,6 +86,7 @@ __device__ __forceinline__ dfc cneg(dfc a) {
 }
 template <> struct CTraits<dfc> {
     using real = dfr;
+    using tw = dfc;
     static constexpr int pad_shift = 3;   // 16-byte elements, as complex128
     __device__ static dfc zero() { return dfc{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
     __device__ static dfc make(dfr a, dfr b) { return dfc{make_float2(a.hi, b.hi), make_float2(a.lo, b.lo)}; }

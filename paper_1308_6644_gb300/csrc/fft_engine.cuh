@@ -22,6 +22,8 @@
 // makes C adjacent columns of a row-major array coalesced.
 #pragma once
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "dfloat.cuh"
 #include "nuasm_internal.h"
@@ -43,23 +45,22 @@ template <int DIR, typename V> struct Dft<2, DIR, V> {
     }
 };
 
+// (the multiplications by +-i go into the sums)
 template <int DIR, typename V> struct Dft<4, DIR, V> {
     __device__ __forceinline__ static void run(V* v) {
-        V t0 = cadd(v[0], v[2]), t1 = csub(v[0], v[2]);
-        V t2 = cadd(v[1], v[3]), t3 = mul_i<DIR>(csub(v[1], v[3]));
+        const V t0 = cadd(v[0], v[2]), t1 = csub(v[0], v[2]);
+        const V t2 = cadd(v[1], v[3]), t3 = csub(v[1], v[3]);
         v[0] = cadd(t0, t2);
         v[2] = csub(t0, t2);
-        v[1] = cadd(t1, t3);
-        v[3] = csub(t1, t3);
+        v[1] = cadd_i<DIR>(t1, t3);
+        v[3] = cadd_i<-DIR>(t1, t3);
     }
 };
 
 // multiply by exp(DIR 2 pi i e / 8) for e = 1 and e = 3
 template <int DIR, typename V> __device__ __forceinline__ V w8_1(V a) {
     using S = typename CTraits<V>::real;
-    const S r = S(0.70710678118654752440);
-    return DIR < 0 ? CTraits<V>::make((a.x + a.y) * r, (a.y - a.x) * r)
-                   : CTraits<V>::make((a.x - a.y) * r, (a.x + a.y) * r);
+    return cscale(cadd_i<DIR>(a, a), S(0.70710678118654752440));
 }
 template <int DIR, typename V> __device__ __forceinline__ V w8_3(V a) { return mul_i<DIR>(w8_1<DIR>(a)); }
 
@@ -69,14 +70,15 @@ template <int DIR, typename V> struct Dft<8, DIR, V> {
         V o[4] = {v[1], v[3], v[5], v[7]};
         Dft<4, DIR, V>::run(e);
         Dft<4, DIR, V>::run(o);
-        o[1] = w8_1<DIR>(o[1]);
-        o[2] = mul_i<DIR>(o[2]);
-        o[3] = w8_3<DIR>(o[3]);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            v[k] = cadd(e[k], o[k]);
-            v[k + 4] = csub(e[k], o[k]);
-        }
+        const V o1 = w8_1<DIR>(o[1]), o3 = w8_1<DIR>(o[3]);   // o[3]'s factor is DIR i exp(DIR 2 pi i / 8)
+        v[0] = cadd(e[0], o[0]);
+        v[4] = csub(e[0], o[0]);
+        v[1] = cadd(e[1], o1);
+        v[5] = csub(e[1], o1);
+        v[2] = cadd_i<DIR>(e[2], o[2]);
+        v[6] = cadd_i<-DIR>(e[2], o[2]);
+        v[3] = cadd_i<DIR>(e[3], o3);
+        v[7] = cadd_i<-DIR>(e[3], o3);
     }
 };
 
@@ -116,38 +118,6 @@ template <int DIR, typename V> struct Dft<16, DIR, V> {
 #pragma unroll
             for (int k1 = 0; k1 < 4; ++k1) v[k2 + 4 * k1] = t[k1];
         }
-    }
-};
-
-// Double-float: the multiplications by +-i go into the sums (cadd_i), which
-// leaves the swaps of their factors as the only cost.
-template <int DIR> struct Dft<4, DIR, dfc> {
-    __device__ __forceinline__ static void run(dfc* v) {
-        const dfc t0 = cadd(v[0], v[2]), t1 = csub(v[0], v[2]);
-        const dfc t2 = cadd(v[1], v[3]), t3 = csub(v[1], v[3]);
-        v[0] = cadd(t0, t2);
-        v[2] = csub(t0, t2);
-        v[1] = cadd_i<DIR>(t1, t3);
-        v[3] = cadd_i<-DIR>(t1, t3);
-    }
-};
-template <int DIR> struct Dft<8, DIR, dfc> {
-    __device__ __forceinline__ static void run(dfc* v) {
-        const dfr r = dfr(0.70710678118654752440);
-        dfc e[4] = {v[0], v[2], v[4], v[6]};
-        dfc o[4] = {v[1], v[3], v[5], v[7]};
-        Dft<4, DIR, dfc>::run(e);
-        Dft<4, DIR, dfc>::run(o);
-        const dfc o1 = cscale(cadd_i<DIR>(o[1], o[1]), r);   // o[1] exp(DIR 2 pi i / 8)
-        const dfc o3 = cscale(cadd_i<DIR>(o[3], o[3]), r);   // o[3] exp(DIR 2 pi i 3 / 8) = DIR i o3
-        v[0] = cadd(e[0], o[0]);
-        v[4] = csub(e[0], o[0]);
-        v[1] = cadd(e[1], o1);
-        v[5] = csub(e[1], o1);
-        v[2] = cadd_i<DIR>(e[2], o[2]);
-        v[6] = cadd_i<-DIR>(e[2], o[2]);
-        v[3] = cadd_i<DIR>(e[3], o3);
-        v[7] = cadd_i<-DIR>(e[3], o3);
     }
 };
 
@@ -207,41 +177,50 @@ __device__ __forceinline__ V half_bin(const V* __restrict__ tw, int q) {
 // few KB of L1.  The table reads are split from the products (twiddle_base /
 // twiddle_powers) so a pass can issue them before its barrier.
 template <typename V, int R> struct TwBase {
-    static constexpr int N = (sizeof(V) == 16 || R == 2) ? R - 1 : 2;
-    V t[N > 0 ? N : 1];
+    using T = typename CTraits<V>::tw;
+    static constexpr int N = (sizeof(T) == 16 || R == 2) ? R - 1 : 2;
+    T t[N > 0 ? N : 1];
 };
 
 // offset of a pass's table from the start of the full table
-template <typename V, int LE, int LOGL, int PASS> struct TwpOffset {
+template <typename T, int LE, int LOGL, int PASS> struct TwpOffset {
     static_assert(LE == 3 || LE == 4, "pass twiddles exist for the radix-8 and radix-16 schedules");
-    static constexpr int v = (2 << LOGL) + twp_pass_offset(sizeof(V) == 16, LE, LOGL, PASS);
+    static constexpr int v = (2 << LOGL) + twp_pass_offset(sizeof(T) == 16, LE, LOGL, PASS);
 };
 
 template <typename V, int R>
-__device__ __forceinline__ void twiddle_base(const V* __restrict__ tp, int k, TwBase<V, R>& b) {
+__device__ __forceinline__ void twiddle_base(const typename CTraits<V>::tw* __restrict__ tp, int k, TwBase<V, R>& b) {
+    using T = typename CTraits<V>::tw;
     constexpr int N = TwBase<V, R>::N;
-    if constexpr (sizeof(V) == 8 && N == 2) {
+    if constexpr (sizeof(T) == 8 && N == 2) {
         const float4 q = __ldg(reinterpret_cast<const float4*>(tp) + k);
-        b.t[0] = CTraits<V>::make(q.x, q.y);
-        b.t[1] = CTraits<V>::make(q.z, q.w);
+        b.t[0] = CTraits<T>::make(q.x, q.y);
+        b.t[1] = CTraits<T>::make(q.z, q.w);
     } else {
 #pragma unroll
         for (int r = 0; r < N; ++r) b.t[r] = ldgv(&tp[k * N + r]);
     }
 }
 
+// (pairs of sequences: the powers are formed in packed arithmetic too, so that
+// every factor is in both halves of its register pairs)
 template <typename V, int R>
 __device__ __forceinline__ void twiddle_powers(const TwBase<V, R>& b, V* w) {
-    if constexpr (sizeof(V) == 16 || R == 2) {
+    using T = typename CTraits<V>::tw;
+    auto base = [&](int i) -> V {
+        if constexpr (std::is_same<V, fp2>::value) return CTraits<V>::make(b.t[i].x, b.t[i].y);
+        else return b.t[i];
+    };
+    if constexpr (sizeof(T) == 16 || R == 2) {
 #pragma unroll
-        for (int r = 1; r < R; ++r) w[r] = b.t[r - 1];
+        for (int r = 1; r < R; ++r) w[r] = base(r - 1);
     } else if constexpr (R == 4) {
-        w[1] = b.t[0];
-        w[2] = b.t[1];
+        w[1] = base(0);
+        w[2] = base(1);
         w[3] = cmul(w[2], w[1]);
     } else {
-        w[1] = b.t[0];
-        w[4] = b.t[1];
+        w[1] = base(0);
+        w[4] = base(1);
         w[2] = cmul(w[1], w[1]);
         w[3] = cmul(w[2], w[1]);
         w[5] = cmul(w[4], w[1]);
@@ -254,14 +233,19 @@ __device__ __forceinline__ void twiddle_powers(const TwBase<V, R>& b, V* w) {
         }
     }
 }
+// v w (DIR < 0) or v conj(w)
+template <int DIR, typename V> __device__ __forceinline__ V tw_mul(V v, V w) {
+    if constexpr (std::is_same<V, fp2>::value) return DIR > 0 ? cmul_conj(v, w) : cmul(v, w);
+    else return cmul(v, DIR > 0 ? cconj(w) : w);
+}
 
 // ---------------------------------------------------------------- one pass
 // Twiddle table: tw[t] = exp(-2 pi i t / 2L), t in [0, 2L), followed by the
 // pass twiddles of the radix-8 and radix-16 schedules.
 template <typename V, int DIR, int E, int LOGL, int LOGC, bool ROWMAJOR, bool SYNC_FIRST, int LR, int LOGNS,
           bool FIRST, bool LAST, class LoadF, class StoreF>
-__device__ __forceinline__ void stockham_pass(V* __restrict__ sm, const V* __restrict__ tw, LoadF& load,
-                                              StoreF& store) {
+__device__ __forceinline__ void stockham_pass(V* __restrict__ sm, const typename CTraits<V>::tw* __restrict__ tw,
+                                              LoadF& load, StoreF& store) {
     constexpr int R = 1 << LR;
     constexpr int NB = E / R;
     constexpr int L = 1 << LOGL;
@@ -271,8 +255,9 @@ __device__ __forceinline__ void stockham_pass(V* __restrict__ sm, const V* __res
     constexpr int P = (L * C) / E;
     constexpr int LE = Log2<E>::v;
     static_assert(LOGNS % LE == 0, "passes start at multiples of the schedule's radix");
-    const V* __restrict__ tp = tw;
-    if constexpr (LOGNS > 0) tp = tw + TwpOffset<V, LE, LOGL, LOGNS / LE>::v;
+    using T = typename CTraits<V>::tw;
+    const T* __restrict__ tp = tw;
+    if constexpr (LOGNS > 0) tp = tw + TwpOffset<T, LE, LOGL, LOGNS / LE>::v;
     // Shared-memory indices: element (c, p) sits at spad(ROWMAJOR ? c L + p : p C + c).  Along
     // one butterfly the unpadded index grows by a fixed step S (loads: L/R, stores: NS; times C
     // when the sequences interleave) from a base b whose residue mod the padding period plus
@@ -316,7 +301,7 @@ __device__ __forceinline__ void stockham_pass(V* __restrict__ sm, const V* __res
             V w[R];
             twiddle_powers<V, R>(twb[b], w);
 #pragma unroll
-            for (int r = 1; r < R; ++r) v[b * R + r] = cmul(v[b * R + r], DIR > 0 ? cconj(w[r]) : w[r]);
+            for (int r = 1; r < R; ++r) v[b * R + r] = tw_mul<DIR>(v[b * R + r], w[r]);
         }
         Dft<R, DIR, V>::run(v + b * R);
     }
@@ -342,7 +327,7 @@ __device__ __forceinline__ void stockham_pass(V* __restrict__ sm, const V* __res
 // passes of radix E, then the remainder (LOGL mod log2 E) as one smaller-radix pass
 template <typename V, int DIR, int E, int LOGL, int LOGC, bool ROWMAJOR, bool SYNC_FIRST, int I, class LoadF,
           class StoreF, class HookF>
-__device__ __forceinline__ void run_passes(V* __restrict__ sm, const V* __restrict__ tw, LoadF& load,
+__device__ __forceinline__ void run_passes(V* __restrict__ sm, const typename CTraits<V>::tw* __restrict__ tw, LoadF& load,
                                            StoreF& store, HookF& after_first) {
     constexpr int LE = Log2<E>::v;
     constexpr int NFULL = LOGL / LE;
@@ -367,14 +352,15 @@ __device__ __forceinline__ void run_passes(V* __restrict__ sm, const V* __restri
 // may be reused from then on.
 template <typename V, int DIR, int E, int LOGL, int LOGC, bool ROWMAJOR, bool SYNC_FIRST = false, class LoadF,
           class StoreF, class HookF>
-__device__ __forceinline__ void block_fft(V* __restrict__ sm, const V* __restrict__ tw, LoadF load, StoreF store,
-                                          HookF after_first) {
+__device__ __forceinline__ void block_fft(V* __restrict__ sm, const typename CTraits<V>::tw* __restrict__ tw, LoadF load,
+                                          StoreF store, HookF after_first) {
     run_passes<V, DIR, E, LOGL, LOGC, ROWMAJOR, SYNC_FIRST, 0>(sm, tw, load, store, after_first);
 }
 
 template <typename V, int DIR, int E, int LOGL, int LOGC, bool ROWMAJOR, bool SYNC_FIRST = false, class LoadF,
           class StoreF>
-__device__ __forceinline__ void block_fft(V* __restrict__ sm, const V* __restrict__ tw, LoadF load, StoreF store) {
+__device__ __forceinline__ void block_fft(V* __restrict__ sm, const typename CTraits<V>::tw* __restrict__ tw, LoadF load,
+                                          StoreF store) {
     auto none = [] {};
     run_passes<V, DIR, E, LOGL, LOGC, ROWMAJOR, SYNC_FIRST, 0>(sm, tw, load, store, none);
 }

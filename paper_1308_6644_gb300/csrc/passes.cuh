@@ -95,17 +95,32 @@ template <> struct Prec<dfc> : Prec<double2> {
     static constexpr int col_e = NUASM_DF_COL_E, col_budget = NUASM_DF_COL_BUDGET, col_cmax = NUASM_DF_COL_CMAX;
 };
 
-template <typename V, int LOGNP> struct RowCfg {
+#ifndef NUASM_ROW_PAIR_MIN
+#define NUASM_ROW_PAIR_MIN 12   // smallest log2 N' of the paired FP32 row passes (type 2: one more)
+#endif
+// TYPE: 1, 2 or 3 (the pass)
+template <typename V, int LOGNP, int TYPE> struct RowCfg {
     static constexpr int NP = 1 << LOGNP;
     static constexpr int LB = Prec<V>::row_logbudget;
     static constexpr int LOGROWS = LOGNP >= LB ? 0 : (LB - LOGNP > LOGNP ? LOGNP : LB - LOGNP);
     static constexpr int ROWS = 1 << LOGROWS;
-    // merged even/odd engines (two sequences per row in one pass sequence)
-    static constexpr bool MERGE = !Prec<V>::f64 && LOGNP <= 12;
-    static constexpr int EF = (!Prec<V>::f64 && LOGNP >= 13) ? 16 : 8;   // single-sequence engines
-    static constexpr int EM = 16;                                         // merged engines
+    // FP32: the even and odd halves of a row's 2N'-point transforms run in one
+    // pass sequence: interleaved (MERGE without PAIR), or as one transform of
+    // pairs (PAIR: fp2, f32x2 arithmetic) with 16 pairs per thread at 128
+    // registers.  Pairs need a third fewer instructions but half the warps and
+    // wait on instruction fetch, so they win only where a row alone fills a CTA
+    // of 256 threads and more (measured, interleaved -> pairs: row_t1 N' = 512
+    // 12.2 -> 14.6 us, N' = 4096 147 -> 127 us; row_t2 N' = 2048 37.9 -> 40.9, N' =
+    // 4096 147 -> 150 us), and at N' = 8192, where two interleaved halves
+    // do not fit a CTA's registers and ran one after the other (row_t1 905 ->
+    // 743 us).
+    static constexpr bool MERGE = !Prec<V>::f64;
+    static constexpr bool PAIR = MERGE && LOGNP >= NUASM_ROW_PAIR_MIN + (TYPE == 2 ? 1 : 0);
+    static constexpr int EF = PAIR ? 16 : 8;   // single-sequence engines
+    static constexpr int EM = 16;              // merged engines
     static constexpr int P = (NP * ROWS) / EF;
-    static constexpr int MINB = (65536 / (P * Prec<V>::row_regs)) > 0 ? 65536 / (P * Prec<V>::row_regs) : 1;
+    static constexpr int REGS = PAIR ? 128 : Prec<V>::row_regs;
+    static constexpr int MINB = (65536 / (P * REGS)) > 0 ? 65536 / (P * REGS) : 1;
     static constexpr int SEQ = MERGE ? 2 * ROWS : ROWS;                  // sequences in the work buffer
     // The mode buffer M (NP x ROWS) between the forward and inverse transforms
     // lives inside the work buffer when the engines are merged (the forward
@@ -113,6 +128,7 @@ template <typename V, int LOGNP> struct RowCfg {
     // inverse one's first pass reads it all before its first write); the
     // sequential engines read it twice, so it gets its own space.
     static size_t smem() {
+        if (PAIR) return size_t(spad_size<fp2>(NP * ROWS)) * sizeof(fp2);
         return (size_t(spad_size<V>(NP * SEQ)) + (MERGE ? size_t(0) : size_t(NP) * ROWS)) * sizeof(V);
     }
 };
@@ -309,11 +325,11 @@ __device__ __forceinline__ V row_factor(int q, int row, int r0, const RowConst<V
 // row restricted to the kept modes (two folded N'-point FFTs), multiply by
 // T1x(kx) T1y(ky) E(kx, ky), inverse N'-point FFT, keep the N outputs.
 template <typename V, int LOGNP>
-__global__ void __launch_bounds__(RowCfg<V, LOGNP>::P, RowCfg<V, LOGNP>::MINB)
+__global__ void __launch_bounds__(RowCfg<V, LOGNP, 1>::P, RowCfg<V, LOGNP, 1>::MINB)
     row_t1_kernel(const MemT<V>* __restrict__ A, MemT<V>* __restrict__ B, const MemT<V>* __restrict__ tx,
                   const MemT<V>* __restrict__ ty, const typename STable<V>::type* __restrict__ s,
                   const V* __restrict__ tw, RowArgs a) {
-    using Cf = RowCfg<V, LOGNP>;
+    using Cf = RowCfg<V, LOGNP, 1>;
     constexpr int NP = Cf::NP, ROWS = Cf::ROWS, HALF = NP / 2;
     extern __shared__ unsigned char smem_raw[];
     V* S = reinterpret_cast<V*>(smem_raw);
@@ -335,13 +351,31 @@ __global__ void __launch_bounds__(RowCfg<V, LOGNP>::P, RowCfg<V, LOGNP>::MINB)
                         ? Mem<V>::ld(x[p + NP], sc) : zero;
         return sgn == 0 ? cadd(u, t) : cmul(csub(u, t), half_bin<V, -1, LOGNP, R0>(tw, p));
     };
+    // both halves of the fold at p (pairs)
+    [[maybe_unused]] auto folded2 = [&](int row, int p) -> fp2 {
+        if constexpr (Cf::PAIR) {
+            const V* x = A + (r0 + row) * Wp;
+            const V u = p < W && NUASM_IN_RANGE((r0 + row) * Wp + p, a_n, dbg::kRowLoad) ? x[p] : zero;
+            const V t = p + NP < W && NUASM_IN_RANGE((r0 + row) * Wp + p + NP, a_n, dbg::kRowLoad) ? x[p + NP] : zero;
+            return fp2_make(cadd(u, t), cmul(csub(u, t), half_bin<V, -1, LOGNP, R0>(tw, p)));
+        } else {
+            return CTraits<fp2>::zero();
+        }
+    };
     auto put = [&](int row, int pk, int sgn, V v) {
         const int pb = 2 * pk + sgn;
         const int q = pb < HALF ? pb : (pb >= 3 * HALF ? pb - NP : -1);
         if (q >= 0 && NUASM_IN_RANGE(row * NP + q, ROWS * NP, dbg::kRowModes))
             M[row * NP + q] = cmul(v, row_factor<V, ROWS>(q, row, r0, rc0, tx, ty, s, a));
     };
-    if constexpr (Cf::MERGE) {
+    if constexpr (Cf::PAIR) {
+        block_fft<fp2, -1, Cf::EM, LOGNP, Cf::LOGROWS, true>(
+            reinterpret_cast<fp2*>(smem_raw), tw, [&](int p, int c) { return folded2(c, p); },
+            [&](int pk, int c, fp2 v) {
+                put(c, pk, 0, fp2_first(v));
+                put(c, pk, 1, fp2_second(v));
+            });
+    } else if constexpr (Cf::MERGE) {
         block_fft<V, -1, Cf::EM, LOGNP, Cf::LOGROWS + 1, false>(
             S, tw, [&](int p, int cs) { return folded(cs >> 1, p, cs & 1); },
             [&](int pk, int cs, V v) { put(cs >> 1, pk, cs & 1, v); });
@@ -367,11 +401,11 @@ __global__ void __launch_bounds__(RowCfg<V, LOGNP>::P, RowCfg<V, LOGNP>::MINB)
 // multiply by T2x T2y E, then the inverse 2N' transform onto the window row
 // (even and odd outputs as two N'-point FFTs), keeping the W window entries.
 template <typename V, int LOGNP>
-__global__ void __launch_bounds__(RowCfg<V, LOGNP>::P, RowCfg<V, LOGNP>::MINB)
+__global__ void __launch_bounds__(RowCfg<V, LOGNP, 2>::P, RowCfg<V, LOGNP, 2>::MINB)
     row_t2_kernel(const MemT<V>* __restrict__ B, MemT<V>* __restrict__ A, const MemT<V>* __restrict__ tx,
                   const MemT<V>* __restrict__ ty, const typename STable<V>::type* __restrict__ s,
                   const V* __restrict__ tw, RowArgs a) {
-    using Cf = RowCfg<V, LOGNP>;
+    using Cf = RowCfg<V, LOGNP, 2>;
     constexpr int NP = Cf::NP, ROWS = Cf::ROWS, HALF = NP / 2;
     extern __shared__ unsigned char smem_raw[];
     V* S = reinterpret_cast<V*>(smem_raw);
@@ -444,7 +478,14 @@ __global__ void __launch_bounds__(RowCfg<V, LOGNP>::P, RowCfg<V, LOGNP>::MINB)
         if (u < W && NUASM_IN_RANGE((r0 + row) * Wp + u, a.np * Wp, dbg::kRowStore))
             A[(r0 + row) * Wp + u] = Mem<V>::st(v, sc);
     };
-    if constexpr (Cf::MERGE) {
+    if constexpr (Cf::PAIR) {
+        block_fft<fp2, +1, Cf::EM, LOGNP, Cf::LOGROWS, true, true>(
+            reinterpret_cast<fp2*>(smem_raw), tw, [&](int q, int c) { return fp2_make(get(c, q, 0), get(c, q, 1)); },
+            [&](int k, int c, fp2 v) {   // entries 2k and 2k + 1 of the row: 16 bytes (Wp and W are even)
+                if (2 * k < W && NUASM_IN_RANGE((r0 + c) * Wp + 2 * k + 1, a.np * Wp, dbg::kRowStore))
+                    *reinterpret_cast<float4*>(&A[(r0 + c) * Wp + 2 * k]) = make_float4(v.re.x, v.im.x, v.re.y, v.im.y);
+            });
+    } else if constexpr (Cf::MERGE) {
         block_fft<V, +1, Cf::EM, LOGNP, Cf::LOGROWS + 1, false, true>(
             S, tw, [&](int q, int cs) { return get(cs >> 1, q, cs & 1); },
             [&](int k, int cs, V v) { put(cs >> 1, k, cs & 1, v); });
@@ -464,10 +505,10 @@ __global__ void __launch_bounds__(RowCfg<V, LOGNP>::P, RowCfg<V, LOGNP>::MINB)
 // window row (even/odd halves, as in row_t2), written over the input row (all
 // reads happen in the first forward pass, before any write).
 template <typename V, int LOGNP>
-__global__ void __launch_bounds__(RowCfg<V, LOGNP>::P, RowCfg<V, LOGNP>::MINB)
+__global__ void __launch_bounds__(RowCfg<V, LOGNP, 3>::P, RowCfg<V, LOGNP, 3>::MINB)
     row_t3_kernel(MemT<V>* __restrict__ A, const MemT<V>* __restrict__ tx, const MemT<V>* __restrict__ ty,
                   const typename STable<V>::type* __restrict__ s, const V* __restrict__ tw, RowArgs a) {
-    using Cf = RowCfg<V, LOGNP>;
+    using Cf = RowCfg<V, LOGNP, 3>;
     constexpr int NP = Cf::NP, ROWS = Cf::ROWS, HALF = NP / 2;
     extern __shared__ unsigned char smem_raw[];
     V* S = reinterpret_cast<V*>(smem_raw);
@@ -488,6 +529,17 @@ __global__ void __launch_bounds__(RowCfg<V, LOGNP>::P, RowCfg<V, LOGNP>::MINB)
                         ? Mem<V>::ld(x[p + NP], sc) : zero;
         return sgn == 0 ? cadd(u, t) : cmul(csub(u, t), half_bin<V, -1, LOGNP, R0>(tw, p));
     };
+    // both halves of the fold at p (pairs)
+    [[maybe_unused]] auto folded2 = [&](int row, int p) -> fp2 {
+        if constexpr (Cf::PAIR) {
+            const V* x = A + (r0 + row) * Wp;
+            const V u = p < W && NUASM_IN_RANGE((r0 + row) * Wp + p, a_n, dbg::kRowLoad) ? x[p] : zero;
+            const V t = p + NP < W && NUASM_IN_RANGE((r0 + row) * Wp + p + NP, a_n, dbg::kRowLoad) ? x[p + NP] : zero;
+            return fp2_make(cadd(u, t), cmul(csub(u, t), half_bin<V, -1, LOGNP, R0>(tw, p)));
+        } else {
+            return CTraits<fp2>::zero();
+        }
+    };
     auto put_mode = [&](int row, int pk, int sgn, V v) {
         const int pb = 2 * pk + sgn;
         const int q = pb < HALF ? pb : (pb >= 3 * HALF ? pb - NP : -1);
@@ -505,7 +557,22 @@ __global__ void __launch_bounds__(RowCfg<V, LOGNP>::P, RowCfg<V, LOGNP>::MINB)
         if (u < W && NUASM_IN_RANGE((r0 + row) * Wp + u, a_n, dbg::kRowStore))
             A[(r0 + row) * Wp + u] = Mem<V>::st(v, sc);
     };
-    if constexpr (Cf::MERGE) {
+    if constexpr (Cf::PAIR) {
+        block_fft<fp2, -1, Cf::EM, LOGNP, Cf::LOGROWS, true>(
+            reinterpret_cast<fp2*>(smem_raw), tw, [&](int p, int c) { return folded2(c, p); },
+            [&](int pk, int c, fp2 v) {
+                put_mode(c, pk, 0, fp2_first(v));
+                put_mode(c, pk, 1, fp2_second(v));
+            });
+        __syncthreads();
+        block_fft<fp2, +1, Cf::EM, LOGNP, Cf::LOGROWS, true, true>(
+            reinterpret_cast<fp2*>(smem_raw), tw,
+            [&](int q, int c) { return fp2_make(get_mode(c, q, 0), get_mode(c, q, 1)); },
+            [&](int k, int c, fp2 v) {   // entries 2k and 2k + 1 of the row: 16 bytes (Wp and W are even)
+                if (2 * k < W && NUASM_IN_RANGE((r0 + c) * Wp + 2 * k + 1, a_n, dbg::kRowStore))
+                    *reinterpret_cast<float4*>(&A[(r0 + c) * Wp + 2 * k]) = make_float4(v.re.x, v.im.x, v.re.y, v.im.y);
+            });
+    } else if constexpr (Cf::MERGE) {
         block_fft<V, -1, Cf::EM, LOGNP, Cf::LOGROWS + 1, false>(
             S, tw, [&](int p, int cs) { return folded(cs >> 1, p, cs & 1); },
             [&](int pk, int cs, V v) { put_mode(cs >> 1, pk, cs & 1, v); });
@@ -926,29 +993,29 @@ inline RowArgs row_args(const nuasm_plan_s* P) {
 
 template <typename V, int LOGNP>
 cudaError_t launch_row(const nuasm_plan_s* P, int type, cudaStream_t st) {
-    using Cf = RowCfg<V, LOGNP>;
+    using C1 = RowCfg<V, LOGNP, 1>;
+    using C2 = RowCfg<V, LOGNP, 2>;
+    using C3 = RowCfg<V, LOGNP, 3>;
     using ST = typename STable<V>::type;
     using M = MemT<V>;
     const RowArgs a = row_args(P);
-    const size_t sm = Cf::smem();
     // double-float passes read the plan's twiddles as float pairs
     const V* tw = static_cast<const V*>(Mem<V>::scaled ? P->d.tw_df : P->d.tw);
     if (!tw) return cudaErrorInvalidValue;
     const ST* s = static_cast<const ST*>(P->d.s);
-    const int blocks = Cf::NP / Cf::ROWS;
     cudaError_t e;
     if (type == 1) {
-        if ((e = set_smem(row_t1_kernel<V, LOGNP>, sm)) != cudaSuccess) return e;
-        e = launch_chained(row_t1_kernel<V, LOGNP>, dim3(blocks), dim3(Cf::P), sm, st,
+        if ((e = set_smem(row_t1_kernel<V, LOGNP>, C1::smem())) != cudaSuccess) return e;
+        e = launch_chained(row_t1_kernel<V, LOGNP>, dim3(C1::NP / C1::ROWS), dim3(C1::P), C1::smem(), st,
                            static_cast<const M*>(P->d.bufA), static_cast<M*>(P->d.bufB),
                            static_cast<const M*>(P->d.t1x), static_cast<const M*>(P->d.t1y), s, tw, a);
     } else if (type == 3) {
-        if ((e = set_smem(row_t3_kernel<V, LOGNP>, sm)) != cudaSuccess) return e;
-        e = launch_chained(row_t3_kernel<V, LOGNP>, dim3(blocks), dim3(Cf::P), sm, st, static_cast<M*>(P->d.bufA),
+        if ((e = set_smem(row_t3_kernel<V, LOGNP>, C3::smem())) != cudaSuccess) return e;
+        e = launch_chained(row_t3_kernel<V, LOGNP>, dim3(C3::NP / C3::ROWS), dim3(C3::P), C3::smem(), st, static_cast<M*>(P->d.bufA),
                            static_cast<const M*>(P->d.t3x), static_cast<const M*>(P->d.t3y), s, tw, a);
     } else {
-        if ((e = set_smem(row_t2_kernel<V, LOGNP>, sm)) != cudaSuccess) return e;
-        e = launch_chained(row_t2_kernel<V, LOGNP>, dim3(blocks), dim3(Cf::P), sm, st,
+        if ((e = set_smem(row_t2_kernel<V, LOGNP>, C2::smem())) != cudaSuccess) return e;
+        e = launch_chained(row_t2_kernel<V, LOGNP>, dim3(C2::NP / C2::ROWS), dim3(C2::P), C2::smem(), st,
                            static_cast<const M*>(P->d.bufB), static_cast<M*>(P->d.bufA),
                            static_cast<const M*>(P->d.t2x), static_cast<const M*>(P->d.t2y), s, tw, a);
     }
