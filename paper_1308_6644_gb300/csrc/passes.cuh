@@ -679,6 +679,92 @@ __global__ void __launch_bounds__(ColCfg<V, LOGNP, MODE>::P, ColCfg<V, LOGNP, MO
     }
 }
 
+// --------------------------------------------------------------- paired column passes (FP32, N' = 8192)
+// A column of N' = 8192 leaves room for two columns per CTA and none for the
+// TMA pipeline's prefetch buffer.  One CTA takes two adjacent columns as one
+// transform of pairs (fp2, 16 pairs per thread, f32x2 arithmetic): 16-byte
+// accesses instead of 8-byte ones, and the folded modes' second half re-reads
+// its columns from L2, not from memory.  Against one column per CTA (and the
+// halves as separate CTAs), N = 4096: col_fwd_fold 1344 -> 907 us, col_inv 302 ->
+// 242 us.  What bounds it now: the latency of its strided loads (one CTA of 16
+// warps per SM; long_scoreboard 8.5 cycles per issue, DRAM 1.06 GB at 18%).
+template <int LOGNP> struct Col2Cfg {
+    static constexpr int NP = 1 << LOGNP, E = 16, P = NP / E;
+    static constexpr size_t SMEM = size_t(spad_size<fp2>(NP)) * sizeof(fp2);
+    static constexpr int BY_SMEM = int((228u * 1024u) / (SMEM + 1024u)), BY_REGS = 65536 / (P * 128);
+    static constexpr int MINB = BY_SMEM < BY_REGS ? BY_SMEM : BY_REGS;
+};
+template <int LOGNP, int MODE>
+__global__ void __launch_bounds__(Col2Cfg<LOGNP>::P, Col2Cfg<LOGNP>::MINB)
+    col2_kernel(const float2* __restrict__ src, float2* __restrict__ dst, const float2* __restrict__ tw, ColArgs a) {
+    using Cf = Col2Cfg<LOGNP>;
+    constexpr int NP = Cf::NP, HALF = NP / 2;
+    extern __shared__ unsigned char smem_raw[];
+    fp2* S = reinterpret_cast<fp2*>(smem_raw);
+    const int col0 = blockIdx.x * 2;
+    const int W = a.W, Wp = a.Wp, n = a.n;
+    constexpr bool SRC_W = MODE == COL_FWD_FOLD || MODE == COL_INV_FOLD;   // window-wide source and output
+    const int pitch = SRC_W ? Wp : n;
+    [[maybe_unused]] const int src_n = MODE == COL_FWD_FOLD ? W * Wp : MODE == COL_INV ? NP * n
+                                     : MODE == COL_FWD ? n * n : NP * Wp;
+    [[maybe_unused]] const int dst_n = MODE == COL_FWD_FOLD ? NP * Wp : MODE == COL_INV ? n * n
+                                     : MODE == COL_FWD ? NP * n : W * Wp;
+    pdl_allow_next();
+    pdl_wait();   // src comes from the previous kernel
+    auto ld = [&](int row) -> fp2 {
+        if (!NUASM_IN_RANGE(row * pitch + col0 + 1, src_n, dbg::kColLoad)) return CTraits<fp2>::zero();
+        const float4 v = *reinterpret_cast<const float4*>(&src[row * pitch + col0]);
+        return fp2{make_float2(v.x, v.z), make_float2(v.y, v.w)};
+    };
+    auto st = [&](int row, fp2 v) {
+        if (NUASM_IN_RANGE(row * pitch + col0 + 1, dst_n, dbg::kColStore))
+            *reinterpret_cast<float4*>(&dst[row * pitch + col0]) = make_float4(v.re.x, v.im.x, v.re.y, v.im.y);
+    };
+    // both columns times one factor (the scalar product's roundings)
+    auto times = [](fp2 v, float2 f) { return fp2_make(cmul(fp2_first(v), f), cmul(fp2_second(v), f)); };
+    if constexpr (MODE == COL_FWD_FOLD) {
+#pragma unroll 1
+        for (int sgn = 0; sgn < 2; ++sgn)
+            block_fft<fp2, -1, Cf::E, LOGNP, 0, true>(
+                S, tw,
+                [&](int p, int) -> fp2 {
+                    const fp2 u = p < W ? ld(p) : CTraits<fp2>::zero();
+                    const fp2 t = p + NP < W ? ld(p + NP) : CTraits<fp2>::zero();
+                    return sgn == 0 ? cadd(u, t) : times(csub(u, t), half_bin<float2, -1, LOGNP, Cf::E>(tw, p));
+                },
+                [&](int pk, int, fp2 v) {
+                    const int pb = 2 * pk + sgn;
+                    const int r = pb < HALF ? pb : (pb >= 3 * HALF ? pb - NP : -1);
+                    if (r >= 0) st(r, v);
+                });
+    } else if constexpr (MODE == COL_INV) {
+        block_fft<fp2, +1, Cf::E, LOGNP, 0, true>(
+            S, tw, [&](int p, int) { return ld(p); },
+            [&](int p, int, fp2 v) {
+                if (p < n) st(p, v);
+            });
+    } else if constexpr (MODE == COL_FWD) {
+        block_fft<fp2, -1, Cf::E, LOGNP, 0, true>(
+            S, tw, [&](int p, int) { return p < n ? ld(p) : CTraits<fp2>::zero(); },
+            [&](int p, int, fp2 v) { st(p, v); });
+    } else {
+#pragma unroll 1
+        for (int sgn = 0; sgn < 2; ++sgn)
+            block_fft<fp2, +1, Cf::E, LOGNP, 0, true>(
+                S, tw,
+                [&](int q, int) -> fp2 {
+                    const fp2 y = ld(q);
+                    if (sgn == 0) return y;
+                    const float2 f = half_bin<float2, +1, LOGNP, Cf::E>(tw, q);
+                    return times(y, q < HALF ? f : cneg(f));
+                },
+                [&](int k, int, fp2 v) {
+                    const int u = 2 * k + sgn;
+                    if (u < W) st(u, v);
+                });
+    }
+}
+
 // --------------------------------------------------------------- TMA column passes (FP32)
 // Persistent variant of col_kernel: each CTA walks column strips s, s + G, ...
 // One elected thread loads a strip (C columns x all needed rows) into a raw
@@ -1045,6 +1131,29 @@ cudaError_t launch_col(const nuasm_plan_s* P, const void* src, void* dst, int nc
     return cudaGetLastError();
 }
 
+// Paired columns; cudaErrorNotSupported when a caller's array is only 8-byte
+// aligned (ncols is even: W, N and the row pitches are), so the caller can fall back.
+template <int LOGNP, int MODE>
+cudaError_t launch_col2(const nuasm_plan_s* P, const void* src, void* dst, int ncols, cudaStream_t st) {
+    using Cf = Col2Cfg<LOGNP>;
+    if (((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) || (ncols & 1))
+        return cudaErrorNotSupported;
+    const ColArgs a{P->g.n, P->g.W, P->g.Wp};
+    cudaError_t e = set_smem(col2_kernel<LOGNP, MODE>, Cf::SMEM);
+    if (e != cudaSuccess) return e;
+    const dim3 grid(ncols / 2), block(Cf::P);
+    const float2* tw = static_cast<const float2*>(P->d.tw);
+    if constexpr (MODE == COL_FWD) {   // first kernel of the type-2 chain
+        col2_kernel<LOGNP, MODE><<<grid, block, Cf::SMEM, st>>>(static_cast<const float2*>(src),
+                                                                static_cast<float2*>(dst), tw, a);
+    } else {
+        e = launch_chained(col2_kernel<LOGNP, MODE>, grid, block, Cf::SMEM, st, static_cast<const float2*>(src),
+                           static_cast<float2*>(dst), tw, a);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaGetLastError();
+}
+
 // TMA variant (FP32, at least two columns per strip); returns cudaErrorNotSupported
 // when the source array breaks the TMA alignment rules, so the caller can fall back.
 template <int LOGNP, int MODE>
@@ -1128,6 +1237,10 @@ template <typename V, int LOGNP> struct Stages {
         if constexpr (kTma) {
             const cudaError_t e = launch_col_tma<LOGNP, MODE>(P, src, dst, ncols, src_cols, src_rows, src_pitch,
                                                               load_rows, s);
+            if (e != cudaErrorNotSupported) return e;
+        }
+        if constexpr (kTma && LOGNP == 13) {
+            const cudaError_t e = launch_col2<LOGNP, MODE>(P, src, dst, ncols, s);
             if (e != cudaErrorNotSupported) return e;
         }
         const int halves = (MODE == COL_FWD_FOLD || MODE == COL_INV_FOLD) ? 2 : 1;

@@ -83,3 +83,31 @@ def test_adjoint_at_a_distance(P, n, type_):
     finally:
         for p in plans:
             p.destroy()
+
+
+def test_arrays_off_the_16_byte_alignment_at_n_4096(P):
+    """The paired column passes of N' = 8192 need 16-byte aligned arrays; others
+    take the one-column passes (equal to FP32 rounding of another order of
+    operations: 2e-6)."""
+    import torch
+    n, pitch, rng, m = 4096, 4e-6, np.random.default_rng(73), 500
+    h = 0.5 * n * pitch * (1 - 1e-9)
+    plan = P.nuasm_plan(P.make_params(n, pitch, 633e-9, 0.05),
+                        *(torch.from_numpy(rng.uniform(-h, h, m)).cuda() for _ in range(2)))
+    try:
+        c = torch.from_numpy((rng.normal(size=m) + 1j * rng.normal(size=m)).astype(np.complex64)).cuda()
+        buf = torch.zeros(n * n + 1, dtype=torch.complex64, device="cuda")
+        out = [buf[:-1], torch.zeros(n * n + 1, dtype=torch.complex64, device="cuda")[1:]]
+        for u in out:
+            P.nuasm1_execute(plan, c, u)
+        src = torch.zeros(n * n + 1, dtype=torch.complex64, device="cuda")[1:]
+        src.copy_(out[0])
+        v = [torch.zeros_like(c) for _ in range(2)]
+        P.nuasm2_execute(plan, out[0], v[0])
+        P.nuasm2_execute(plan, src, v[1])
+        torch.cuda.synchronize()
+        assert out[1].data_ptr() % 16 == 8 and src.data_ptr() % 16 == 8
+        assert O.rel_l2(out[1].cpu().numpy(), out[0].cpu().numpy()) < 2e-6
+        assert O.rel_l2(v[1].cpu().numpy(), v[0].cpu().numpy()) < 2e-6
+    finally:
+        plan.destroy()
