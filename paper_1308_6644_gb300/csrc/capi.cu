@@ -180,7 +180,7 @@ cudaError_t upload_tables(nuasm_plan_s* P, const HostTables& t, cudaStream_t st)
     P->d.tw = base + tw_off;
     P->d.tw_df = P->f64 ? base + bytes : nullptr;
     std::vector<char> host(bytes + df_bytes);
-    pack_tables(t, P->g, P->f64, true, host.data());
+    pack_tables(t, P->g, P->f64, true, host.data(), P->texp);
     if (P->f64) {
         const double* tw = reinterpret_cast<const double*>(host.data() + tw_off);
         float* out = reinterpret_cast<float*>(host.data() + bytes);

@@ -104,62 +104,62 @@ __device__ __forceinline__ double dfr_pow2(int k) {
     return __longlong_as_double(static_cast<long long>(k + 1023) << 52);
 }
 
-// x 2^-s (s in [-1022, 1023]) as a double-float by integer operations on the
-// bits: hi the leading 24 significant bits of x (truncated), lo the next 23,
-// relative error below 2^-46.  The caller picks s so that the result stays
-// within the float range.  A subnormal x is first scaled by 2^-s in FP64
-// (exact while the product is normal); zeros and values below 2^-100 after
-// the scaling give zero, infinities and NaNs give themselves in hi.
-__device__ __forceinline__ dfr dfr_split(double x, int s) {
+// The general conversions (infinities, NaNs, subnormals, exponents outside the
+// float range), out of line.
+static __device__ __noinline__ dfr dfr_split_any(double x, int s) {
     unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
     int ex = int(b >> 52) & 0x7ff;
     if (ex == 0x7ff) return dfr(__double2float_rn(x), 0.f);
     if (ex == 0) {   // zero or subnormal
         if ((b << 1) == 0 || s > -923) return dfr(0.f, 0.f);   // zero, or below 2^-100 of 2^s
-        b = static_cast<unsigned long long>(__double_as_longlong(x * dfr_pow2(-s)));
-        ex = int(b >> 52) & 0x7ff;
+        x *= dfr_pow2(-s);
         s = 0;
+    } else {
+        const int e = ex - 1023 - s;
+        if (e < -100) return dfr(0.f, 0.f);
+        x = scalbn(x, -s);
     }
-    const int e = ex - 1023 - s;
-    if (e < -100) return dfr(0.f, 0.f);
-    const unsigned sign = unsigned(b >> 32) & 0x80000000u;
-    const unsigned hb = sign | (unsigned(e + 127) << 23) | unsigned((b >> 29) & 0x7fffffu);
-    const unsigned r = unsigned(b) & 0x1fffffffu;   // the 29 mantissa bits below hi
-    const unsigned lb = unsigned(e - 23 + 127) << 23;
-    const float lo = __uint_as_float(lb | (r >> 6)) - __uint_as_float(lb);   // (r >> 6) 2^(e - 46), exact
-    return dfr(__uint_as_float(hb), sign ? -lo : lo);
+    const float hi = float(x);
+    return dfr(hi, float(x - double(hi)));
+}
+static __device__ __noinline__ double dfr_to_double_any(dfr a, int s) {
+    if (a.hi == 0.f) return 0.0;
+    if (!isfinite(a.hi)) return double(a.hi);
+    return scalbn(double(a.hi) + double(a.lo), s);
 }
 
-// (hi + lo) 2^s as a double by integer operations (the 53 leading bits of
-// the exact sum, truncated), for a normalised pair (|lo| below ulp(hi)); a
-// result outside the normal double range (subnormal, or beyond the largest
-// double) is formed in FP64 arithmetic instead.  Zeros and subnormal hi give
-// zero; infinities and NaNs give themselves.
+// x 2^-s (s in [-1022, 1023]) as a double-float by integer operations on the
+// bits: hi the leading 24 significant bits of x (truncated), lo the next 23,
+// relative error below 2^-46.  Values below 2^-100 after the scaling give zero,
+// infinities and NaNs give themselves in hi.  (An FP64 conversion holds the
+// FP64 pipe for 64 cycles a warp.)
+__device__ __forceinline__ dfr dfr_split(double x, int s) {
+    const unsigned h = unsigned(__double2hiint(x)), l = unsigned(__double2loint(x));
+    const int ex = int(h >> 20) & 0x7ff, e = ex - 1023 - s;
+    if (e > 126 || ex == 0x7ff || s < -900) return dfr_split_any(x, s);
+    const unsigned sign = h & 0x80000000u;
+    const unsigned hb = sign | (unsigned(e + 127) << 23) | (__funnelshift_l(l, h, 3) & 0x7fffffu);
+    const unsigned lb = unsigned(e + 104) << 23;   // 2^(e - 23); the mantissa bits below hi's go behind it
+    const float lo = __uint_as_float(lb | ((l >> 6) & 0x7fffffu)) - __uint_as_float(lb);
+    const bool tiny = e < -100;
+    return dfr(tiny ? 0.f : __uint_as_float(hb), tiny ? 0.f : __uint_as_float(__float_as_uint(lo) ^ sign));
+}
+
+// (hi + lo) 2^s as a double: hi's bits, plus lo in units of 2^-29 ulp(hi) (of
+// 2^-30 where a power of two loses to a lo of the other sign), for a
+// normalised pair (|lo| at most an ulp of hi).  Infinities and NaNs give
+// themselves.
 __device__ __forceinline__ double dfr_to_double(dfr a, int s) {
-    const unsigned hb = __float_as_uint(a.hi), lb = __float_as_uint(a.lo);
-    const int eh = int(hb >> 23) & 0xff;
+    const unsigned u = __float_as_uint(a.hi), sign = u & 0x80000000u;
+    const int eh = int(u >> 23) & 0xff, E = eh - 127 + 1023 + s;
     if (eh == 0) return 0.0;
-    if (eh == 0xff) return double(a.hi);
-    // |hi| = Mh 2^(eh - 150); X = Mh 2^39 in units of 2^(eh - 189)
-    long long X = static_cast<long long>((hb & 0x7fffffu) | 0x800000u) << 39;
-    const int el = int(lb >> 23) & 0xff;
-    if (el != 0) {
-        const long long L = static_cast<long long>((lb & 0x7fffffu) | 0x800000u);
-        const int d = eh - el;   // lo's mantissa sits d bits below hi's
-        const long long Ls = d <= 39 ? (d >= 0 ? L << (39 - d) : 0) : (d - 39 < 63 ? L >> (d - 39) : 0);
-        X = ((hb ^ lb) >> 31) ? X - Ls : X + Ls;
-    }
-    const int lz = __clzll(X);                  // leading bit at 63 - lz
-    const int E = eh - 126 - lz + s;            // unbiased exponent of the result
-    if (E < -1022 || E > 1023) {                // s is within [-1022, 1023]: two exact halves
-        const int s1 = s / 2;
-        return ((double(a.hi) + double(a.lo)) * dfr_pow2(s1)) * dfr_pow2(s - s1);
-    }
-    const unsigned long long m = lz <= 11 ? static_cast<unsigned long long>(X) >> (11 - lz)
-                                          : static_cast<unsigned long long>(X) << (lz - 11);
-    const unsigned long long bits = (static_cast<unsigned long long>(hb >> 31) << 63) |
-                                    (static_cast<unsigned long long>(E + 1023) << 52) | (m & 0xfffffffffffffull);
-    return __longlong_as_double(static_cast<long long>(bits));
+    if (eh < 53 || eh == 255 || E < 2 || E > 2045) return dfr_to_double_any(a, s);
+    // lo times +-2^29 / ulp(hi), the sign hi's
+    int i = __float2int_rn(a.lo * __uint_as_float(sign | (unsigned(127 + 127 + 23 + 29 - eh) << 23)));
+    const unsigned m = u & 0x7fffffu;
+    if (m == 0 && i < 0) i *= 2;
+    const unsigned bh = sign | (unsigned(E) << 20) | (m >> 3), bl = m << 29;
+    return __longlong_as_double((static_cast<long long>((static_cast<unsigned long long>(bh) << 32) | bl)) + i);
 }
 
 }  // namespace nuasm

@@ -330,6 +330,25 @@ struct GridArgs {
     __device__ int skew_of(int tile) const { return tskew ? int(tskew[tile]) : skew; }
 };
 
+// exponent k of a double with 2^k <= |x| < 2^(k+1) (-1023 for zeros and
+// subnormals, 1024 for infinities and NaNs)
+__device__ __forceinline__ int dexp(double x) {
+    return (int(static_cast<unsigned long long>(__double_as_longlong(x)) >> 52) & 0x7ff) - 1023;
+}
+
+
+// The exponent of a solve's values for its double-float FFT passes (FP64): the
+// threads keep a maximum, each warp adds its own to the solve's word.
+__device__ __forceinline__ void note_expo(float2, int&) {}
+__device__ __forceinline__ void note_expo(double2 v, int& em) { em = max(em, max(dexp(v.x), dexp(v.y))); }
+template <typename S> __device__ __forceinline__ void report_expo([[maybe_unused]] int em, [[maybe_unused]] int* expo) {
+    if constexpr (sizeof(S) == 8) {
+        if (!expo) return;
+        em = __reduce_max_sync(0xffffffffu, em);
+        if ((threadIdx.x & 31) == 0) atomicMax(expo, em);
+    }
+}
+
 // --------------------------------------------------------------- spreading (type 1)
 // EXACT: the kernel width is WMAX itself (compile-time loops); else w <= WMAX at run time.
 // Three accumulation schemes, picked by precision and tile side in spread_impl:
@@ -363,10 +382,11 @@ __global__ void __launch_bounds__(256, sizeof(S) == 4 ? NUASM_SPREAD_MINB : 1) s
                                                      const typename VecOf<S>::type* __restrict__ c,
                                                      typename VecOf<S>::type* __restrict__ win, GridArgs a,
                                                      const typename PolyOf<S>::type kp,
-                                                     const int4* __restrict__ items) {
+                                                     const int4* __restrict__ items, int* __restrict__ expo) {
     using V = typename VecOf<S>::type;
     extern __shared__ unsigned char smem_raw[];
     int tile, b, e, chunked = 0;
+    int em = -1023;   // FP64: the largest exponent among the values, for the double-float FFT passes
     if (items) {   // a chunk of a tile's records (several CTAs add into the tile)
         const int4 it = items[blockIdx.x];
         tile = it.x;
@@ -393,6 +413,7 @@ __global__ void __launch_bounds__(256, sizeof(S) == 4 ? NUASM_SPREAD_MINB : 1) s
         const int lx = int(r.cell & 0xffffu) - x0, ly = int(r.cell >> 16) - y0;
         V val = c[r.j];
         if (wpt) { const S wt = S(wpt[r.j]); val.x *= wt; val.y *= wt; }
+        note_expo(val, em);
         S wx[WMAX], wy[WMAX];
         tap_weights<WMAX>(S(r.fx), kp, wx);
         tap_weights<WMAX>(S(r.fy), kp, wy);
@@ -413,6 +434,7 @@ __global__ void __launch_bounds__(256, sizeof(S) == 4 ? NUASM_SPREAD_MINB : 1) s
             }
         }
     }
+    report_expo<S>(em, expo);
     __syncthreads();
     for (int i = threadIdx.x; i < T * T; i += blockDim.x) {
         const int yy = i / T, xx = i - yy * T;
@@ -640,12 +662,14 @@ __global__ void __launch_bounds__(256, 2) spread_private_kernel(const typename R
                                                              const typename VecOf<S>::type* __restrict__ c,
                                                              typename VecOf<S>::type* __restrict__ win, GridArgs a,
                                                              const typename PolyOf<S>::type kp,
-                                                             const int4* __restrict__ items) {
+                                                             const int4* __restrict__ items,
+                                                             int* __restrict__ expo) {
     using V = typename VecOf<S>::type;
     using Rec = typename RecOf<S>::type;
     extern __shared__ unsigned char smem_raw[];
     V* copies = reinterpret_cast<V*>(smem_raw);
     int tile, b, e, chunked = 0;
+    int em = -1023;   // FP64: the largest exponent among the values, for the double-float FFT passes
     if (items) {   // a chunk of a tile's records (several CTAs add into the tile)
         const int4 it = items[blockIdx.x];
         tile = it.x;
@@ -680,6 +704,7 @@ __global__ void __launch_bounds__(256, 2) spread_private_kernel(const typename R
         if (live) {
             val = c[r.j];
             if (wpt) { const S wt = S(wpt[r.j]); val.x *= wt; val.y *= wt; }
+            note_expo(val, em);
         }
         S wx[WMAX], wy[WMAX];
         tap_weights<WMAX>(S(r.fx), kp, wx);
@@ -713,6 +738,7 @@ __global__ void __launch_bounds__(256, 2) spread_private_kernel(const typename R
         }
         __syncwarp();
     }
+    report_expo<S>(em, expo);
     __syncthreads();
     for (int i = threadIdx.x; i < T * T; i += blockDim.x) {
         const int yy = i / T, xx = i - yy * T;
@@ -887,12 +913,6 @@ __global__ void __launch_bounds__(kInterpThreads, sizeof(S) == 4 ? NUASM_INTERP_
 __device__ __forceinline__ df df_split(double x, int s) {
     const dfr r = dfr_split(x, s);
     return {r.hi, r.lo};
-}
-
-// exponent k of a double with 2^k <= |x| < 2^(k+1) (-1023 for zeros and
-// subnormals, 1024 for infinities and NaNs)
-__device__ __forceinline__ int dexp(double x) {
-    return (int(static_cast<unsigned long long>(__double_as_longlong(x)) >> 52) & 0x7ff) - 1023;
 }
 
 // Two double-floats side by side, their high and their low parts each a
@@ -1092,7 +1112,7 @@ __global__ void __launch_bounds__(256, WMAX <= 13 ? NUASM_DF_SPREAD_MINB : 2) sp
                                                           const int* __restrict__ order,
                                                           const double2* __restrict__ c, double2* __restrict__ win,
                                                           GridArgs a, const KernelPolyDF kp,
-                                                          const int4* __restrict__ items) {
+                                                          const int4* __restrict__ items, int* __restrict__ expo) {
     constexpr int NT = 256, RPB = kDfBatch / NT;
     extern __shared__ unsigned char smem_raw[];
     __shared__ float4 cs[(WMAX + 1) / 2 * kDfSteps];
@@ -1184,6 +1204,7 @@ __global__ void __launch_bounds__(256, WMAX <= 13 ? NUASM_DF_SPREAD_MINB : 2) sp
         }
         __syncthreads();   // the previous batch's fold is done before the sum reuses red
         const double S = block_sum(part);
+        if (expo && threadIdx.x == 0) atomicMax(expo, dexp(S));   // for the double-float FFT passes
         if (S == 0.0) continue;
         if (!(S <= 1.7976931348623157e308)) {   // infinity or NaN among the values
             nonfinite = true;
@@ -1396,6 +1417,13 @@ template <typename K> cudaError_t set_smem(K kernel, size_t bytes) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
 }
 
+// the solve's exponent word where its FFT passes are double-float (null elsewhere), below every exponent
+cudaError_t clear_expo(const nuasm_plan_s* P, int** expo, cudaStream_t st) {
+    if (!fft_double_float(P->f64, P->g.np)) return cudaSuccess;
+    *expo = expo_words(P);
+    return cudaMemsetAsync(*expo, 0x80, sizeof(int), st);
+}
+
 // the tap polynomials of the plan's precision
 template <typename S> typename PolyOf<S>::type taps_arg(const nuasm_plan_s* P) {
     if constexpr (sizeof(S) == 8) return P->poly64;
@@ -1409,6 +1437,8 @@ cudaError_t spread_impl(const nuasm_plan_s* P, const void* c, cudaStream_t st) {
     // chunked tiles add into a cleared window
     const int4* items = P->d.spread_items;
     const int grid = items ? P->n_spread_items : P->g.ntiles;
+    int* expo = nullptr;
+    if (cudaError_t e = clear_expo(P, &expo, st); e != cudaSuccess) return e;
     auto clear = [&]() -> cudaError_t {
         return items ? cudaMemsetAsync(P->d.win, 0, ws_win_elems(P->g) * sizeof(V), st) : cudaSuccess;
     };
@@ -1422,7 +1452,7 @@ cudaError_t spread_impl(const nuasm_plan_s* P, const void* c, cudaStream_t st) {
         if (e != cudaSuccess) return e;
         spread_private_kernel<S, WMAX, EXACT><<<grid, 256, sm, st>>>(
             static_cast<const typename RecOf<S>::type*>(P->d.rec), P->d.tile_off, P->d.wpt, P->d.tile_order,
-            static_cast<const V*>(c), static_cast<V*>(P->d.win), a, taps_arg<S>(P), items);
+            static_cast<const V*>(c), static_cast<V*>(P->d.win), a, taps_arg<S>(P), items, expo);
         return cudaGetLastError();
     }
     if constexpr (sizeof(S) == 4) {
@@ -1442,7 +1472,7 @@ cudaError_t spread_impl(const nuasm_plan_s* P, const void* c, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     spread_kernel<S, WMAX, EXACT><<<grid, 256, sm, st>>>(
         static_cast<const typename RecOf<S>::type*>(P->d.rec), P->d.tile_off, P->d.wpt, P->d.tile_order,
-        static_cast<const V*>(c), static_cast<V*>(P->d.win), a, taps_arg<S>(P), items);
+        static_cast<const V*>(c), static_cast<V*>(P->d.win), a, taps_arg<S>(P), items, expo);
     return cudaGetLastError();
 }
 
@@ -1471,12 +1501,15 @@ template <int WMAX> cudaError_t spread_df_impl(const nuasm_plan_s* P, const void
     const int4* items = P->d.spread_items;   // chunks of split tiles add into a cleared window
     cudaError_t e = items ? cudaMemsetAsync(P->d.win, 0, ws_win_elems(P->g) * sizeof(double2), st) : cudaSuccess;
     if (e != cudaSuccess) return e;
+    int* expo = nullptr;
+    if ((e = clear_expo(P, &expo, st)) != cudaSuccess) return e;
     const size_t sm = size_t(4) * a.T * plane_stride(a.T, a.max_skew) * sizeof(int);
     if ((e = set_smem(spread_df_kernel<WMAX>, sm)) != cudaSuccess) return e;
     const int grid = items ? P->n_spread_items : P->g.ntiles;
     spread_df_kernel<WMAX><<<grid, 256, sm, st>>>(static_cast<const RecD*>(P->d.rec), P->d.tile_off, P->d.wpt,
                                                   P->d.tile_order, static_cast<const double2*>(c),
-                                                  static_cast<double2*>(P->d.win), a, P->poly64df, items);
+                                                  static_cast<double2*>(P->d.win), a, P->poly64df, items,
+                                                  expo);
     return cudaGetLastError();
 }
 

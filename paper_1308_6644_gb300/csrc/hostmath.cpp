@@ -3,6 +3,7 @@
 // the per-axis transfer-function tables (Eq. 4 separable part, Eq. 5) and the
 // FFT twiddles.  Everything here runs once per plan in FP64 (double-double
 // where a phase can exceed 1e5 cycles).
+#include <algorithm>
 #include <cmath>
 #include <complex>
 #include <cstdlib>
@@ -459,7 +460,7 @@ void pack_twp(const double* tw, int logl, bool f64, void* dst) {
 
 // Device image of the tables: T1x T1y T2x T2y T3x T3y (complex, plan precision),
 // s (double, or float hi/lo pairs), then the twiddles when present.
-void pack_tables(const HostTables& t, const Geometry& g, bool f64, bool with_twiddles, void* dst) {
+void pack_tables(const HostTables& t, const Geometry& g, bool f64, bool with_twiddles, void* dst, int texp[3]) {
     const int np = g.np;
     const size_t eb = f64 ? 16 : 8;
     char* out = static_cast<char*>(dst);
@@ -471,7 +472,31 @@ void pack_tables(const HostTables& t, const Geometry& g, bool f64, bool with_twi
         }
     };
     const double* six[6] = {t.t1x, t.t1y, t.t2x, t.t2y, t.t3x, t.t3y};
-    for (int i = 0; i < 6; ++i) put_c(size_t(i) * np * eb, six[i], np);
+    texp[0] = texp[1] = texp[2] = 0;
+    if (fft_double_float(f64, np)) {
+        int ex[6] = {};
+        for (int i = 0; i < 6; ++i) {
+            double top = 0.0;
+            for (int k = 0; k < 2 * np; ++k) top = std::max(top, std::fabs(six[i][k]));
+            if (i >= 4) {
+                ex[i] = ex[i - 2];   // type 3 shares type 2's inverse column pass and its exponents
+            } else if (top > 0.0 && std::isfinite(top)) {
+                std::frexp(top, &ex[i]);
+                ex[i] -= 1;
+            }
+            const int e = ex[i];
+            texp[i / 2] += e;
+            float* d = reinterpret_cast<float*>(out + size_t(i) * np * eb);
+            for (int k = 0; k < 2 * np; ++k) {
+                const double v = std::ldexp(six[i][k], -e);
+                const float hi = float(v);
+                d[4 * (k / 2) + (k & 1)] = hi;
+                d[4 * (k / 2) + 2 + (k & 1)] = float(v - double(hi));
+            }
+        }
+    } else {
+        for (int i = 0; i < 6; ++i) put_c(size_t(i) * np * eb, six[i], np);
+    }
     const size_t soff = 6 * size_t(np) * eb;
     if (f64) std::memcpy(out + soff, t.s, sizeof(double) * np);
     else {

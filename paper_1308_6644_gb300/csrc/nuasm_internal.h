@@ -107,6 +107,7 @@ struct nuasm_plan_s {
     bool has_w = false;
     bool f64 = false;
     double rc = 0.0;            // z / (2 lambda)
+    int texp[3] = {0, 0, 0};    // double-float FFT passes: power of two taken out of type t's tables
     int nonsep_mode = 0;        // ASM non-separable phase: 0 none, 1 plain, 2 double-float
     int etab_pitch = 0;         // entries per row of d.etab
     int skew = 0;               // bank skew of the gridding tile layouts and record order: the one most
@@ -171,7 +172,11 @@ void build_tables(const nuasm_params_t& p, const Geometry& g, HostTables* t, con
 void phihat_table(const Geometry& g, double* out);
 void free_tables(HostTables* t);
 size_t table_bytes(const Geometry& g, bool f64, bool with_twiddles);
-void pack_tables(const HostTables& t, const Geometry& g, bool f64, bool with_twiddles, void* dst);
+// Double-float plans (fft_double_float) get the six factor tables as pairs of
+// floats (re.hi, im.hi, re.lo, im.lo), each scaled by a power of two to a
+// largest component in [1, 2) (type 3's by type 2's powers); texp[t - 1] receives
+// the sum of type t's two exponents.
+void pack_tables(const HostTables& t, const Geometry& g, bool f64, bool with_twiddles, void* dst, int texp[3]);
 
 // Pass twiddles.  The full twiddle table tw[t] = exp(-2 pi i t / 2N'),
 // t < 2N', is followed by the twiddle bases of every pass I >= 1 of the
@@ -225,7 +230,20 @@ cudaError_t chain_type3(nuasm_plan_s* P, const nuasm_plan_s* Q, const void* c, v
 // workspace elements (complex) of a geometry: window W x Wp, bufA N' x Wp, bufB N' x N
 inline size_t ws_win_elems(const Geometry& g) { return size_t(g.W) * g.Wp; }
 inline size_t ws_bufA_elems(const Geometry& g) { return size_t(g.np) * g.Wp; }
-inline size_t ws_bufB_elems(const Geometry& g) { return size_t(g.np) * g.n; }
+// (bufB ends with the exponents of expo_words)
+constexpr int kExpoWords = 2080;
+inline size_t ws_bufB_elems(const Geometry& g) { return size_t(g.np) * g.n + kExpoWords * sizeof(int) / 8; }
+// FP64 plans from N' = 512 up run their FFT passes in double-float arithmetic
+// (passes.cuh): the mode-side arrays bufA and bufB and the transfer-function
+// tables then hold pairs of floats (dfc), the window and the caller's arrays FP64
+constexpr int kDfMinNp = 512;
+inline bool fft_double_float(bool f64, int np) { return f64 && np >= kDfMinNp; }
+// The exponents of a solve's double-float data, behind bufB's elements: word 0
+// the solve's (types 1 and 3: set by the spreading; type 2: by the row pass),
+// then type 2's one per strip of columns of the forward column pass.
+inline int* expo_words(const nuasm_plan_s* P) {
+    return reinterpret_cast<int*>(static_cast<char*>(P->d.bufB) + size_t(P->g.np) * P->g.n * 16);
+}
 
 // Resource acquisition (resources.cu): device, pool and pinned host
 // allocations, streams, events and graph instantiations, with a count of the

@@ -6,6 +6,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "dfloat.cuh"
 #include "nuasm_internal.h"
 #include "tma.cuh"
 
@@ -110,7 +111,8 @@ __global__ void etab_kernel(V* __restrict__ out, int half, int pitch, double c, 
                 sincospi(-2.0 * (r - rint(r)), &im, &re);
             }
         }
-        out[i] = CTraits<V>::make(re, im);
+        using R = typename CTraits<V>::real;
+        out[i] = CTraits<V>::make(R(re), R(im));
     }
 }
 }  // namespace
@@ -144,7 +146,9 @@ cudaError_t build_etab(const nuasm_plan_s* P, cudaStream_t s) {
     const double k = P->p.lambda / (double(P->g.np) * P->p.pitch);
     const int threads = 256;
     const int blocks = int(std::min<size_t>((n + threads - 1) / threads, size_t(152) * 8));
-    if (P->f64)
+    if (fft_double_float(P->f64, P->g.np))
+        etab_kernel<<<blocks, threads, 0, s>>>(static_cast<dfc*>(P->d.etab), P->g.np / 2, pitch, k * k, P->rc);
+    else if (P->f64)
         etab_kernel<<<blocks, threads, 0, s>>>(static_cast<double2*>(P->d.etab), P->g.np / 2, pitch, k * k, P->rc);
     else
         etab_kernel<<<blocks, threads, 0, s>>>(static_cast<float2*>(P->d.etab), P->g.np / 2, pitch, k * k, P->rc);

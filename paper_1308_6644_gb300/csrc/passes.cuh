@@ -153,23 +153,24 @@ template <> struct STable<float2> { using type = float2; };
 template <> struct STable<double2> { using type = double; };
 template <> struct STable<dfc> { using type = double; };
 
-// Global-memory element type of a pass's register type and the conversions
-// between them: the identity, except for double-float registers over FP64
-// arrays (scale s: the arrays hold the values times 2^s, so that a CTA's data
-// stays in the float range).
-template <typename V> struct Mem {
+// Element type of the arrays outside the mode side (the window, the caller's
+// planes) and the conversions from and to a pass's registers: the identity,
+// except that the double-float passes meet FP64 there (scale s: the registers
+// hold the values times 2^-s, so that a solve's data stays in the float
+// range).  The mode-side arrays and the tables hold the register type.
+template <typename V> struct Ext {
     using type = V;
     static constexpr bool scaled = false;
     __device__ static V ld(V x, int) { return x; }
     __device__ static V st(V v, int) { return v; }
 };
-template <> struct Mem<dfc> {
+template <> struct Ext<dfc> {
     using type = double2;
     static constexpr bool scaled = true;
     __device__ static dfc ld(double2 x, int sc) { return CTraits<dfc>::make(dfr_split(x.x, sc), dfr_split(x.y, sc)); }
     __device__ static double2 st(dfc v, int sc) { return make_double2(dfr_to_double(v.x(), sc), dfr_to_double(v.y(), sc)); }
 };
-template <typename V> using MemT = typename Mem<V>::type;
+template <typename V> using ExtT = typename Ext<V>::type;
 
 __device__ __forceinline__ bool nonzero(float2 v) { return v.x != 0.f || v.y != 0.f; }
 __device__ __forceinline__ bool nonzero(double2 v) { return v.x != 0.0 || v.y != 0.0; }
@@ -180,29 +181,26 @@ __device__ __forceinline__ int dexp2(double x) {
     return (int(static_cast<unsigned long long>(__double_as_longlong(x)) >> 52) & 0x7ff) - 1023;
 }
 
-// The CTA's scale for double-float registers: the largest exponent among the
-// n elements at stride 1 of the rows r0 .. r0 + rows - 1 of an FP64 array
-// (row pitch `pitch`), clamped to the normal range; 0 for other types.  All
-// threads call it; it synchronises the block.
-template <typename V>
-__device__ __forceinline__ int cta_scale(const MemT<V>* __restrict__ x, int r0, int rows, int n, int pitch) {
-    if constexpr (!Mem<V>::scaled) {
-        return 0;
-    } else {
-        __shared__ int emax;
-        if (threadIdx.x == 0) emax = -1023;
-        __syncthreads();
-        int em = -1023;
-        for (int i = threadIdx.x; i < rows * n; i += blockDim.x) {
-            const int row = i / n, p = i - row * n;
-            const double2 v = x[size_t(r0 + row) * pitch + p];
-            em = max(em, max(dexp2(v.x), dexp2(v.y)));
-        }
-        em = __reduce_max_sync(0xffffffffu, em);
-        if ((threadIdx.x & 31) == 0) atomicMax(&emax, em);
-        __syncthreads();
-        return min(max(emax, -1022), 1023);
-    }
+__device__ __forceinline__ int clamp_expo(int e) { return min(max(e, -1022), 1023); }
+
+// The solve's scale for double-float registers: about the largest exponent
+// among its input values, clamped to the normal range; 0 for other types.  One
+// scale for the whole solve: the passes between need no conversion and no
+// extra look at their data, where a scale per CTA cost each pass a second read
+// of its source and a split and a reassembly of every value.
+template <typename V> __device__ __forceinline__ int solve_scale(const int* __restrict__ expo) {
+    if constexpr (!Ext<V>::scaled) return 0;
+    else return clamp_expo(__ldg(expo));
+}
+
+// the largest of one int per thread, to every thread (one barrier before the caller's next use of it)
+__device__ __forceinline__ int block_max(int v) {
+    __shared__ int wmax[32];
+    v = __reduce_max_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = v;
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    return __reduce_max_sync(0xffffffffu, lane < int(blockDim.x >> 5) ? wmax[lane] : -2000);
 }
 
 struct RowArgs {
@@ -214,10 +212,13 @@ struct RowArgs {
     const void* etab2;     // type 2: T2x(kx) E(|kx|, |ky|), rows of N' entries, or null
     int ep;                // entries per table row
     int np;                // N'
+    int* expo;             // double-float: the solve's exponents (expo_words)
 };
 
 struct ColArgs {
     int n, W, Wp;
+    int* expo;         // double-float: the solve's exponents (expo_words)
+    int texp;          // double-float: power of two taken out of the tables
 };
 
 // --------------------------------------------------------------- non-separable ASM factor
@@ -263,31 +264,31 @@ __device__ __forceinline__ double2 nonsep_factor(double sa, double sb, const Row
 template <typename V> struct RowConst {
     V ty;
     typename STable<V>::type s;
-    const MemT<V>* erow;
+    const V* erow;
 };
 
 template <typename V>
-__device__ __forceinline__ RowConst<V> row_const(int r, const MemT<V>* __restrict__ ty,
+__device__ __forceinline__ RowConst<V> row_const(int r, const V* __restrict__ ty,
                                                  const typename STable<V>::type* __restrict__ s, const RowArgs& a) {
-    const MemT<V>* erow = nullptr;
-    if (a.etab) erow = static_cast<const MemT<V>*>(a.etab) + size_t(min(r, a.np - r)) * a.ep;
-    return RowConst<V>{Mem<V>::ld(__ldg(&ty[r]), 0), __ldg(&s[r]), erow};
+    const V* erow = nullptr;
+    if (a.etab) erow = static_cast<const V*>(a.etab) + size_t(min(r, a.np - r)) * a.ep;
+    return RowConst<V>{ldgv(&ty[r]), __ldg(&s[r]), erow};
 }
 
 template <typename V>
-__device__ __forceinline__ V mode_factor(int q, const RowConst<V>& rc, const MemT<V>* __restrict__ tx,
+__device__ __forceinline__ V mode_factor(int q, const RowConst<V>& rc, const V* __restrict__ tx,
                                          const typename STable<V>::type* __restrict__ s, const RowArgs& a) {
-    V f = cmul(Mem<V>::ld(__ldg(&tx[q]), 0), rc.ty);
+    V f = cmul(ldgv(&tx[q]), rc.ty);
     if (rc.erow) {
-        f = cmul(f, Mem<V>::ld(__ldg(&rc.erow[min(q, a.np - q)]), 0));   // both loads in flight together
+        f = cmul(f, ldgv(&rc.erow[min(q, a.np - q)]));   // both loads in flight together
     } else if (a.nonsep && nonzero(f)) {
-        f = cmul(f, Mem<V>::ld(nonsep_factor(__ldg(&s[q]), rc.s, a), 0));
+        f = cmul(f, Ext<V>::ld(nonsep_factor(__ldg(&s[q]), rc.s, a), 0));
     }
     return f;
 }
 
 template <typename V>
-__device__ __forceinline__ V mode_factor(int q, int r, const MemT<V>* __restrict__ tx, const MemT<V>* __restrict__ ty,
+__device__ __forceinline__ V mode_factor(int q, int r, const V* __restrict__ tx, const V* __restrict__ ty,
                                          const typename STable<V>::type* __restrict__ s, const RowArgs& a) {
     return mode_factor<V>(q, row_const<V>(r, ty, s, a), tx, s, a);
 }
@@ -299,7 +300,7 @@ __device__ __forceinline__ V mode_factor(int q, int r, const MemT<V>* __restrict
 // same for every thread of the block.
 template <typename V, int ROWS>
 __device__ __forceinline__ bool stage_erows(V* dst, int r0, const RowArgs& a) {
-    using M = MemT<V>;
+    using M = V;
     if (!a.etab || (reinterpret_cast<uintptr_t>(dst) & 15)) return false;
     const int chunks = int((size_t(a.ep) * sizeof(M)) / 16);   // ep * sizeof(M) is a multiple of 16
     for (int i = threadIdx.x; i < ROWS * chunks; i += blockDim.x) {
@@ -313,8 +314,8 @@ __device__ __forceinline__ bool stage_erows(V* dst, int r0, const RowArgs& a) {
 
 // the factor of mode q in the CTA's row `row` (ROWS == 1: the constants held in registers)
 template <typename V, int ROWS>
-__device__ __forceinline__ V row_factor(int q, int row, int r0, const RowConst<V>& rc0, const MemT<V>* __restrict__ tx,
-                                        const MemT<V>* __restrict__ ty, const typename STable<V>::type* __restrict__ s,
+__device__ __forceinline__ V row_factor(int q, int row, int r0, const RowConst<V>& rc0, const V* __restrict__ tx,
+                                        const V* __restrict__ ty, const typename STable<V>::type* __restrict__ s,
                                         const RowArgs& a) {
     if constexpr (ROWS == 1) return mode_factor<V>(q, rc0, tx, s, a);
     else return mode_factor<V>(q, r0 + row, tx, ty, s, a);
@@ -326,8 +327,8 @@ __device__ __forceinline__ V row_factor(int q, int row, int r0, const RowConst<V
 // T1x(kx) T1y(ky) E(kx, ky), inverse N'-point FFT, keep the N outputs.
 template <typename V, int LOGNP>
 __global__ void __launch_bounds__(RowCfg<V, LOGNP, 1>::P, RowCfg<V, LOGNP, 1>::MINB)
-    row_t1_kernel(const MemT<V>* __restrict__ A, MemT<V>* __restrict__ B, const MemT<V>* __restrict__ tx,
-                  const MemT<V>* __restrict__ ty, const typename STable<V>::type* __restrict__ s,
+    row_t1_kernel(const V* __restrict__ A, V* __restrict__ B, const V* __restrict__ tx,
+                  const V* __restrict__ ty, const typename STable<V>::type* __restrict__ s,
                   const V* __restrict__ tw, RowArgs a) {
     using Cf = RowCfg<V, LOGNP, 1>;
     constexpr int NP = Cf::NP, ROWS = Cf::ROWS, HALF = NP / 2;
@@ -340,15 +341,14 @@ __global__ void __launch_bounds__(RowCfg<V, LOGNP, 1>::P, RowCfg<V, LOGNP, 1>::M
     pdl_allow_next();
     const RowConst<V> rc0 = row_const<V>(r0, ty, s, a);
     pdl_wait();   // A comes from the previous kernel
-    const int sc = cta_scale<V>(A, r0, ROWS, W, Wp);
 
     constexpr int R0 = Cf::MERGE ? Cf::EM : Cf::EF;   // first-pass radix of the forward engines
     [[maybe_unused]] const int a_n = a.np * Wp;   // extent of A (N' x Wp)
     auto folded = [&](int row, int p, int sgn) -> V {
-        const MemT<V>* x = A + (r0 + row) * Wp;
-        const V u = p < W && NUASM_IN_RANGE((r0 + row) * Wp + p, a_n, dbg::kRowLoad) ? Mem<V>::ld(x[p], sc) : zero;
+        const V* x = A + (r0 + row) * Wp;
+        const V u = p < W && NUASM_IN_RANGE((r0 + row) * Wp + p, a_n, dbg::kRowLoad) ? x[p] : zero;
         const V t = p + NP < W && NUASM_IN_RANGE((r0 + row) * Wp + p + NP, a_n, dbg::kRowLoad)
-                        ? Mem<V>::ld(x[p + NP], sc) : zero;
+                        ? x[p + NP] : zero;
         return sgn == 0 ? cadd(u, t) : cmul(csub(u, t), half_bin<V, -1, LOGNP, R0>(tw, p));
     };
     // both halves of the fold at p (pairs)
@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(RowCfg<V, LOGNP, 1>::P, RowCfg<V, LOGNP, 1>::M
         S, tw, [&](int p, int c) { return NUASM_IN_RANGE(c * NP + p, ROWS * NP, dbg::kRowModes) ? M[c * NP + p] : zero; },
         [&](int p, int c, V v) {
             if (p < n && NUASM_IN_RANGE((r0 + c) * n + p, a.np * n, dbg::kRowStore))
-                B[(r0 + c) * n + p] = Mem<V>::st(v, sc);
+                B[(r0 + c) * n + p] = v;
         });
 }
 
@@ -402,8 +402,8 @@ __global__ void __launch_bounds__(RowCfg<V, LOGNP, 1>::P, RowCfg<V, LOGNP, 1>::M
 // (even and odd outputs as two N'-point FFTs), keeping the W window entries.
 template <typename V, int LOGNP>
 __global__ void __launch_bounds__(RowCfg<V, LOGNP, 2>::P, RowCfg<V, LOGNP, 2>::MINB)
-    row_t2_kernel(const MemT<V>* __restrict__ B, MemT<V>* __restrict__ A, const MemT<V>* __restrict__ tx,
-                  const MemT<V>* __restrict__ ty, const typename STable<V>::type* __restrict__ s,
+    row_t2_kernel(const V* __restrict__ B, V* __restrict__ A, const V* __restrict__ tx,
+                  const V* __restrict__ ty, const typename STable<V>::type* __restrict__ s,
                   const V* __restrict__ tw, RowArgs a) {
     using Cf = RowCfg<V, LOGNP, 2>;
     constexpr int NP = Cf::NP, ROWS = Cf::ROWS, HALF = NP / 2;
@@ -440,21 +440,36 @@ __global__ void __launch_bounds__(RowCfg<V, LOGNP, 2>::P, RowCfg<V, LOGNP, 2>::M
         if (staged) cp_async_commit();
     }
     pdl_wait();   // B comes from the previous kernel
-    const int sc = cta_scale<V>(B, r0, ROWS, n, n);
+    // double-float: B's strips of columns have a scale each; the solve's is their maximum
+    [[maybe_unused]] int top = 0;
+    if constexpr (Ext<V>::scaled) {
+        constexpr int C = ColCfg<V, LOGNP, 2>::C;   // columns of a strip: a CTA of the forward column pass
+        static_assert(NP / 2 / C < kExpoWords, "one word a strip");
+        int e = -2000;
+        for (int i = threadIdx.x; i < n / C; i += Cf::P) e = max(e, __ldg(a.expo + 1 + i));
+        top = block_max(e);
+        if (blockIdx.x == 0 && threadIdx.x == 0) a.expo[0] = top;
+    }
     block_fft<V, -1, Cf::EF, LOGNP, Cf::LOGROWS, true>(
         S, tw,
         [&](int p, int c) {
-            return p < n && NUASM_IN_RANGE((r0 + c) * n + p, a.np * n, dbg::kRowLoad)
-                       ? Mem<V>::ld(B[(r0 + c) * n + p], sc) : zero;
+            if (!(p < n && NUASM_IN_RANGE((r0 + c) * n + p, a.np * n, dbg::kRowLoad))) return zero;
+            V v = B[(r0 + c) * n + p];
+            if constexpr (Ext<V>::scaled) {
+                const int d = __ldg(a.expo + 1 + p / ColCfg<V, LOGNP, 2>::C) - top;
+                const float2 f = f2_dup(d < -126 ? 0.f : __uint_as_float(unsigned(d + 127) << 23));
+                v = dfc{mul2(v.h, f), mul2(v.l, f)};
+            }
+            return v;
         },
         [&](int p, int c, V v) {
             V f;
-            const V t = ROWS == 1 ? rc0.ty : Mem<V>::ld(__ldg(&ty[r0 + c]), 0);
+            const V t = ROWS == 1 ? rc0.ty : ldgv(&ty[r0 + c]);
             if (staged == 2) {
                 f = cmul(Es[c * NP + p], t);
             } else if (staged == 1) {
-                const MemT<V>* Em = reinterpret_cast<const MemT<V>*>(Es);
-                f = cmul(cmul(Mem<V>::ld(__ldg(&tx[p]), 0), t), Mem<V>::ld(Em[c * a.ep + min(p, NP - p)], 0));
+                const V* Em = reinterpret_cast<const V*>(Es);
+                f = cmul(cmul(ldgv(&tx[p]), t), Em[c * a.ep + min(p, NP - p)]);
             } else {
                 f = row_factor<V, ROWS>(p, c, r0, rc0, tx, ty, s, a);
             }
@@ -476,7 +491,7 @@ __global__ void __launch_bounds__(RowCfg<V, LOGNP, 2>::P, RowCfg<V, LOGNP, 2>::M
     auto put = [&](int row, int k, int sgn, V v) {
         const int u = 2 * k + sgn;
         if (u < W && NUASM_IN_RANGE((r0 + row) * Wp + u, a.np * Wp, dbg::kRowStore))
-            A[(r0 + row) * Wp + u] = Mem<V>::st(v, sc);
+            A[(r0 + row) * Wp + u] = v;
     };
     if constexpr (Cf::PAIR) {
         block_fft<fp2, +1, Cf::EM, LOGNP, Cf::LOGROWS, true, true>(
@@ -506,7 +521,7 @@ __global__ void __launch_bounds__(RowCfg<V, LOGNP, 2>::P, RowCfg<V, LOGNP, 2>::M
 // reads happen in the first forward pass, before any write).
 template <typename V, int LOGNP>
 __global__ void __launch_bounds__(RowCfg<V, LOGNP, 3>::P, RowCfg<V, LOGNP, 3>::MINB)
-    row_t3_kernel(MemT<V>* __restrict__ A, const MemT<V>* __restrict__ tx, const MemT<V>* __restrict__ ty,
+    row_t3_kernel(V* __restrict__ A, const V* __restrict__ tx, const V* __restrict__ ty,
                   const typename STable<V>::type* __restrict__ s, const V* __restrict__ tw, RowArgs a) {
     using Cf = RowCfg<V, LOGNP, 3>;
     constexpr int NP = Cf::NP, ROWS = Cf::ROWS, HALF = NP / 2;
@@ -519,14 +534,13 @@ __global__ void __launch_bounds__(RowCfg<V, LOGNP, 3>::P, RowCfg<V, LOGNP, 3>::M
     pdl_allow_next();
     const RowConst<V> rc0 = row_const<V>(r0, ty, s, a);
     pdl_wait();   // A comes from the previous kernel
-    const int sc = cta_scale<V>(A, r0, ROWS, W, Wp);
     constexpr int R0 = Cf::MERGE ? Cf::EM : Cf::EF;   // first-pass radix of the engines
     [[maybe_unused]] const int a_n = a.np * Wp;   // extent of A (N' x Wp)
     auto folded = [&](int row, int p, int sgn) -> V {
-        const MemT<V>* x = A + (r0 + row) * Wp;
-        const V u = p < W && NUASM_IN_RANGE((r0 + row) * Wp + p, a_n, dbg::kRowLoad) ? Mem<V>::ld(x[p], sc) : zero;
+        const V* x = A + (r0 + row) * Wp;
+        const V u = p < W && NUASM_IN_RANGE((r0 + row) * Wp + p, a_n, dbg::kRowLoad) ? x[p] : zero;
         const V t = p + NP < W && NUASM_IN_RANGE((r0 + row) * Wp + p + NP, a_n, dbg::kRowLoad)
-                        ? Mem<V>::ld(x[p + NP], sc) : zero;
+                        ? x[p + NP] : zero;
         return sgn == 0 ? cadd(u, t) : cmul(csub(u, t), half_bin<V, -1, LOGNP, R0>(tw, p));
     };
     // both halves of the fold at p (pairs)
@@ -555,7 +569,7 @@ __global__ void __launch_bounds__(RowCfg<V, LOGNP, 3>::P, RowCfg<V, LOGNP, 3>::M
     auto put_row = [&](int row, int k, int sgn, V v) {
         const int u = 2 * k + sgn;
         if (u < W && NUASM_IN_RANGE((r0 + row) * Wp + u, a_n, dbg::kRowStore))
-            A[(r0 + row) * Wp + u] = Mem<V>::st(v, sc);
+            A[(r0 + row) * Wp + u] = v;
     };
     if constexpr (Cf::PAIR) {
         block_fft<fp2, -1, Cf::EM, LOGNP, Cf::LOGROWS, true>(
@@ -598,11 +612,18 @@ __global__ void __launch_bounds__(RowCfg<V, LOGNP, 3>::P, RowCfg<V, LOGNP, 3>::M
 // --------------------------------------------------------------- column passes
 enum ColMode { COL_FWD_FOLD = 0, COL_INV = 1, COL_FWD = 2, COL_INV_FOLD = 3 };
 
+// the forward modes read and the inverse modes write outside the mode side
+template <typename V, int MODE>
+using ColSrcT = std::conditional_t<MODE == COL_FWD_FOLD || MODE == COL_FWD, ExtT<V>, V>;
+template <typename V, int MODE>
+using ColDstT = std::conditional_t<MODE == COL_FWD_FOLD || MODE == COL_FWD, V, ExtT<V>>;
+
 // One CTA = C adjacent columns (blockIdx.x) and, for the folded modes, one
 // half (blockIdx.y: 0 even, 1 odd).
 template <typename V, int LOGNP, int MODE>
 __global__ void __launch_bounds__(ColCfg<V, LOGNP, MODE>::P, ColCfg<V, LOGNP, MODE>::MINB)
-    col_kernel(const MemT<V>* __restrict__ src, MemT<V>* __restrict__ dst, const V* __restrict__ tw, ColArgs a) {
+    col_kernel(const ColSrcT<V, MODE>* __restrict__ src, ColDstT<V, MODE>* __restrict__ dst, const V* __restrict__ tw,
+               ColArgs a) {
     using Cf = ColCfg<V, LOGNP, MODE>;
     constexpr int NP = Cf::NP, HALF = NP / 2, C = Cf::C;
     extern __shared__ unsigned char smem_raw[];
@@ -618,17 +639,36 @@ __global__ void __launch_bounds__(ColCfg<V, LOGNP, MODE>::P, ColCfg<V, LOGNP, MO
                                      : MODE == COL_FWD ? NP * n : W * Wp;
     pdl_allow_next();
     pdl_wait();   // src comes from the previous kernel (no-op for the first kernel of a chain)
-    // double-float passes: the CTA's scale over the source rows and columns it reads
+    constexpr bool FORWARD = MODE == COL_FWD_FOLD || MODE == COL_FWD;
+    // the scale: the solve's (and what the tables left out), or, in the forward
+    // pass of type 2, which is a solve's first look at its data, the strip's own:
+    // the largest exponent among the values, which wait in registers (butterfly
+    // inputs j + r N'/E of column c) for the CTA's maximum
     int sc = 0;
-    if constexpr (Mem<V>::scaled) {
-        const bool win_cols = MODE == COL_FWD_FOLD || MODE == COL_INV_FOLD;   // window-wide arrays
-        const int cols = win_cols ? W : n, pitch = win_cols ? Wp : n;
-        const int rows = MODE == COL_FWD_FOLD ? W : MODE == COL_FWD ? n : NP;
-        sc = cta_scale<V>(src + col0, 0, rows, min(C, cols - col0), pitch);
+    [[maybe_unused]] ExtT<V> raw[MODE == COL_FWD && Ext<V>::scaled ? Cf::E : 1];
+    if constexpr (MODE == COL_FWD && Ext<V>::scaled) {
+        const int c = threadIdx.x & (C - 1), j = threadIdx.x >> Cf::LOGC;
+        int e = -2000;
+#pragma unroll
+        for (int r = 0; r < Cf::E; ++r) {
+            const int p = j + r * (NP / Cf::E), i = p * n + col0 + c;
+            raw[r] = p < n && NUASM_IN_RANGE(i, src_n, dbg::kColLoad) ? src[i] : make_double2(0.0, 0.0);
+            e = max(e, max(dexp2(raw[r].x), dexp2(raw[r].y)));
+        }
+        sc = clamp_expo(block_max(e));
+        if (threadIdx.x == 0) a.expo[1 + blockIdx.x] = sc;
+    } else {
+        sc = solve_scale<V>(a.expo) + (FORWARD ? 0 : a.texp);
     }
-    auto ld = [&](int i) -> V { return NUASM_IN_RANGE(i, src_n, dbg::kColLoad) ? Mem<V>::ld(src[i], sc) : zero; };
+    auto ld = [&](int i) -> V {
+        if (!NUASM_IN_RANGE(i, src_n, dbg::kColLoad)) return zero;
+        if constexpr (FORWARD) return Ext<V>::ld(src[i], sc);
+        else return src[i];
+    };
     auto st = [&](int i, V v) {
-        if (NUASM_IN_RANGE(i, dst_n, dbg::kColStore)) dst[i] = Mem<V>::st(v, sc);
+        if (!NUASM_IN_RANGE(i, dst_n, dbg::kColStore)) return;
+        if constexpr (FORWARD) dst[i] = v;
+        else dst[i] = Ext<V>::st(v, sc);
     };
     if constexpr (MODE == COL_FWD_FOLD) {
         // src: window (W x Wp); dst: A (N' x Wp), kept modes in natural N'-bin rows
@@ -657,7 +697,11 @@ __global__ void __launch_bounds__(ColCfg<V, LOGNP, MODE>::P, ColCfg<V, LOGNP, MO
     } else if constexpr (MODE == COL_FWD) {
         // src: u1 (N x N); dst: B (N' x N)
         block_fft<V, -1, Cf::E, LOGNP, Cf::LOGC, false>(
-            S, tw, [&](int p, int c) { return p < n ? ld(p * n + col0 + c) : zero; },
+            S, tw,
+            [&](int p, int c) {
+                if constexpr (Ext<V>::scaled) return Ext<V>::ld(raw[p / (NP / Cf::E)], sc);
+                else return p < n ? ld(p * n + col0 + c) : zero;
+            },
             [&](int p, int c, V v) { st(p * n + col0 + c, v); });
     } else {
         // src: A (N' x Wp); dst: window (W x Wp)
@@ -1074,6 +1118,7 @@ inline RowArgs row_args(const nuasm_plan_s* P) {
     a.etab2 = P->d.etab2;
     a.ep = P->etab_pitch;
     a.np = P->g.np;
+    a.expo = expo_words(P);
     return a;
 }
 
@@ -1083,10 +1128,10 @@ cudaError_t launch_row(const nuasm_plan_s* P, int type, cudaStream_t st) {
     using C2 = RowCfg<V, LOGNP, 2>;
     using C3 = RowCfg<V, LOGNP, 3>;
     using ST = typename STable<V>::type;
-    using M = MemT<V>;
+    using M = V;
     const RowArgs a = row_args(P);
     // double-float passes read the plan's twiddles as float pairs
-    const V* tw = static_cast<const V*>(Mem<V>::scaled ? P->d.tw_df : P->d.tw);
+    const V* tw = static_cast<const V*>(Ext<V>::scaled ? P->d.tw_df : P->d.tw);
     if (!tw) return cudaErrorInvalidValue;
     const ST* s = static_cast<const ST*>(P->d.s);
     cudaError_t e;
@@ -1109,23 +1154,28 @@ cudaError_t launch_row(const nuasm_plan_s* P, int type, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+inline ColArgs col_args(const nuasm_plan_s* P, int mode) {
+    return ColArgs{P->g.n, P->g.W, P->g.Wp, expo_words(P), mode == COL_INV ? P->texp[0] : P->texp[1]};
+}
+
 template <typename V, int LOGNP, int MODE>
 cudaError_t launch_col(const nuasm_plan_s* P, const void* src, void* dst, int ncols, int halves, cudaStream_t st) {
     using Cf = ColCfg<V, LOGNP, MODE>;
-    const ColArgs a{P->g.n, P->g.W, P->g.Wp};
+    const ColArgs a = col_args(P, MODE);
     const size_t sm = Cf::smem();
     cudaError_t e = set_smem(col_kernel<V, LOGNP, MODE>, sm);
     if (e != cudaSuccess) return e;
     dim3 grid((ncols + Cf::C - 1) / Cf::C, halves);
-    using M = MemT<V>;
+    using MS = ColSrcT<V, MODE>;
+    using MD = ColDstT<V, MODE>;
     // double-float passes read the plan's twiddles as float pairs
-    const V* tw = static_cast<const V*>(Mem<V>::scaled ? P->d.tw_df : P->d.tw);
+    const V* tw = static_cast<const V*>(Ext<V>::scaled ? P->d.tw_df : P->d.tw);
     if (!tw) return cudaErrorInvalidValue;
     if constexpr (MODE == COL_FWD) {   // first kernel of the type-2 chain
-        col_kernel<V, LOGNP, MODE><<<grid, Cf::P, sm, st>>>(static_cast<const M*>(src), static_cast<M*>(dst), tw, a);
+        col_kernel<V, LOGNP, MODE><<<grid, Cf::P, sm, st>>>(static_cast<const MS*>(src), static_cast<MD*>(dst), tw, a);
     } else {
-        e = launch_chained(col_kernel<V, LOGNP, MODE>, grid, dim3(Cf::P), sm, st, static_cast<const M*>(src),
-                           static_cast<M*>(dst), tw, a);
+        e = launch_chained(col_kernel<V, LOGNP, MODE>, grid, dim3(Cf::P), sm, st, static_cast<const MS*>(src),
+                           static_cast<MD*>(dst), tw, a);
         if (e != cudaSuccess) return e;
     }
     return cudaGetLastError();
@@ -1138,7 +1188,7 @@ cudaError_t launch_col2(const nuasm_plan_s* P, const void* src, void* dst, int n
     using Cf = Col2Cfg<LOGNP>;
     if (((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) || (ncols & 1))
         return cudaErrorNotSupported;
-    const ColArgs a{P->g.n, P->g.W, P->g.Wp};
+    const ColArgs a = col_args(P, MODE);
     cudaError_t e = set_smem(col2_kernel<LOGNP, MODE>, Cf::SMEM);
     if (e != cudaSuccess) return e;
     const dim3 grid(ncols / 2), block(Cf::P);
@@ -1213,7 +1263,7 @@ cudaError_t launch_col_tma(const nuasm_plan_s* P, const void* src, void* dst, in
             nitems = nfull + (tail + hc - 1) / hc;
             if ((hc & 1) || ((nfull * Cf::C) & 1)) return cudaErrorNotSupported;   // an odd TMA x: never issued
         }
-        const ColArgs a{P->g.n, P->g.W, P->g.Wp};
+        const ColArgs a = col_args(P, MODE);
         if constexpr (MODE == COL_FWD) {   // first kernel of the type-2 chain
             col_tma_kernel<LOGNP, MODE><<<grid, Cf::P, sm, st>>>(map, omap, omap_h, static_cast<float2*>(dst),
                                                                  static_cast<const float2*>(P->d.tw), a, nfull,

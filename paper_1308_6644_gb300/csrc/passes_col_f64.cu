@@ -1,17 +1,11 @@
 // Column-pass instantiations of FP64 plans for every supported N': from
 // N' = 512 up in double-float arithmetic (dfc, on the FP32 pipe) over the
 // plan's FP64 arrays, below in FP64 (double2), as the row passes.
-// NUASM_F64_DF_COLS=0 keeps FP64 throughout.
 #include "passes.cuh"
-
-#ifndef NUASM_F64_DF_COLS
-#define NUASM_F64_DF_COLS 1
-#endif
 
 namespace nuasm {
 
 cudaError_t col_f64(const nuasm_plan_s* P, int mode, const void* ext, cudaStream_t s) {
-    using R = std::conditional_t<NUASM_F64_DF_COLS != 0, dfc, double2>;
     auto run = [&](auto st) -> cudaError_t {
         using S = decltype(st);
         switch (mode) {
@@ -26,10 +20,10 @@ cudaError_t col_f64(const nuasm_plan_s* P, int mode, const void* ext, cudaStream
         case 6: return run(passes::Stages<double2, 6>{});
         case 7: return run(passes::Stages<double2, 7>{});
         case 8: return run(passes::Stages<double2, 8>{});
-        case 9: return run(passes::Stages<R, 9>{});
-        case 10: return run(passes::Stages<R, 10>{});
-        case 11: return run(passes::Stages<R, 11>{});
-        case 12: return run(passes::Stages<R, 12>{});
+        case 9: return run(passes::Stages<dfc, 9>{});
+        case 10: return run(passes::Stages<dfc, 10>{});
+        case 11: return run(passes::Stages<dfc, 11>{});
+        case 12: return run(passes::Stages<dfc, 12>{});
         default: return cudaErrorInvalidValue;
     }
 }

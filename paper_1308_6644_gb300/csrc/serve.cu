@@ -287,7 +287,8 @@ nuasm_status run_job(Server& S, Slot& sl, const Job& j, PointSet* ps, bool build
         }
         sl.h_tab_bytes = tb;
     }
-    pack_tables(ht, g, f64, false, sl.h_tab);
+    int texp[3];
+    pack_tables(ht, g, f64, false, sl.h_tab, texp);
     const double rc = ht.rc, rmax = ht.rmax;
     free_tables(&ht);
 
@@ -315,6 +316,7 @@ nuasm_status run_job(Server& S, Slot& sl, const Job& j, PointSet* ps, bool build
     view.g = g;
     view.rc = rc;
     view.nonsep_mode = choose_nonsep_mode(j.rp, rmax);
+    std::copy(texp, texp + 3, view.texp);
     view.d.tables = part[0];
     view.d.t1x = part[0];
     view.d.t1y = part[0] + np * eb;
