@@ -148,8 +148,8 @@ template <int DIR, typename V> __device__ __forceinline__ V cis_pi16(int k) {
 // every input of a butterfly and r a compile-time constant of the unrolled
 // loop, so the factor is tw[j] (or its conjugate; tw[t] = exp(-i pi t / L))
 // times the constant exp(DIR i pi r / R0): one table load per butterfly
-// instead of one per input (FP32; on the FP64 pipe the extra complex product
-// costs more than the loads it saves, so FP64 reads tw[q] itself).
+// instead of one per input (FP32; in double-float the extra complex product
+// costs more than the loads it saves, so it reads tw[q] itself).
 template <typename V, int DIR, int LOGL, int E>
 __device__ __forceinline__ V half_bin(const V* __restrict__ tw, int q) {
     if constexpr (sizeof(V) == 16) {
@@ -167,7 +167,7 @@ __device__ __forceinline__ V half_bin(const V* __restrict__ tw, int q) {
 }
 
 // ---------------------------------------------------------------- twiddle powers
-// w[r] = exp(-2 pi i k r / (Ns R)) for r in [1, R).  FP64 reads every power;
+// w[r] = exp(-2 pi i k r / (Ns R)) for r in [1, R).  Double-float reads every power;
 // FP32 reads w^1 and w^4 (w^1 and w^2 for R = 4) and forms the others by
 // complex products (at most four roundings, about 2.4e-7 relative), which
 // trades table loads for FMA-pipe work.  The reads come from the pass's own

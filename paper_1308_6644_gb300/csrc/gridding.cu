@@ -1417,9 +1417,9 @@ template <typename K> cudaError_t set_smem(K kernel, size_t bytes) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
 }
 
-// the solve's exponent word where its FFT passes are double-float (null elsewhere), below every exponent
+// the exponent word of a solve with double-float passes (null elsewhere), below every exponent
 cudaError_t clear_expo(const nuasm_plan_s* P, int** expo, cudaStream_t st) {
-    if (!fft_double_float(P->f64, P->g.np)) return cudaSuccess;
+    if (!fft_double_float(P)) return cudaSuccess;
     *expo = expo_words(P);
     return cudaMemsetAsync(*expo, 0x80, sizeof(int), st);
 }

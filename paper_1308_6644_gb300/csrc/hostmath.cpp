@@ -460,7 +460,8 @@ void pack_twp(const double* tw, int logl, bool f64, void* dst) {
 
 // Device image of the tables: T1x T1y T2x T2y T3x T3y (complex, plan precision),
 // s (double, or float hi/lo pairs), then the twiddles when present.
-void pack_tables(const HostTables& t, const Geometry& g, bool f64, bool with_twiddles, void* dst, int texp[3]) {
+void pack_tables(const HostTables& t, const Geometry& g, bool f64, bool df, bool with_twiddles, void* dst,
+                 int texp[3]) {
     const int np = g.np;
     const size_t eb = f64 ? 16 : 8;
     char* out = static_cast<char*>(dst);
@@ -473,7 +474,7 @@ void pack_tables(const HostTables& t, const Geometry& g, bool f64, bool with_twi
     };
     const double* six[6] = {t.t1x, t.t1y, t.t2x, t.t2y, t.t3x, t.t3y};
     texp[0] = texp[1] = texp[2] = 0;
-    if (fft_double_float(f64, np)) {
+    if (df) {
         int ex[6] = {};
         for (int i = 0; i < 6; ++i) {
             double top = 0.0;
@@ -511,6 +512,19 @@ void pack_tables(const HostTables& t, const Geometry& g, bool f64, bool with_twi
         const size_t toff = soff + size_t(np) * (f64 ? sizeof(double) : 2 * sizeof(float));
         put_c(toff, t.tw, g.G);
         pack_twp(t.tw, log2_of(np), f64, out + toff + size_t(g.G) * eb);
+        if (df) {   // both hi parts of an entry, then both lo, in its 16 bytes
+            const size_t count = size_t(g.G) + size_t(twp_entries(true, log2_of(np)));
+            for (size_t i = 0; i < count; ++i) {
+                double v[2];
+                float d[4];
+                std::memcpy(v, out + toff + 16 * i, sizeof(v));
+                for (int k = 0; k < 2; ++k) {
+                    d[k] = float(v[k]);
+                    d[2 + k] = float(v[k] - double(d[k]));
+                }
+                std::memcpy(out + toff + 16 * i, d, sizeof(d));
+            }
+        }
     }
 }
 

@@ -69,9 +69,7 @@ struct PlanDevice {
     void* t1x = nullptr; void* t1y = nullptr; void* t2x = nullptr; void* t2y = nullptr;
     void* t3x = nullptr; void* t3y = nullptr;
     void* s = nullptr;          // float2 (hi, lo) per bin (F32) or double (F64)
-    void* tw = nullptr;         // twiddles, G complex
-    void* tw_df = nullptr;      // F64 plans: the twiddles as float pairs (re.hi, im.hi, re.lo, im.lo), for
-                                // the double-float row passes
+    void* tw = nullptr;         // twiddles, G complex and the pass twiddles (float pairs, dfc, where fft_double_float)
     void* etab = nullptr;       // ASM non-separable factor E(|kx|, |ky|): N'/2 + 1 rows of etab_pitch
                                 // entries in the plan precision (null: evaluated per mode)
     void* etab2 = nullptr;      // type 2's T2x(kx) E(|kx|, |ky|): N'/2 + 1 rows of N' entries (FP32 plans
@@ -172,11 +170,12 @@ void build_tables(const nuasm_params_t& p, const Geometry& g, HostTables* t, con
 void phihat_table(const Geometry& g, double* out);
 void free_tables(HostTables* t);
 size_t table_bytes(const Geometry& g, bool f64, bool with_twiddles);
-// Double-float plans (fft_double_float) get the six factor tables as pairs of
-// floats (re.hi, im.hi, re.lo, im.lo), each scaled by a power of two to a
-// largest component in [1, 2) (type 3's by type 2's powers); texp[t - 1] receives
-// the sum of type t's two exponents.
-void pack_tables(const HostTables& t, const Geometry& g, bool f64, bool with_twiddles, void* dst, int texp[3]);
+// With df (fft_double_float) the twiddles and the six factor tables are pairs of
+// floats (re.hi, im.hi, re.lo, im.lo), each factor table scaled by a power of two
+// to a largest component in [1, 2) (type 3's by type 2's powers); texp[t - 1]
+// receives the sum of type t's two exponents.
+void pack_tables(const HostTables& t, const Geometry& g, bool f64, bool df, bool with_twiddles, void* dst,
+                 int texp[3]);
 
 // Pass twiddles.  The full twiddle table tw[t] = exp(-2 pi i t / 2N'),
 // t < 2N', is followed by the twiddle bases of every pass I >= 1 of the
@@ -233,11 +232,13 @@ inline size_t ws_bufA_elems(const Geometry& g) { return size_t(g.np) * g.Wp; }
 // (bufB ends with the exponents of expo_words)
 constexpr int kExpoWords = 2080;
 inline size_t ws_bufB_elems(const Geometry& g) { return size_t(g.np) * g.n + kExpoWords * sizeof(int) / 8; }
-// FP64 plans from N' = 512 up run their FFT passes in double-float arithmetic
-// (passes.cuh): the mode-side arrays bufA and bufB and the transfer-function
-// tables then hold pairs of floats (dfc), the window and the caller's arrays FP64
-constexpr int kDfMinNp = 512;
-inline bool fft_double_float(bool f64, int np) { return f64 && np >= kDfMinNp; }
+// FP64 plans run their FFT passes in double-float arithmetic (passes.cuh): the
+// mode-side arrays bufA and bufB, the transfer-function tables and the twiddles
+// hold pairs of floats (dfc), the window and the caller's arrays FP64.  Its
+// error, about 2e-14, hides behind the gridding's at tolerances down to 1e-12;
+// plans below N' = 512 with a smaller one keep FP64 passes.
+inline bool fft_double_float(bool f64, int np, double tol) { return f64 && (np >= 512 || tol >= 1e-12); }
+inline bool fft_double_float(const nuasm_plan_s* P) { return fft_double_float(P->f64, P->g.np, P->p.tol); }
 // The exponents of a solve's double-float data, behind bufB's elements: word 0
 // the solve's (types 1 and 3: set by the spreading; type 2: by the row pass),
 // then type 2's one per strip of columns of the forward column pass.

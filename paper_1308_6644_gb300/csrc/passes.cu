@@ -146,7 +146,7 @@ cudaError_t build_etab(const nuasm_plan_s* P, cudaStream_t s) {
     const double k = P->p.lambda / (double(P->g.np) * P->p.pitch);
     const int threads = 256;
     const int blocks = int(std::min<size_t>((n + threads - 1) / threads, size_t(152) * 8));
-    if (fft_double_float(P->f64, P->g.np))
+    if (fft_double_float(P))
         etab_kernel<<<blocks, threads, 0, s>>>(static_cast<dfc*>(P->d.etab), P->g.np / 2, pitch, k * k, P->rc);
     else if (P->f64)
         etab_kernel<<<blocks, threads, 0, s>>>(static_cast<double2*>(P->d.etab), P->g.np / 2, pitch, k * k, P->rc);

@@ -52,16 +52,21 @@ template <typename V> struct Prec;
 #ifndef NUASM_COL_BUDGET
 #define NUASM_COL_BUDGET 8192   // FP32 column passes: complex elements per CTA (columns = budget / N')
 #endif
-// FP64 passes run at the FP64 pipe's pace, so small planes want many CTAs:
-// measured on the N' = 128 plane (C1), 2^9 elements per row-pass CTA and 512
-// per column-pass CTA against 2^11 and 4096: row_t1 57 -> 33 us, the column
-// passes 24 -> 16 and 17 -> 11 us (N' = 512: 440 -> 412 us per solve); the
-// same configuration as before at N' = 4096
-#ifndef NUASM_COL_BUDGET64
-#define NUASM_COL_BUDGET64 512    // FP64 column passes: complex elements per CTA
-#endif
+// Double-float passes of FP64 plans: up to 2^NUASM_ROW_LOGBUDGET64 elements per
+// row CTA (N' = 128: 17.0 us with 2^8, 18.6 with 2^9), and column CTAs of up to
+// NUASM_DF_COL_BUDGET elements and 2 columns below N' = 2048, 4 there
+// (col_fwd_fold with 4 and with 2: N' = 512 16.8 / 16.6, N' = 1024 51.8 / 45.1, N' =
+// 2048 158 / 211 us; the budget leaves 2 at N' = 4096).  In FP64 arithmetic,
+// which takes 64 cycles a warp instruction, a 64 x 64 plane's row_t1 took 30.9
+// us and type 1 75.8 us against 17.0 and 56 us.
 #ifndef NUASM_ROW_LOGBUDGET64
-#define NUASM_ROW_LOGBUDGET64 9   // FP64 row passes: log2 of the complex elements per CTA
+#define NUASM_ROW_LOGBUDGET64 8
+#endif
+#ifndef NUASM_DF_COL_E
+#define NUASM_DF_COL_E 8
+#endif
+#ifndef NUASM_DF_COL_BUDGET
+#define NUASM_DF_COL_BUDGET 8192
 #endif
 template <> struct Prec<float2> {
     static constexpr bool f64 = false;
@@ -71,28 +76,20 @@ template <> struct Prec<float2> {
     static constexpr int regs = 64;
     static constexpr int row_regs = NUASM_ROW_REGS;
 };
+// FP64 passes (N' <= 256, tolerances below 1e-12), bound by the FP64 pipe: many small CTAs
 template <> struct Prec<double2> {
     static constexpr bool f64 = true;
-    static constexpr int col_e = 8, col_budget = NUASM_COL_BUDGET64, col_cmax = 16;
-    static constexpr int row_logbudget = NUASM_ROW_LOGBUDGET64;
+    static constexpr int col_e = 8, col_budget = 512, col_cmax = 16;
+    static constexpr int row_logbudget = 9;
     static constexpr int regs = 128;
     static constexpr int row_regs = 128;
 };
-
-// double-float passes of FP64 plans: the FP64 row configuration (16-byte
-// elements, as complex128); column CTAs of up to NUASM_DF_COL_BUDGET elements
-// and NUASM_DF_COL_CMAX columns, NUASM_DF_COL_E elements per thread
-#ifndef NUASM_DF_COL_E
-#define NUASM_DF_COL_E 8
-#endif
-#ifndef NUASM_DF_COL_BUDGET
-#define NUASM_DF_COL_BUDGET 8192
-#endif
-#ifndef NUASM_DF_COL_CMAX
-#define NUASM_DF_COL_CMAX 4
-#endif
-template <> struct Prec<dfc> : Prec<double2> {
-    static constexpr int col_e = NUASM_DF_COL_E, col_budget = NUASM_DF_COL_BUDGET, col_cmax = NUASM_DF_COL_CMAX;
+template <> struct Prec<dfc> {
+    static constexpr bool f64 = true;
+    static constexpr int col_e = NUASM_DF_COL_E, col_budget = NUASM_DF_COL_BUDGET, col_cmax = 4;
+    static constexpr int row_logbudget = NUASM_ROW_LOGBUDGET64;
+    static constexpr int regs = 128;
+    static constexpr int row_regs = 128;
 };
 
 #ifndef NUASM_ROW_PAIR_MIN
@@ -119,6 +116,7 @@ template <typename V, int LOGNP, int TYPE> struct RowCfg {
     static constexpr int EF = PAIR ? 16 : 8;   // single-sequence engines
     static constexpr int EM = 16;              // merged engines
     static constexpr int P = (NP * ROWS) / EF;
+    static_assert(!std::is_same<V, dfc>::value || P % 32 == 0, "block_max works on whole warps");
     static constexpr int REGS = PAIR ? 128 : Prec<V>::row_regs;
     static constexpr int MINB = (65536 / (P * REGS)) > 0 ? 65536 / (P * REGS) : 1;
     static constexpr int SEQ = MERGE ? 2 * ROWS : ROWS;                  // sequences in the work buffer
@@ -141,9 +139,12 @@ template <typename V, int LOGNP, int MODE = 0> struct ColCfg {
     static constexpr int E = Prec<V>::col_e;
     static constexpr int BUDGET = (MODE == 2 && !Prec<V>::f64) ? NUASM_COL_FWD_BUDGET : Prec<V>::col_budget;
     static constexpr int CRAW = BUDGET / NP;
-    static constexpr int C = CRAW > Prec<V>::col_cmax ? Prec<V>::col_cmax : (CRAW < 1 ? 1 : CRAW);
+    // (double-float: a whole warp at least)
+    static constexpr int CMAX = std::is_same<V, dfc>::value && LOGNP < 11 ? (NP >= 128 ? 2 : 256 / NP) : Prec<V>::col_cmax;
+    static constexpr int C = CRAW > CMAX ? CMAX : (CRAW < 1 ? 1 : CRAW);
     static constexpr int LOGC = Log2<C>::v;
     static constexpr int P = (NP * C) / E;
+    static_assert(!std::is_same<V, dfc>::value || P % 32 == 0, "block_max works on whole warps");
     static constexpr int MINB = (65536 / (P * Prec<V>::regs)) > 0 ? 65536 / (P * Prec<V>::regs) : 1;
     static size_t smem() { return size_t(spad_size<V>(NP * C)) * sizeof(V); }
 };
@@ -1130,9 +1131,7 @@ cudaError_t launch_row(const nuasm_plan_s* P, int type, cudaStream_t st) {
     using ST = typename STable<V>::type;
     using M = V;
     const RowArgs a = row_args(P);
-    // double-float passes read the plan's twiddles as float pairs
-    const V* tw = static_cast<const V*>(Ext<V>::scaled ? P->d.tw_df : P->d.tw);
-    if (!tw) return cudaErrorInvalidValue;
+    const V* tw = static_cast<const V*>(P->d.tw);
     const ST* s = static_cast<const ST*>(P->d.s);
     cudaError_t e;
     if (type == 1) {
@@ -1168,9 +1167,7 @@ cudaError_t launch_col(const nuasm_plan_s* P, const void* src, void* dst, int nc
     dim3 grid((ncols + Cf::C - 1) / Cf::C, halves);
     using MS = ColSrcT<V, MODE>;
     using MD = ColDstT<V, MODE>;
-    // double-float passes read the plan's twiddles as float pairs
-    const V* tw = static_cast<const V*>(Ext<V>::scaled ? P->d.tw_df : P->d.tw);
-    if (!tw) return cudaErrorInvalidValue;
+    const V* tw = static_cast<const V*>(P->d.tw);
     if constexpr (MODE == COL_FWD) {   // first kernel of the type-2 chain
         col_kernel<V, LOGNP, MODE><<<grid, Cf::P, sm, st>>>(static_cast<const MS*>(src), static_cast<MD*>(dst), tw, a);
     } else {
@@ -1316,20 +1313,12 @@ template <typename V, int LOGNP> struct Stages {
 };
 
 // dispatch on log2 N' (5 .. LOGMAX) at run time
-template <typename V, int LOGMAX, class F> cudaError_t dispatch(int lognp, F&& f) {
-    switch (lognp) {
-        case 5: return f(Stages<V, 5>{});
-        case 6: return f(Stages<V, 6>{});
-        case 7: return f(Stages<V, 7>{});
-        case 8: return f(Stages<V, 8>{});
-        case 9: return f(Stages<V, 9>{});
-        case 10: return f(Stages<V, 10>{});
-        case 11: return f(Stages<V, 11>{});
-        case 12: return f(Stages<V, 12>{});
-        case 13:
-            if constexpr (LOGMAX >= 13) return f(Stages<V, 13>{});
-            else return cudaErrorInvalidValue;
-        default: return cudaErrorInvalidValue;
+template <typename V, int LOGMAX, int L = 5, class F> cudaError_t dispatch(int lognp, F&& f) {
+    if constexpr (L > LOGMAX) {
+        return cudaErrorInvalidValue;
+    } else {
+        if (lognp == L) return f(Stages<V, L>{});
+        return dispatch<V, LOGMAX, L + 1>(lognp, f);
     }
 }
 

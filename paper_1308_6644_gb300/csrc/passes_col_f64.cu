@@ -1,6 +1,6 @@
-// Column-pass instantiations of FP64 plans for every supported N': from
-// N' = 512 up in double-float arithmetic (dfc, on the FP32 pipe) over the
-// plan's FP64 arrays, below in FP64 (double2), as the row passes.
+// Column-pass instantiations of FP64 plans for every supported N', in
+// double-float arithmetic (dfc, on the FP32 pipe) or FP64, as the row passes;
+// the window and the caller's planes are FP64.
 #include "passes.cuh"
 
 namespace nuasm {
@@ -15,17 +15,8 @@ cudaError_t col_f64(const nuasm_plan_s* P, int mode, const void* ext, cudaStream
             default: return S::col_inv_fold(P, s);
         }
     };
-    switch (P->g.lognp) {
-        case 5: return run(passes::Stages<double2, 5>{});
-        case 6: return run(passes::Stages<double2, 6>{});
-        case 7: return run(passes::Stages<double2, 7>{});
-        case 8: return run(passes::Stages<double2, 8>{});
-        case 9: return run(passes::Stages<dfc, 9>{});
-        case 10: return run(passes::Stages<dfc, 10>{});
-        case 11: return run(passes::Stages<dfc, 11>{});
-        case 12: return run(passes::Stages<dfc, 12>{});
-        default: return cudaErrorInvalidValue;
-    }
+    if (fft_double_float(P)) return passes::dispatch<dfc, 12>(P->g.lognp, run);
+    return passes::dispatch<double2, 8>(P->g.lognp, run);
 }
 
 }  // namespace nuasm

@@ -288,7 +288,7 @@ nuasm_status run_job(Server& S, Slot& sl, const Job& j, PointSet* ps, bool build
         sl.h_tab_bytes = tb;
     }
     int texp[3];
-    pack_tables(ht, g, f64, false, sl.h_tab, texp);
+    pack_tables(ht, g, f64, fft_double_float(f64, g.np, j.rp.tol), false, sl.h_tab, texp);
     const double rc = ht.rc, rmax = ht.rmax;
     free_tables(&ht);
 
@@ -326,7 +326,6 @@ nuasm_status run_job(Server& S, Slot& sl, const Job& j, PointSet* ps, bool build
     view.d.t3y = part[0] + 5 * np * eb;
     view.d.s = part[0] + 6 * np * eb;
     view.d.tw = B->d.tw;
-    view.d.tw_df = B->d.tw_df;
     view.d.etab = nullptr;   // one solve per table: E is evaluated per mode
     view.d.etab2 = nullptr;
     view.d.win = part[1];

@@ -83,3 +83,32 @@ def test_zero_sources(P, m):
         assert not u.cpu().numpy().any()
     finally:
         plan.destroy()
+
+
+@pytest.mark.parametrize("tol,bound", [(0.0, 1e-10), (1e-14, 1e-13)])
+@pytest.mark.parametrize("n", [16, 64, 128])
+@pytest.mark.parametrize("type_", [1, 2])
+def test_small_planes_in_both_arithmetics(P, n, type_, tol, bound):
+    """N' <= 256: double-float passes at the default tolerance, FP64 ones below
+    1e-12 (1e-13: the kernel's error at 1e-14 with some margin)."""
+    import torch
+    pitch, m = 5e-6, 301
+    rng = np.random.default_rng(83)
+    x, y = _points(rng, n, pitch, m)
+    p = dict(n=n, pitch=pitch, lam=500e-9, z=2e-3)
+    plan = P.nuasm_plan(P.make_params(n, pitch, 500e-9, 2e-3, prec="f64", tol=tol), _dev(x), _dev(y))
+    try:
+        if type_ == 1:
+            c = rng.normal(size=m) + 1j * rng.normal(size=m)
+            out = torch.zeros(n * n, dtype=torch.complex128, device="cuda")
+            P.nuasm1_execute(plan, _dev(c), out)
+            ref = O.nuasm1(x, y, c, p).ravel()
+        else:
+            u1 = rng.normal(size=(n, n)) + 1j * rng.normal(size=(n, n))
+            out = torch.zeros(m, dtype=torch.complex128, device="cuda")
+            P.nuasm2_execute(plan, _dev(u1.ravel()), out)
+            ref = O.nuasm2(u1, x, y, p)
+        torch.cuda.synchronize()
+        assert O.rel_l2(out.cpu().numpy(), ref) < bound
+    finally:
+        plan.destroy()
