@@ -125,7 +125,7 @@ typedef struct {
                               same bit for bit; values 1..63 or < 0 return NUASM_EINVAL. */
     int32_t spread_chunk;  /* type-1 spreading, for the kernels that can split a tile (FP64, and
                               FP32 tiles of side <= 32): 0 = the library's rule (a tile with
-                              more records than the larger of 128 (FP64) / 512 (FP32) and an
+                              more records than the larger of 128 (FP64) / 1024 (FP32) and an
                               even share over two CTAs per SM is split into chunks of at most
                               that many, each adding into the window); -1 = never split;
                               N >= 32 = split above N records.  Results agree to rounding;

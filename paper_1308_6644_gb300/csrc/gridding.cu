@@ -302,6 +302,15 @@ template <int WMAX> __device__ __forceinline__ void tap_weights(float f, const K
         out[i] = acc;
     }
 }
+// one tap's weight, the tap chosen at run time
+template <int WMAX> __device__ __forceinline__ float tap_weight(float f, const KernelPoly& kp, int i) {
+    constexpr int DMAX = WMAX + 2 < kPolyMaxD ? WMAX + 2 : kPolyMaxD;
+    const float x = fmaf(2.f, f, -1.f);
+    float acc = kp.c[i][DMAX - 1];
+#pragma unroll 1
+    for (int k = DMAX - 2; k >= 0; --k) acc = fmaf(acc, x, kp.c[i][k]);
+    return acc;
+}
 template <int WMAX> __device__ __forceinline__ void tap_weights(double f, const KernelPoly64& kp, double* out) {
     const double x = fma(2.0, f, -1.0);
 #pragma unroll
@@ -352,11 +361,11 @@ template <typename S> __device__ __forceinline__ void report_expo([[maybe_unused
 // --------------------------------------------------------------- spreading (type 1)
 // EXACT: the kernel width is WMAX itself (compile-time loops); else w <= WMAX at run time.
 // Three accumulation schemes, picked by precision and tile side in spread_impl:
-// warp-private copies (small tiles), batched int32 sums (FP32, T = 64) and,
-// here, shared-memory atomicAdd in the plan's precision (FP64 large tiles; on
-// sm_103a a float or double shared-memory atomicAdd is a compare-and-swap
-// loop -- 9.4 instructions and 2 wavefronts per float add, against one native
-// operation for a 32-bit integer).  Also measured and not kept: one int32
+// batched int32 sums (FP32), warp-private copies (FP64, T = 16) and, here,
+// shared-memory atomicAdd in FP64 (larger tiles; on sm_103a a float or double
+// shared-memory atomicAdd is a compare-and-swap loop -- 9.4 instructions and 2
+// wavefronts per float add, against one native operation for a 32-bit
+// integer).  Also measured and not kept: one int32
 // word per value at a single quantum per 8-row band for all of a tile's
 // records (1.6x faster than float but 1.1e-5 end to end where thousands of
 // random-phase points crowd a few cells -- the batched scheme fixes this by a
@@ -366,19 +375,13 @@ template <typename S> __device__ __forceinline__ void report_expo([[maybe_unused
 #ifndef NUASM_SPREAD_MINB
 #define NUASM_SPREAD_MINB 1
 #endif
-#ifndef NUASM_SPREAD_FIXED
-#define NUASM_SPREAD_FIXED 1       // FP32 tiles beyond the private-copy sizes: batched integer accumulation
-#endif
 #ifndef NUASM_SPREAD_FIXED_RPB
 #define NUASM_SPREAD_FIXED_RPB 2   // records per thread per batch (4: 4% faster, 1.6x the error of dense cancelling sums)
-#endif
-#ifndef NUASM_SPREAD_PRIVATE
-#define NUASM_SPREAD_PRIVATE 1   // per-warp private tiles where they fit (T <= 32 F32, <= 16 F64)
 #endif
 template <typename S, int WMAX, bool EXACT>
 __global__ void __launch_bounds__(256, sizeof(S) == 4 ? NUASM_SPREAD_MINB : 1) spread_kernel(const typename RecOf<S>::type* __restrict__ rec,
                                                      const int* __restrict__ off, const double* __restrict__ wpt,
-                                                     const int* __restrict__ order,
+                                                     const int4* __restrict__ order,
                                                      const typename VecOf<S>::type* __restrict__ c,
                                                      typename VecOf<S>::type* __restrict__ win, GridArgs a,
                                                      const typename PolyOf<S>::type kp,
@@ -394,9 +397,10 @@ __global__ void __launch_bounds__(256, sizeof(S) == 4 ? NUASM_SPREAD_MINB : 1) s
         e = it.z;
         chunked = it.w;
     } else {       // a whole tile, heaviest tiles first
-        tile = order ? order[blockIdx.x] : blockIdx.x;
-        b = off[tile];
-        e = off[tile + 1];
+        const int4 d = order[blockIdx.x];
+        tile = d.x;
+        b = d.y;
+        e = d.w;
     }
     const int T = a.T, w = EXACT ? WMAX : a.w, TS = plane_stride(T, a.skew_of(tile)), TT = T * TS;
     S* sre = reinterpret_cast<S*>(smem_raw);
@@ -454,22 +458,25 @@ __global__ void __launch_bounds__(256, sizeof(S) == 4 ? NUASM_SPREAD_MINB : 1) s
     }
 }
 
-// Spreading for large FP32 tiles with integer accumulation in batches.  On
-// sm_103a a shared-memory float atomicAdd is a compare-and-swap loop while a
-// 32-bit integer atomicAdd is native.  The CTA takes its records in batches of
-// RPB x 256; per batch it sums S = sum(|re| + |im|) of the batch's values
-// (weights included) and adds every tap contribution v wx wy / q, q = S 2^-30,
-// rounded to an integer, into int32 planes: a batch's sum at one cell is at
-// most S / q = 2^30 in magnitude because the kernel is at most 1.  The planes
-// are then folded into FP32 totals (tot += q acc) and cleared.  A contribution
-// is thus rounded to within max(q/2, its own FP32 rounding), q being a 2^-30
-// share of one batch's magnitude, where a float atomic rounds to the running
-// cell value.  A batch whose S is zero is skipped; one whose S is not a normal
-// finite number (infinities, NaNs, or values so small that q would underflow)
-// adds to the totals with float atomics, so non-finite inputs propagate as in
-// the float path.  The last batch of a tile folds its planes straight into
-// the window write (no fold into the totals, no clearing), and folds work
-// on pairs of cells (8-byte shared accesses).
+// Spreading of FP32 tiles with integer accumulation (every tile side: against
+// warp-private float copies, which tiles of side 16 and 32 had, whose chains of
+// dependent shared loads and stores took 19 us for 16,000 jittered points and 56
+// us for 200,000 clustered ones, T = 32).  On sm_103a a shared-memory float
+// atomicAdd is a compare-and-swap loop while a 32-bit integer atomicAdd is
+// native.  A contribution v wx wy is rounded to a multiple of the quantum q and
+// added to int32 planes, q such that no cell's sum leaves the range:
+//  * the plan knows each tile's load L, the largest sum of wx wy over its
+//    records at one cell (tile_load_kernel), so with V the largest |re| or |im|
+//    of the CTA's values (weights included) q = V L 2^-31 (1 + 2^-8) serves all
+//    of them at once: one pass for V, one that adds, one write of the window
+//    (the 2^-8 is room for the roundings of up to 2^24 contributions);
+//  * where records crowd a few cells (L > kMaxLoad; the error of a cell is about
+//    L 1e-9 of its value, that of FP32 sums of the same records sqrt(L) 7e-8),
+//    they go in batches with q = S 2^-30, S = sum(|re| + |im|) of the batch, each
+//    folded into FP32 totals (tot += q acc) and cleared.
+// Zero values are skipped; values so small that q would underflow (the skirts of
+// a Gaussian beam) are taken times 2^64 and back; values that are not finite add
+// with float atomics, so they propagate.
 //
 // Measured and not kept: planes extended by a (w - 1)-cell margin so that no
 // tap needs clipping (the 49 taps become straight-line atomics; 31% of the
@@ -484,54 +491,78 @@ __global__ void __launch_bounds__(256, sizeof(S) == 4 ? NUASM_SPREAD_MINB : 1) s
 // tile, then the others, so that whole warps spread without clipping (283 ->
 // 265 us there), since the second segment's bank classes crowd into the
 // tile's last columns and the interpolation over the same records slowed by
-// more (94.8 -> 109.5 us).  And: the FP32 totals kept in the tile's own
-// window cells (read and written through L2 by the folds) instead of shared
-// memory, which leaves 32 KB per CTA and room for five CTAs per SM: 279 ->
-// 288 us (304 us at four CTAs, 320 us at six), so more resident tiles do not
-// make the shared atomics go faster.
+// more (94.8 -> 109.5 us).
 #ifndef NUASM_SPREAD_FIXED_MINB
-#define NUASM_SPREAD_FIXED_MINB 3   // CTAs per SM the register budget is set for
+#define NUASM_SPREAD_FIXED_MINB 4   // CTAs of 256 threads per SM the register budget is set for
 #endif
-constexpr int kFixedThreads = 256;
-template <int WMAX, bool EXACT, int RPB>
-__global__ void __launch_bounds__(kFixedThreads, NUASM_SPREAD_FIXED_MINB) spread_fixed_kernel(const RecF* __restrict__ rec,
+constexpr float kMaxLoad = 256.f;
+template <int WMAX, bool EXACT, int RPB, int NT>
+__global__ void __launch_bounds__(NT, NUASM_SPREAD_FIXED_MINB * 256 / NT) spread_fixed_kernel(const RecF* __restrict__ rec,
                                                                       const int* __restrict__ off,
                                                                       const double* __restrict__ wpt,
-                                                                      const int* __restrict__ order,
+                                                                      const int4* __restrict__ order,
+                                                                      const float* __restrict__ load,
                                                                       const float2* __restrict__ c,
                                                                       float2* __restrict__ win, GridArgs a,
-                                                                      const KernelPoly kp) {
+                                                                      const KernelPoly kp,
+                                                                      const int4* __restrict__ items) {
     extern __shared__ unsigned char smem_raw[];
-    __shared__ float red[kFixedThreads / 32];
-    __shared__ float batch_sum;
-    const int tile = order ? order[blockIdx.x] : blockIdx.x;   // heaviest tiles first
+    __shared__ unsigned red[NT / 32];
+    int tile, b, e;
+    bool chunked = false;
+    if (items) {   // a chunk of a tile's records: several CTAs add into the tile (window cleared)
+        const int4 it = items[blockIdx.x];
+        tile = it.x;
+        b = it.y;
+        e = it.z;
+        chunked = it.w != 0;
+    } else {       // a whole tile, heaviest tiles first
+        const int4 d = order[blockIdx.x];
+        tile = d.x;
+        b = d.y;
+        e = d.w;
+    }
     const int T = a.T, w = EXACT ? WMAX : a.w, TS = plane_stride(T, a.skew_of(tile)), TT = T * TS;
     int* are = reinterpret_cast<int*>(smem_raw);
     int* aim = are + TT;
-    float* tre = reinterpret_cast<float*>(aim + TT);
+    float* tre = reinterpret_cast<float*>(aim + TT);   // totals: only where the plan has a crowded tile
     float* tim = tre + TT;
     pdl_allow_next();
     const int ty = tile / a.ntx, tx = tile - ty * a.ntx;
     const int x0 = tx * T, y0 = ty * T;
-    for (int i = threadIdx.x; i < TT; i += kFixedThreads) {
-        are[i] = 0;
-        aim[i] = 0;
-        tre[i] = 0.f;
-        tim[i] = 0.f;
-    }
-    const int b = off[tile], e = off[tile + 1];
+    const float L = load[tile];
+    const bool crowded = L > kMaxLoad;
+    for (int i = threadIdx.x; i < (crowded ? 4 : 2) * TT; i += NT) are[i] = 0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int half = T / 2;   // cells are folded and written in pairs
-    for (int i0 = b; i0 < e; i0 += RPB * kFixedThreads) {
-        RecF r[RPB];
-        float2 val[RPB];
-        float part = 0.f;
+    // cells (gx, gy) and (gx + 1, gy) of the window: W, x0 and xx are even, so both lie in it or neither
+    auto emit = [&](int gx, int gy, float4 v) {
+        if (gy >= a.W || gx >= a.W ||
+            !NUASM_IN_RANGE(gy * (long long)a.Wp + gx + 1, (long long)a.W * a.Wp, dbg::kSpreadWindow))
+            return;
+        float2* p = &win[size_t(gy) * a.Wp + gx];
+        if (!chunked) {
+            *reinterpret_cast<float4*>(p) = v;
+        } else {
+            if (v.x != 0.f || v.y != 0.f) {
+                atomicAdd(&p[0].x, v.x);
+                atomicAdd(&p[0].y, v.y);
+            }
+            if (v.z != 0.f || v.w != 0.f) {
+                atomicAdd(&p[1].x, v.z);
+                atomicAdd(&p[1].y, v.w);
+            }
+        }
+    };
+    RecF r[RPB];
+    float2 val[RPB];
+    auto fetch = [&](int i0, int end) {   // up to RPB records per thread from i0 on; none: zero values
 #pragma unroll
         for (int k = 0; k < RPB; ++k) {
-            const int i = i0 + threadIdx.x + k * kFixedThreads;
+            const int i = i0 + threadIdx.x + k * NT;
             val[k] = make_float2(0.f, 0.f);
             r[k].cell = 0;
-            if (i < e && NUASM_IN_RANGE(i, a.nrec, dbg::kSpreadRec)) {
+            if (i < end && NUASM_IN_RANGE(i, a.nrec, dbg::kSpreadRec)) {
                 r[k] = rec[i];
                 if (!NUASM_IN_RANGE(r[k].j, a.m, dbg::kSpreadValue)) r[k].j = 0;
                 val[k] = c[r[k].j];
@@ -540,108 +571,188 @@ __global__ void __launch_bounds__(kFixedThreads, NUASM_SPREAD_FIXED_MINB) spread
                     val[k].x *= wt;
                     val[k].y *= wt;
                 }
-                part += fabsf(val[k].x) + fabsf(val[k].y);
             }
         }
+    };
+    // add the fetched records' taps (times inv) to the int32 planes, or (rare: rolled
+    // loops, to keep the kernel's code small) as floats in their place
+    auto add_taps = [&](int i0, int end, float pre, float inv, bool fixed) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-        if (lane == 0) red[warp] = part;
-        __syncthreads();   // also orders the clearing above and the previous batch's fold
-        if (threadIdx.x == 0) {
-            float t = 0.f;
-#pragma unroll
-            for (int k = 0; k < kFixedThreads / 32; ++k) t += red[k];
-            batch_sum = t;
-        }
-        __syncthreads();
-        const float S = batch_sum;
-        if (S == 0.f) continue;   // every value of the batch is zero (uniform)
-        const bool fixed = S >= 1e-30f && S <= 3.0e38f;
-        const float q = ldexpf(S, -30), inv = fixed ? 1.f / q : 1.f;
-        // The batch's mode is uniform across the CTA: one copy of the tap loops
-        // per mode, so that the integer atomics of clipped taps are predicated
-        // instead of branching around the float path's compare-and-swap loops.
-        auto add_taps = [&](auto fixed_mode) {
-            constexpr bool FX = decltype(fixed_mode)::value;
-            auto add = [&](int cell, float vr, float vi) {
-                if (!NUASM_IN_RANGE(cell, TT, dbg::kSpreadPlane)) return;
-                if constexpr (FX) {
-                    atomicAdd(&are[cell], __float2int_rn(vr));
-                    atomicAdd(&aim[cell], __float2int_rn(vi));
-                } else {
-                    atomicAdd(&tre[cell], vr);
-                    atomicAdd(&tim[cell], vi);
-                }
-            };
-#pragma unroll
-            for (int k = 0; k < RPB; ++k) {
-                const int i = i0 + threadIdx.x + k * kFixedThreads;
-                if (i >= e) continue;
-                const int lx = int(r[k].cell & 0xffffu) - x0, ly = int(r[k].cell >> 16) - y0;
-                float wx[WMAX], wy[WMAX];
-                tap_weights<WMAX>(r[k].fx, kp, wx);
-                tap_weights<WMAX>(r[k].fy, kp, wy);
-                const float sr = val[k].x * inv, si = val[k].y * inv;
-                const int ya = max(0, -ly), yb = min(w, T - ly);
-                const int xa = max(0, -lx), xb = min(w, T - lx);
-#pragma unroll(WMAX <= 16 ? WMAX : 1)
-                for (int qy = 0; qy < WMAX; ++qy) {
-                    if (qy < ya || qy >= yb) continue;
-                    const float vr = sr * wy[qy], vi = si * wy[qy];
-                    const int rowi = (ly + qy) * TS + lx;
-#pragma unroll
-                    for (int qx = 0; qx < WMAX; ++qx) {
-                        if (qx < xa || qx >= xb) continue;
-                        add(rowi + qx, vr * wx[qx], vi * wx[qx]);
+        for (int k = 0; k < RPB; ++k) {
+            const int i = i0 + threadIdx.x + k * NT;
+            if (i >= end) continue;
+            const int lx = int(r[k].cell & 0xffffu) - x0, ly = int(r[k].cell >> 16) - y0;
+            const float sr = val[k].x * pre * inv, si = val[k].y * pre * inv;
+            const int ya = max(0, -ly), yb = min(w, T - ly);
+            const int xa = max(0, -lx), xb = min(w, T - lx);
+            if (!fixed) {
+#pragma unroll 1
+                for (int qy = ya; qy < yb; ++qy) {
+                    const float wyq = tap_weight<WMAX>(r[k].fy, kp, qy);
+#pragma unroll 1
+                    for (int qx = xa; qx < xb; ++qx) {
+                        const float wxy = wyq * tap_weight<WMAX>(r[k].fx, kp, qx);
+                        const int cell = (ly + qy) * TS + lx + qx;
+                        if (!NUASM_IN_RANGE(cell, TT, dbg::kSpreadPlane)) continue;
+                        atomicAdd(reinterpret_cast<float*>(&are[cell]), sr * wxy);
+                        atomicAdd(reinterpret_cast<float*>(&aim[cell]), si * wxy);
                     }
                 }
+                continue;
             }
-        };
-        if (fixed) add_taps(std::true_type{});
-        else add_taps(std::false_type{});
-        if (fixed) {
-            __syncthreads();
-            if (i0 + RPB * kFixedThreads >= e) {
-                // last batch: fold into the window write
-                for (int i = threadIdx.x; i < T * half; i += kFixedThreads) {
-                    const int yy = i / half, xx = 2 * (i - yy * half), j = yy * TS + xx;
-                    const int2 rr = *reinterpret_cast<const int2*>(&are[j]);
-                    const int2 mm = *reinterpret_cast<const int2*>(&aim[j]);
-                    const float2 tr = *reinterpret_cast<const float2*>(&tre[j]);
-                    const float2 ti = *reinterpret_cast<const float2*>(&tim[j]);
-                    const int gy = y0 + yy, gx = x0 + xx;
-                    if (gy < a.W && gx < a.W &&   // W, x0 and xx are even: both cells or neither
-                        NUASM_IN_RANGE(gy * (long long)a.Wp + gx + 1, (long long)a.W * a.Wp, dbg::kSpreadWindow))
-                        *reinterpret_cast<float4*>(&win[size_t(gy) * a.Wp + gx]) =
-                            make_float4(fmaf(float(rr.x), q, tr.x), fmaf(float(mm.x), q, ti.x),
-                                        fmaf(float(rr.y), q, tr.y), fmaf(float(mm.y), q, ti.y));
+            float wx[WMAX], wy[WMAX];
+            tap_weights<WMAX>(r[k].fx, kp, wx);
+            tap_weights<WMAX>(r[k].fy, kp, wy);
+#pragma unroll(WMAX <= 16 ? WMAX : 1)
+            for (int qy = 0; qy < WMAX; ++qy) {
+                if (qy < ya || qy >= yb) continue;
+                const float vr = sr * wy[qy], vi = si * wy[qy];
+                const int rowi = (ly + qy) * TS + lx;
+#pragma unroll
+                for (int qx = 0; qx < WMAX; ++qx) {
+                    if (qx < xa || qx >= xb) continue;
+                    if (!NUASM_IN_RANGE(rowi + qx, TT, dbg::kSpreadPlane)) continue;
+                    atomicAdd(&are[rowi + qx], __float2int_rn(vr * wx[qx]));
+                    atomicAdd(&aim[rowi + qx], __float2int_rn(vi * wx[qx]));
                 }
-                return;
             }
-            for (int i = threadIdx.x; i < T * half; i += kFixedThreads) {
-                const int yy = i / half, xx = 2 * (i - yy * half), j = yy * TS + xx;
-                int2* pr = reinterpret_cast<int2*>(&are[j]);
-                int2* pm = reinterpret_cast<int2*>(&aim[j]);
-                float2* pa = reinterpret_cast<float2*>(&tre[j]);
-                float2* pb = reinterpret_cast<float2*>(&tim[j]);
-                const int2 rr = *pr, mm = *pm;
-                const float2 tr = *pa, ti = *pb;
-                *pa = make_float2(fmaf(float(rr.x), q, tr.x), fmaf(float(rr.y), q, tr.y));
-                *pb = make_float2(fmaf(float(mm.x), q, ti.x), fmaf(float(mm.y), q, ti.y));
-                *pr = make_int2(0, 0);
-                *pm = make_int2(0, 0);
+        }
+    };
+    constexpr int BATCH = RPB * NT;
+    // one quantum for all records (fixed, q), or one per batch
+    bool fixed = false, empty = false;
+    float q = 1.f, pre = 1.f, post = 1.f;   // the planes hold the values times pre in units of q; post = 1 / pre
+    auto set_quantum = [&](float bound, float scale) {
+        fixed = bound <= 3e38f;
+        pre = fixed && bound < 1e-20f ? 18446744073709551616.f : 1.f;
+        post = fixed && bound < 1e-20f ? 5.42101086242752217e-20f : 1.f;
+        q = fixed ? bound * pre * scale : 1.f;
+    };
+    int step = BATCH;
+    if (!crowded) {
+        unsigned top = 0;   // bits of the largest |re| or |im| (an infinity or a NaN tops every number)
+        for (int i0 = b; i0 < e; i0 += BATCH) {
+            fetch(i0, e);
+#pragma unroll
+            for (int k = 0; k < RPB; ++k)
+                top = max(top, max(__float_as_uint(val[k].x) & 0x7fffffffu, __float_as_uint(val[k].y) & 0x7fffffffu));
+        }
+        top = __reduce_max_sync(0xffffffffu, top);
+        if (lane == 0) red[warp] = top;
+        __syncthreads();   // also orders the clearing above
+#pragma unroll
+        for (int k = 0; k < NT / 32; ++k) top = max(top, red[k]);
+        const float bound = __uint_as_float(top) * L;   // of every cell's sum
+        empty = top == 0;
+        if (!empty) set_quantum(bound, 1.00390625f / 2147483648.f);
+    } else if (T <= 32) {
+        step = BATCH / 2;   // folds are cheap on small tiles: batches of half the records, half the quantum
+    }
+    for (int i0 = empty ? e : b; i0 < e; i0 += step) {
+        const int end = crowded ? min(e, i0 + step) : e;
+        if (crowded || e - b > BATCH) fetch(i0, end);   // else the first pass left the records in registers
+        if (crowded) {
+            float part = 0.f;
+#pragma unroll
+            for (int k = 0; k < RPB; ++k) part += fabsf(val[k].x) + fabsf(val[k].y);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+            __syncthreads();   // the clearing above, or the previous batch's fold and its reads of red, are done
+            if (lane == 0) red[warp] = __float_as_uint(part);
+            __syncthreads();
+            float S = 0.f;
+#pragma unroll
+            for (int k = 0; k < NT / 32; ++k) S += __uint_as_float(red[k]);
+            if (S == 0.f) continue;   // every value of the batch is zero (uniform)
+            set_quantum(S, 1.f / 1073741824.f);
+        }
+        add_taps(i0, end, pre, 1.f / q, fixed);
+        if (!crowded) continue;
+        // fold the batch into the totals and clear the planes
+        __syncthreads();
+        for (int i = threadIdx.x; i < T * half; i += NT) {
+            const int yy = i / half, xx = 2 * (i - yy * half), j = yy * TS + xx;
+            int2* pr = reinterpret_cast<int2*>(&are[j]);
+            int2* pm = reinterpret_cast<int2*>(&aim[j]);
+            float2* pa = reinterpret_cast<float2*>(&tre[j]);
+            float2* pb = reinterpret_cast<float2*>(&tim[j]);
+            const int2 rr = *pr, mm = *pm;
+            const float2 tr = *pa, ti = *pb;
+            if (fixed) {
+                *pa = make_float2(fmaf(float(rr.x) * q, post, tr.x), fmaf(float(rr.y) * q, post, tr.y));
+                *pb = make_float2(fmaf(float(mm.x) * q, post, ti.x), fmaf(float(mm.y) * q, post, ti.y));
+            } else {
+                *pa = make_float2(tr.x + __int_as_float(rr.x), tr.y + __int_as_float(rr.y));
+                *pb = make_float2(ti.x + __int_as_float(mm.x), ti.y + __int_as_float(mm.y));
+            }
+            *pr = make_int2(0, 0);
+            *pm = make_int2(0, 0);
+        }
+    }
+    __syncthreads();
+    // the window's cells: the planes in units of q, the planes as floats, or the totals
+    const int* ore = crowded ? reinterpret_cast<const int*>(tre) : are;
+    const int* oim = crowded ? reinterpret_cast<const int*>(tim) : aim;
+    const bool ints = fixed && !crowded;
+    for (int i = threadIdx.x; i < T * half; i += NT) {
+        const int yy = i / half, xx = 2 * (i - yy * half), j = yy * TS + xx;
+        const int2 rr = *reinterpret_cast<const int2*>(&ore[j]), mm = *reinterpret_cast<const int2*>(&oim[j]);
+        float4 v = make_float4(__int_as_float(rr.x), __int_as_float(mm.x), __int_as_float(rr.y), __int_as_float(mm.y));
+        if (ints)
+            v = make_float4(float(rr.x) * q * post, float(mm.x) * q * post, float(rr.y) * q * post,
+                            float(mm.y) * q * post);
+        emit(x0 + xx, y0 + yy, v);
+    }
+}
+
+// Plan time (FP32): each tile's load, the largest sum over its records of wx wy
+// at one cell, rounded up, and the largest of all tiles' (bits, in *most).  Sums
+// in units of 2^-14 fit int32 for 2^17 records at one cell; tiles with more
+// records take their count.
+template <int WMAX, bool EXACT>
+__global__ void __launch_bounds__(256) tile_load_kernel(const RecF* __restrict__ rec, const int* __restrict__ off,
+                                                        GridArgs a, const KernelPoly kp, float* __restrict__ load,
+                                                        unsigned* __restrict__ most) {
+    extern __shared__ unsigned char smem_raw[];
+    __shared__ int red[8];
+    const int tile = blockIdx.x, b = off[tile], e = off[tile + 1];
+    const int T = a.T, w = EXACT ? WMAX : a.w, TS = plane_stride(T, a.skew_of(tile)), TT = T * TS;
+    int* sum = reinterpret_cast<int*>(smem_raw);
+    const int ty = tile / a.ntx, tx = tile - ty * a.ntx;
+    const int x0 = tx * T, y0 = ty * T;
+    for (int i = threadIdx.x; i < TT; i += 256) sum[i] = 0;
+    __syncthreads();
+    const bool count = e - b > 100000;
+    for (int i = b + threadIdx.x; i < e && !count; i += 256) {
+        if (!NUASM_IN_RANGE(i, a.nrec, dbg::kSpreadRec)) continue;
+        const RecF r = rec[i];
+        const int lx = int(r.cell & 0xffffu) - x0, ly = int(r.cell >> 16) - y0;
+        float wx[WMAX], wy[WMAX];
+        tap_weights<WMAX>(r.fx, kp, wx);
+        tap_weights<WMAX>(r.fy, kp, wy);
+#pragma unroll(WMAX <= 16 ? WMAX : 1)
+        for (int qy = 0; qy < WMAX; ++qy) {
+            if (qy >= w || ly + qy < 0 || ly + qy >= T) continue;
+#pragma unroll
+            for (int qx = 0; qx < WMAX; ++qx) {
+                if (qx >= w || lx + qx < 0 || lx + qx >= T) continue;
+                const int cell = (ly + qy) * TS + lx + qx;
+                if (NUASM_IN_RANGE(cell, TT, dbg::kSpreadPlane))
+                    atomicAdd(&sum[cell], __float2int_ru(fabsf(wx[qx] * wy[qy]) * 16384.f));
             }
         }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < T * half; i += kFixedThreads) {
-        const int yy = i / half, xx = 2 * (i - yy * half), j = yy * TS + xx;
-        const float2 tr = *reinterpret_cast<const float2*>(&tre[j]);
-        const float2 ti = *reinterpret_cast<const float2*>(&tim[j]);
-        const int gy = y0 + yy, gx = x0 + xx;
-        if (gy < a.W && gx < a.W &&
-            NUASM_IN_RANGE(gy * (long long)a.Wp + gx + 1, (long long)a.W * a.Wp, dbg::kSpreadWindow))
-            *reinterpret_cast<float4*>(&win[size_t(gy) * a.Wp + gx]) = make_float4(tr.x, ti.x, tr.y, ti.y);
+    int top = 0;
+    for (int i = threadIdx.x; i < TT; i += 256) top = max(top, sum[i]);
+    top = __reduce_max_sync(0xffffffffu, top);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = top;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < 8; ++k) top = max(top, red[k]);
+        const float v = count ? 1.0001f * float(e - b) : 1.0001f * (float(top) / 16384.f);
+        load[tile] = v;
+        atomicMax(most, __float_as_uint(v));
     }
 }
 
@@ -652,13 +763,12 @@ __global__ void __launch_bounds__(kFixedThreads, NUASM_SPREAD_FIXED_MINB) spread
 // is seen by the loads of the next.  Within one offset two lanes touch the
 // same cell only if their records share the first-tap cell; such a batch
 // (found with __match_any_sync) adds with atomics instead.  The copies are
-// summed at the end.  Shared memory: 8 warps x T^2 complex, so T <= 32 (F32)
-// or T <= 16 (F64).
+// summed at the end.  Shared memory: 8 warps x T^2 complex, so T = 16 (FP64).
 template <typename S, int WMAX, bool EXACT>
 __global__ void __launch_bounds__(256, 2) spread_private_kernel(const typename RecOf<S>::type* __restrict__ rec,
                                                              const int* __restrict__ off,
                                                              const double* __restrict__ wpt,
-                                                             const int* __restrict__ order,
+                                                             const int4* __restrict__ order,
                                                              const typename VecOf<S>::type* __restrict__ c,
                                                              typename VecOf<S>::type* __restrict__ win, GridArgs a,
                                                              const typename PolyOf<S>::type kp,
@@ -677,9 +787,10 @@ __global__ void __launch_bounds__(256, 2) spread_private_kernel(const typename R
         e = it.z;
         chunked = it.w;
     } else {       // a whole tile, heaviest tiles first
-        tile = order ? order[blockIdx.x] : blockIdx.x;
-        b = off[tile];
-        e = off[tile + 1];
+        const int4 d = order[blockIdx.x];
+        tile = d.x;
+        b = d.y;
+        e = d.w;
     }
     const int T = a.T, w = EXACT ? WMAX : a.w, TS = plane_stride(T, a.skew_of(tile)), TT = T * TS;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -817,7 +928,7 @@ template <typename S, int WMAX, bool EXACT>
 __global__ void __launch_bounds__(kInterpThreads, sizeof(S) == 4 ? NUASM_INTERP_MINB : 2) interp_kernel(const typename RecOf<S>::type* __restrict__ rec,
                                                                 const int* __restrict__ off,
                                                                 const int* __restrict__ home,
-                                                                const int* __restrict__ order,
+                                                                const int4* __restrict__ order,
                                                                 const int4* __restrict__ items,
                                                                 const typename VecOf<S>::type* __restrict__ win,
                                                                 typename VecOf<S>::type* __restrict__ v, GridArgs a,
@@ -834,9 +945,11 @@ __global__ void __launch_bounds__(kInterpThreads, sizeof(S) == 4 ? NUASM_INTERP_
         b = it.y;
         e = it.z;
     } else {       // a whole tile, heaviest tiles first
-        tile = order ? order[blockIdx.x] : blockIdx.x;
-        b = off[tile];
-        e = b + home[tile];
+        const int4 d = order ? order[blockIdx.x] : make_int4(blockIdx.x, off[blockIdx.x],
+                                                             off[blockIdx.x] + home[blockIdx.x], 0);
+        tile = d.x;
+        b = d.y;
+        e = d.z;
     }
     const int THP = halo_pitch(TH, a.skew_of(tile));
     const int ty = tile / a.ntx, tx = tile - ty * a.ntx;
@@ -1109,7 +1222,7 @@ __device__ __forceinline__ double scaled_int(long long V, int k) {
 template <int WMAX>
 __global__ void __launch_bounds__(256, WMAX <= 13 ? NUASM_DF_SPREAD_MINB : 2) spread_df_kernel(const RecD* __restrict__ rec, const int* __restrict__ off,
                                                           const double* __restrict__ wpt,
-                                                          const int* __restrict__ order,
+                                                          const int4* __restrict__ order,
                                                           const double2* __restrict__ c, double2* __restrict__ win,
                                                           GridArgs a, const KernelPolyDF kp,
                                                           const int4* __restrict__ items, int* __restrict__ expo) {
@@ -1127,9 +1240,10 @@ __global__ void __launch_bounds__(256, WMAX <= 13 ? NUASM_DF_SPREAD_MINB : 2) sp
         e = it.z;
         chunked = it.w != 0;
     } else {       // a whole tile, heaviest tiles first
-        tile = order ? order[blockIdx.x] : blockIdx.x;
-        b = off[tile];
-        e = off[tile + 1];
+        const int4 d = order[blockIdx.x];
+        tile = d.x;
+        b = d.y;
+        e = d.w;
     }
     const int T = a.T, TS = plane_stride(T, a.skew_of(tile)), TT = T * TS;
     int* rh = reinterpret_cast<int*>(smem_raw);
@@ -1321,7 +1435,7 @@ template <int WMAX>
 __global__ void __launch_bounds__(kInterpThreads, 2) interp_df_kernel(const RecD* __restrict__ rec,
                                                                       const int* __restrict__ off,
                                                                       const int* __restrict__ home,
-                                                                      const int* __restrict__ order,
+                                                                      const int4* __restrict__ order,
                                                                       const int4* __restrict__ items,
                                                                       const double2* __restrict__ win,
                                                                       double2* __restrict__ v, GridArgs a,
@@ -1340,9 +1454,11 @@ __global__ void __launch_bounds__(kInterpThreads, 2) interp_df_kernel(const RecD
         b = it.y;
         e = it.z;
     } else {
-        tile = order ? order[blockIdx.x] : blockIdx.x;
-        b = off[tile];
-        e = b + home[tile];
+        const int4 d = order ? order[blockIdx.x] : make_int4(blockIdx.x, off[blockIdx.x],
+                                                             off[blockIdx.x] + home[blockIdx.x], 0);
+        tile = d.x;
+        b = d.y;
+        e = d.z;
     }
     const int THP = halo_pitch(TH, a.skew_of(tile));
     const int ty = tile / a.ntx, tx = tile - ty * a.ntx;
@@ -1391,12 +1507,9 @@ __global__ void __launch_bounds__(kInterpThreads, 2) interp_df_kernel(const RecD
     }
 }
 
-// whether the plan's spreading runs spread_private_kernel or spread_kernel,
-// which take work items (spread_fixed_kernel keeps one CTA per tile)
-bool spread_by_items(const nuasm_plan_s* P) {
-    if (NUASM_SPREAD_PRIVATE && P->g.T <= (P->f64 ? 16 : 32)) return true;
-    return P->f64 || !NUASM_SPREAD_FIXED;
-}
+// whether the plan's spreading may split a tile's records over CTAs (FP32 tiles
+// of side 64 keep one CTA each)
+bool spread_by_items(const nuasm_plan_s* P) { return P->f64 || P->g.T <= 32; }
 
 GridArgs grid_args(const nuasm_plan_s* P) {
     GridArgs a;
@@ -1446,27 +1559,34 @@ cudaError_t spread_impl(const nuasm_plan_s* P, const void* c, cudaStream_t st) {
         cudaError_t e = clear();
         if (e != cudaSuccess) return e;
     }
-    if (NUASM_SPREAD_PRIVATE && a.T <= (sizeof(S) == 4 ? 32 : 16)) {
-        const size_t sm = size_t(8) * a.T * plane_stride(a.T, a.max_skew) * sizeof(V);
-        cudaError_t e = set_smem(spread_private_kernel<S, WMAX, EXACT>, sm);
-        if (e != cudaSuccess) return e;
-        spread_private_kernel<S, WMAX, EXACT><<<grid, 256, sm, st>>>(
-            static_cast<const typename RecOf<S>::type*>(P->d.rec), P->d.tile_off, P->d.wpt, P->d.tile_order,
-            static_cast<const V*>(c), static_cast<V*>(P->d.win), a, taps_arg<S>(P), items, expo);
-        return cudaGetLastError();
-    }
     if constexpr (sizeof(S) == 4) {
-        if (NUASM_SPREAD_FIXED) {
-            constexpr int RPB = NUASM_SPREAD_FIXED_RPB;
-            const size_t sm = size_t(4) * a.T * plane_stride(a.T, a.max_skew) * sizeof(float);
-            cudaError_t e = set_smem(spread_fixed_kernel<WMAX, EXACT, RPB>, sm);
+        auto fixed = [&](auto threads) -> cudaError_t {
+            constexpr int RPB = NUASM_SPREAD_FIXED_RPB, NT = decltype(threads)::value;
+            // int32 planes, and totals where the plan has a crowded tile
+            const size_t sm = size_t(P->max_load > kMaxLoad ? 4 : 2) * a.T * plane_stride(a.T, a.max_skew) * sizeof(float);
+            cudaError_t e = set_smem(spread_fixed_kernel<WMAX, EXACT, RPB, NT>, sm);
             if (e != cudaSuccess) return e;
-            spread_fixed_kernel<WMAX, EXACT, RPB><<<P->g.ntiles, kFixedThreads, sm, st>>>(
-                static_cast<const RecF*>(P->d.rec), P->d.tile_off, P->d.wpt, P->d.tile_order,
-                static_cast<const float2*>(c), static_cast<float2*>(P->d.win), a, taps_arg<S>(P));
+            spread_fixed_kernel<WMAX, EXACT, RPB, NT><<<grid, NT, sm, st>>>(
+                static_cast<const RecF*>(P->d.rec), P->d.tile_off, P->d.wpt, P->d.tile_order, P->d.tile_load,
+                static_cast<const float2*>(c), static_cast<float2*>(P->d.win), a, taps_arg<S>(P), items);
+            return cudaGetLastError();
+        };
+        // tiles of side 16 with at most two records a thread in the fullest (kept
+        // in registers from the first pass) take 128 threads, so that twice as many CTAs run side by side
+        // (uniform 256 x 256 plane 13.0 against 15.1 us with 256 threads; where
+        // tiles are fuller 256 threads, 200,000 clustered points 29.7 against 42.7 us)
+        if (a.T <= 16 && P->max_tile_rec <= 256) return fixed(std::integral_constant<int, 128>{});
+        return fixed(std::integral_constant<int, 256>{});
+    } else {
+        if (a.T <= 16) {
+            const size_t sm = size_t(8) * a.T * plane_stride(a.T, a.max_skew) * sizeof(V);
+            cudaError_t e = set_smem(spread_private_kernel<S, WMAX, EXACT>, sm);
+            if (e != cudaSuccess) return e;
+            spread_private_kernel<S, WMAX, EXACT><<<grid, 256, sm, st>>>(
+                static_cast<const typename RecOf<S>::type*>(P->d.rec), P->d.tile_off, P->d.wpt, P->d.tile_order,
+                static_cast<const V*>(c), static_cast<V*>(P->d.win), a, taps_arg<S>(P), items, expo);
             return cudaGetLastError();
         }
-    }
     const size_t sm = size_t(2) * a.T * plane_stride(a.T, a.max_skew) * sizeof(S);
     cudaError_t e = set_smem(spread_kernel<S, WMAX, EXACT>, sm);
     if (e != cudaSuccess) return e;
@@ -1474,6 +1594,7 @@ cudaError_t spread_impl(const nuasm_plan_s* P, const void* c, cudaStream_t st) {
         static_cast<const typename RecOf<S>::type*>(P->d.rec), P->d.tile_off, P->d.wpt, P->d.tile_order,
         static_cast<const V*>(c), static_cast<V*>(P->d.win), a, taps_arg<S>(P), items, expo);
     return cudaGetLastError();
+    }
 }
 
 template <typename S, int WMAX, bool EXACT>
@@ -1488,7 +1609,7 @@ cudaError_t interp_impl(const nuasm_plan_s* P, void* v, cudaStream_t st) {
     cudaError_t e = set_smem(interp_kernel<S, WMAX, EXACT>, sm);
     if (e != cudaSuccess) return e;
     const int grid = P->d.interp_items ? P->n_interp_items : P->g.ntiles;
-    e = launch_chained(interp_kernel<S, WMAX, EXACT>, dim3(grid), dim3(kInterpThreads), sm, st,
+    e = launch_chained(launch_early(P), interp_kernel<S, WMAX, EXACT>, dim3(grid), dim3(kInterpThreads), sm, st,
                        static_cast<const typename RecOf<S>::type*>(P->d.rec), P->d.tile_off, P->d.tile_home,
                        P->d.tile_order, static_cast<const int4*>(P->d.interp_items), static_cast<const V*>(P->d.win),
                        static_cast<V*>(v), a, taps_arg<S>(P));
@@ -1523,7 +1644,7 @@ template <int WMAX> cudaError_t interp_df_impl(const nuasm_plan_s* P, void* v, c
     cudaError_t e = set_smem(interp_df_kernel<WMAX>, sm);
     if (e != cudaSuccess) return e;
     const int grid = P->d.interp_items ? P->n_interp_items : P->g.ntiles;
-    e = launch_chained(interp_df_kernel<WMAX>, dim3(grid), dim3(kInterpThreads), sm, st,
+    e = launch_chained(false, interp_df_kernel<WMAX>, dim3(grid), dim3(kInterpThreads), sm, st,
                        static_cast<const RecD*>(P->d.rec), P->d.tile_off, P->d.tile_home, P->d.tile_order,
                        static_cast<const int4*>(P->d.interp_items), static_cast<const double2*>(P->d.win),
                        static_cast<double2*>(v), a, P->poly64df);
@@ -1582,6 +1703,36 @@ template <bool SPREAD> cudaError_t gridding(const nuasm_plan_s* P, const void* i
     }
 }
 
+// Fill the plan's tile loads (FP32) and their maximum.
+cudaError_t fill_tile_load(nuasm_plan_s* P, cudaStream_t st) {
+    if (P->f64) return cudaSuccess;
+    const GridArgs a = grid_args(P);
+    unsigned* most = reinterpret_cast<unsigned*>(P->d.tile_load + P->g.ntiles);
+    cudaError_t e = cudaMemsetAsync(most, 0, sizeof(unsigned), st);
+    if (e != cudaSuccess) return e;
+    auto run = [&](auto tag) -> cudaError_t {
+        using Tg = decltype(tag);
+        auto kernel = tile_load_kernel<Tg::W, Tg::X>;
+        const size_t sm = size_t(a.T) * plane_stride(a.T, a.max_skew) * sizeof(int);
+        cudaError_t err = set_smem(kernel, sm);
+        if (err != cudaSuccess) return err;
+        kernel<<<P->g.ntiles, 256, sm, st>>>(static_cast<const RecF*>(P->d.rec), P->d.tile_off, a, P->poly,
+                                             P->d.tile_load, most);
+        return cudaGetLastError();
+    };
+    switch (P->g.w) {
+        case 4: e = run(GTag<float, 4, true>{}); break;
+        case 5: e = run(GTag<float, 5, true>{}); break;
+        case 6: e = run(GTag<float, 6, true>{}); break;
+        case 7: e = run(GTag<float, 7, true>{}); break;
+        case 8: e = run(GTag<float, 8, true>{}); break;
+        default: e = P->g.w <= 16 ? run(GTag<float, 16, false>{}) : run(GTag<float, kPolyMaxW, false>{});
+    }
+    if (e != cudaSuccess) return e;
+    e = cudaMemcpyAsync(&P->max_load, most, sizeof(float), cudaMemcpyDeviceToHost, st);
+    return e != cudaSuccess ? e : cudaStreamSynchronize(st);
+}
+
 }  // namespace
 
 static nuasm_status cuda_status(cudaError_t e) {
@@ -1606,7 +1757,7 @@ static nuasm_status cuda_status(cudaError_t e) {
 #define NUASM_SPREAD_CHUNK64 128
 #endif
 #ifndef NUASM_SPREAD_CHUNK32
-#define NUASM_SPREAD_CHUNK32 512
+#define NUASM_SPREAD_CHUNK32 1024
 #endif
 constexpr int64_t kSpreadChunk64 = NUASM_SPREAD_CHUNK64, kSpreadChunk32 = NUASM_SPREAD_CHUNK32;
 cudaError_t make_tile_order(nuasm_plan_s* P, cudaStream_t st) {
@@ -1620,9 +1771,18 @@ cudaError_t make_tile_order(nuasm_plan_s* P, cudaStream_t st) {
     std::iota(order.begin(), order.end(), 0);
     std::stable_sort(order.begin(), order.end(),
                      [&](int a, int b) { return off[a + 1] - off[a] > off[b + 1] - off[b]; });
-    if ((e = xmalloc(reinterpret_cast<void**>(&P->d.tile_order), sizeof(int) * size_t(nt))) != cudaSuccess) return e;
-    P->device_bytes += int64_t(sizeof(int)) * nt;
-    e = cudaMemcpyAsync(P->d.tile_order, order.data(), sizeof(int) * size_t(nt), cudaMemcpyHostToDevice, st);
+    P->max_tile_rec = off[order[0] + 1] - off[order[0]];
+    // the tiles with their record ranges, then their loads and the largest (fill_tile_load)
+    const size_t bytes = sizeof(int4) * size_t(nt) + sizeof(float) * (size_t(nt) + 1);
+    if ((e = xmalloc(reinterpret_cast<void**>(&P->d.tile_order), bytes)) != cudaSuccess) return e;
+    P->d.tile_load = reinterpret_cast<float*>(P->d.tile_order + nt);
+    P->device_bytes += int64_t(bytes);
+    std::vector<int4> desc(nt);
+    for (int i = 0; i < nt; ++i) {
+        const int t = order[i];
+        desc[i] = make_int4(t, off[t], off[t] + home[t], off[t + 1]);
+    }
+    e = cudaMemcpyAsync(P->d.tile_order, desc.data(), sizeof(int4) * size_t(nt), cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess || (e = cudaStreamSynchronize(st)) != cudaSuccess) return e;   // host vectors go out of scope
     if (spread_by_items(P) && P->nrec > 0 && P->p.spread_chunk >= 0) {
         // Spreading items: a tile whose records would keep one SM busy well past
@@ -1875,6 +2035,7 @@ nuasm_status run_binning(nuasm_plan_s* P, const double* x, const double* y, cons
         if ((e = cudaGetLastError()) != cudaSuccess) return fail(e);
     }
     if (P->m > 0 && total > 0 && (e = order_records(P, st)) != cudaSuccess) return fail(e);
+    if ((e = fill_tile_load(P, st)) != cudaSuccess) return fail(e);
     xfree_async(cnt, st);
     return cuda_status(cudaStreamSynchronize(st));
 }
@@ -1973,6 +2134,7 @@ nuasm_status run_binning_lattice(nuasm_plan_s* P, const LatticeSpec& lat, cudaSt
         if ((e = cudaGetLastError()) != cudaSuccess) return fail(e);
         if ((e = order_records(P, st)) != cudaSuccess) return fail(e);
     }
+    if ((e = fill_tile_load(P, st)) != cudaSuccess) return fail(e);
     xfree_async(scratch, st);
     return cuda_status(cudaStreamSynchronize(st));
 }

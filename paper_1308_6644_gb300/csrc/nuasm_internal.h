@@ -78,7 +78,10 @@ struct PlanDevice {
     double* wpt = nullptr;      // optional per-point weights, in point order
     int* tile_off = nullptr;    // ntiles + 1 offsets into rec
     int* tile_home = nullptr;   // home-record count per tile
-    int* tile_order = nullptr;  // launch order of the tiles (heaviest first); null = index order
+    int4* tile_order = nullptr; // launch order of the tiles (heaviest first): tile, its first record, the end of
+                                // its home records and of all its records in one load; null = index order
+                                // (interpolation of the allocation-free solve)
+    float* tile_load = nullptr; // FP32: largest sum of tap products at one cell of each tile (behind tile_order)
     int8_t* tile_skew = nullptr;    // bank skew of each tile's layouts and record order; null: skew for all
     int4* interp_items = nullptr;   // interpolation work items (tile, first record, end record, 0),
                                     // heaviest first; null = one item per tile in tile_order
@@ -104,6 +107,7 @@ struct nuasm_plan_s {
     int64_t nrec = 0;
     bool has_w = false;
     bool f64 = false;
+    bool batched = false;       // a view recorded into a batch
     double rc = 0.0;            // z / (2 lambda)
     int texp[3] = {0, 0, 0};    // double-float FFT passes: power of two taken out of type t's tables
     int nonsep_mode = 0;        // ASM non-separable phase: 0 none, 1 plain, 2 double-float
@@ -112,6 +116,8 @@ struct nuasm_plan_s {
                                 // tiles use when d.tile_skew is set, else the one every tile uses
     int n_interp_items = 0;     // entries of d.interp_items
     int n_spread_items = 0;     // entries of d.spread_items
+    int max_tile_rec = 0;       // records of the fullest tile
+    float max_load = 0.f;       // FP32: largest of d.tile_load
     nuasm::KernelPoly poly{};   // kernel taps as polynomials (F32 gridding)
     nuasm::KernelPoly64 poly64{};   // the same in FP64 (F64 gridding)
     nuasm::KernelPolyDF poly64df{};   // poly64 as float pairs (F64 gridding in double-float arithmetic)
@@ -239,6 +245,17 @@ inline size_t ws_bufB_elems(const Geometry& g) { return size_t(g.np) * g.n + kEx
 // plans below N' = 512 with a smaller one keep FP64 passes.
 inline bool fft_double_float(bool f64, int np, double tol) { return f64 && (np >= 512 || tol >= 1e-12); }
 inline bool fft_double_float(const nuasm_plan_s* P) { return fft_double_float(P->f64, P->g.np, P->p.tol); }
+// Whether a solve's kernels after the first launch before the previous one has
+// finished (launch_chained).  FP32 chains up to N' = 1024 do: the gaps between
+// the four kernels are hidden (N = 32 type 1 26.5 -> 20.5 us, N = 512 type 2 43.5 ->
+// 37.3).  At N' = 2048 the early CTAs cost as much as they hide (jittered points
+// 106 -> 97 us, graded ones 107 -> 113); from N' = 4096 on they must not run
+// early: the column passes there write with bulk tensor stores, which the early
+// kernel's wait does not cover (the next pass read stale values).  Batches
+// overlap whole planes instead (709 -> 727 us for 12 planes with early launches),
+// and FP64 chains gained 5% at N = 32 and 512 and lost as much at N = 128 and 256.
+inline bool launch_early(const nuasm_plan_s* P) { return !P->f64 && P->g.np <= 1024 && !P->batched; }
+
 // The exponents of a solve's double-float data, behind bufB's elements: word 0
 // the solve's (types 1 and 3: set by the spreading; type 2: by the row pass),
 // then type 2's one per strip of columns of the forward column pass.
