@@ -115,11 +115,13 @@ typedef struct {
     int32_t kernel;     /* nuasm_kernel: spreading kernel of the NUFFT gridding */
     int32_t tile;       /* side of the gridding tiles (bins) in fine-grid cells: 16, 32 or 64;
                            0 = the library's rule (the largest side giving at least 608
-                           tiles over the fine-grid window, else 16; at least w - 1 for
+                           tiles over the fine-grid window, else 16, or 32 for
+                           double-float gridding with 64 tiles; at least w - 1 for
                            a kernel of w taps).  A side below w - 1 returns
                            NUASM_EUNSUPPORTED.  Results agree to rounding for every
                            choice; nuasm_autotune_tile measures which is fastest. */
-    int32_t interp_chunk;  /* type-2 interpolation: 0 = one CTA per tile; N >= 64 = a tile with
+    int32_t interp_chunk;  /* type-2 interpolation: 0 = the library's rule (tiles of side 16 and 32
+                              that hold far more than their share are split); N >= 64 = a tile with
                               more than N home records is split into chunks of at most N
                               (rounded up to a multiple of 32), one CTA each.  Results are the
                               same bit for bit; values 1..63 or < 0 return NUASM_EINVAL. */

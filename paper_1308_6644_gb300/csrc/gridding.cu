@@ -1745,13 +1745,9 @@ static nuasm_status cuda_status(cudaError_t e) {
 // wave holds the lightest.
 //
 // Interpolation items: a tile with more than the plan's interp_chunk home
-// records (NUASM_INTERP_CHUNK where the plan leaves it 0) is split into
-// chunks of at most that many, each its own CTA (which stages the same tile),
-// so that the densest tiles do not hold the last wave; items are launched
-// heaviest first.  0 keeps one item per tile.
-#ifndef NUASM_INTERP_CHUNK
-#define NUASM_INTERP_CHUNK 0
-#endif
+// records is split into chunks of at most that many, each its own CTA (which
+// stages the same tile), so that the densest tiles do not hold the last wave;
+// items are launched heaviest first.
 // smallest spreading chunk (records) of a split tile, by precision
 #ifndef NUASM_SPREAD_CHUNK64
 #define NUASM_SPREAD_CHUNK64 128
@@ -1819,7 +1815,18 @@ cudaError_t make_tile_order(nuasm_plan_s* P, cudaStream_t st) {
             if (e != cudaSuccess || (e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
         }
     }
-    const int ich = P->p.interp_chunk > 0 ? P->p.interp_chunk : NUASM_INTERP_CHUNK;
+    // By default tiles of side 16 and 32 are split above K home records, K an even
+    // share over two CTAs per SM, at least 128 (FP64) or 512 (FP32) and at most
+    // 1024: where the plane has fewer tiles than SMs, or a tile with twice that
+    // (FP64, 60,000 clustered points at N = 128: 220 -> 58 us at side 32; FP32,
+    // 800,000 at N = 512: 54 -> 44 us; tiles of side 64 measured slower split, 94
+    // -> 101 us on the 4M clustered points).
+    int ich = P->p.interp_chunk;
+    if (ich == 0 && P->g.T <= 32) {
+        const int64_t k = std::min<int64_t>(1024, std::max<int64_t>(P->f64 ? 128 : 512, P->m / (2 * 152)));
+        const int most = nt > 0 ? *std::max_element(home.begin(), home.end()) : 0;
+        if (most > (nt < 152 ? k : 2 * k)) ich = int(k);
+    }
     if (ich > 0) {
         const int ch = ich;
         std::vector<int4> items;

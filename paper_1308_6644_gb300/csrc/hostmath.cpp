@@ -310,10 +310,14 @@ Geometry make_geometry(const nuasm_params_t& p) {
     g.Wp = (g.W + 31) & ~31;
     g.Lo = p.n_pad - p.n - g.h;
     // default tile: the largest side that still gives at least 608 tiles
-    // (four CTAs per SM on 152 SMs), else the smallest
+    // (four CTAs per SM on 152 SMs), else the smallest; in double-float gridding
+    // side 32 where that gives 64 tiles, since a side of 16 duplicates a record of
+    // 13 taps two more times (N = 128 type 1 76 -> 62 us, N = 256 123 -> 99; N = 64,
+    // 25 tiles of side 32: 58 -> 60 us)
     g.T = p.tile;
     if (!g.T) {
-        g.T = 16;
+        const int n32 = (g.W + 31) / 32;
+        g.T = gridding_double_float(p.prec == NUASM_PREC_F64, g.kernel, g.w) && n32 * n32 >= 64 ? 32 : 16;
         for (int t : {64, 32}) {
             const int per_axis = (g.W + t - 1) / t;
             if (per_axis * per_axis >= 608) {

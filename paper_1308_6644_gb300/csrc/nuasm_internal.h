@@ -138,11 +138,12 @@ namespace nuasm {
 #ifndef NUASM_F64_DF
 #define NUASM_F64_DF 1   // 0: FP64 gridding on the FP64 pipe throughout
 #endif
-inline bool gridding_double_float(const nuasm_plan_s* P) {
-    if (!NUASM_F64_DF || !P->f64) return false;
-    if (P->g.kernel == NUASM_KERNEL_ES) return P->g.w == 11 || P->g.w == 13;
-    return P->g.w == 15 || P->g.w == 21 || P->g.w == 25;
+inline bool gridding_double_float(bool f64, int kernel, int w) {
+    if (!NUASM_F64_DF || !f64) return false;
+    if (kernel == NUASM_KERNEL_ES) return w == 11 || w == 13;
+    return w == 15 || w == 21 || w == 25;
 }
+inline bool gridding_double_float(const nuasm_plan_s* P) { return gridding_double_float(P->f64, P->g.kernel, P->g.w); }
 
 // Gauss-Legendre quadrature of the kernel on [0, w/2] for its Fourier transform.
 struct KernelQuad {
