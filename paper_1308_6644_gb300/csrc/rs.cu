@@ -18,7 +18,7 @@
 // reproducible.  One destination point per thread and all sources in turn (the
 // earlier split) put 16384 points on 64 of the 152 SMs.  Measured (sources x
 // points, before -> now): FP32 65536 x 65536 14.6 -> 6.0 ms, 30000 x 3000 5.2 ->
-// 0.20 ms; FP64 16384 x 16384 83.6 -> 16.9 ms, 5001 x 1001 25.5 -> 0.48 ms.
+// 0.18 ms; FP64 16384 x 16384 83.6 -> 13.5 ms, 5001 x 1001 25.5 -> 0.39 ms.
 //
 // Lengths are scaled by the power of two that takes z into [1, 2), so the FP32
 // seeds below neither overflow nor meet subnormals for any unit of length.
@@ -196,10 +196,10 @@ __global__ void __launch_bounds__(kThreads, 3) rs_f32_kernel(const double* __res
 //    d (2z + d) = rho^2 in FP64;
 //  * 1 / r: rsqrt in FP32, then 1/r = y (1 + e + e^2), e = 1 - r y;
 //  * the phase: rounded to 1/2048 turn by an addition of 1.5 2^41, the rest
-//    (|theta| <= pi/2048) through short series whose last terms are FP32, times
-//    exp(2 pi i j / 2048) from shared memory.
-// exp(2 pi i frac(z/lambda)) is one factor of the whole sum.  33 FP64 operations
-// a pair, which bound it (85% of that pipe's rate).
+//    (|theta| <= pi/2048) through short series in double-float: exp(i theta) - 1
+//    times exp(2 pi i j / 2048) from shared memory, added to it in FP64.
+// exp(2 pi i frac(z/lambda)) is one factor of the whole sum.  27 FP64 operations
+// a pair, which bound it (33 with the series in FP64).
 struct Src64 { double x, y, re, im; };
 struct Pair64 { double re, im; };
 
@@ -216,28 +216,12 @@ __device__ __noinline__ Pair64 rs_pair_direct(double dx, double dy, const double
 }
 
 // The FP64 conversion instructions run at the FP64 rate, so values cross between
-// the two by their bits: a float as a double (a zero as 2^-127), a positive or
-// negative double of ordinary size truncated to a float, and the sum of a
-// double-float (|lo| at most half an ulp of hi) as a double.
+// the two by their bits (dfr_split, dfr_to_double, and here a float as a double, a
+// zero as 2^-127).
 __device__ __forceinline__ double wide(float x) {
     const unsigned u = __float_as_uint(x);
     return __hiloint2double(int((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), int(u << 29));
 }
-__device__ __forceinline__ float narrow(double x) {
-    const unsigned h = unsigned(__double2hiint(x)), l = unsigned(__double2loint(x));
-    const unsigned m = ((h & 0x7fffffffu) - 0x38000000u) << 3 | l >> 29;
-    return (h & 0x7fffffffu) > 0x38000000u ? __uint_as_float(m | (h & 0x80000000u)) : 0.f;
-}
-__device__ __forceinline__ double wide_sum(float hi, float lo) {
-    // hi's bits as a double, plus lo in units of 2^-29 ulp(hi) (of 2^-30 where a
-    // power of two loses to a negative lo)
-    const unsigned u = __float_as_uint(hi);
-    const int unit = 127 + 127 + 23 + 29 - int(u >> 23);   // exponent field of 2^29 / ulp(hi)
-    long long i = __float2int_rn(lo * __uint_as_float(unsigned(unit) << 23));
-    if ((u & 0x7fffffu) == 0 && i < 0) i *= 2;
-    return __longlong_as_double((static_cast<long long>((u >> 3) + 0x38000000u) << 32 | (u << 29)) + i);
-}
-
 // (1 - i k r) exp(i k (r - z)) / r^3 of one pair
 __device__ __forceinline__ Pair64 rs_pair(double dx, double dy, const RsArgs& a, const df z, const df z2,
                                           const double2* __restrict__ tab) {
@@ -256,7 +240,7 @@ __device__ __forceinline__ Pair64 rs_pair(double dx, double dy, const RsArgs& a,
     const df g = df_fast_two_sum(g0, rc * ((fmaf(-g0, t1.hi, rho.hi) + rho.lo) - g0 * t1.lo));
     // one Newton step in FP64 on d (2 z + d) = rho^2 (slope 2 r)
     const double yd = wide(yf);
-    const double d1 = g.hi > 1e-30f ? wide_sum(g.hi, g.lo) : 0.0;
+    const double d1 = dfr_to_double(dfr(g.hi, g.lo), 0);
     const double d = fma(fma(-d1, fma(2.0, a.z, d1), rho2), wide(0.5f * yf), d1);
     const double r = a.z + d;
     const double e = fma(-r, yd, 1.0);
@@ -265,12 +249,16 @@ __device__ __forceinline__ Pair64 rs_pair(double dx, double dy, const RsArgs& a,
     constexpr double magic = 3298534883328.0;   // 1.5 2^41: spacing 2^-11
     const double n = fma(d, a.il, magic);
     const double2 T = tab[__double2loint(n) & (kFine - 1)];
-    const double th = fma(d, a.il, magic - n) * 6.283185307179586477;
-    const float tf = narrow(th), hf = tf * tf;
-    const double h = th * th;
-    const double sn = th + wide(tf * hf * fmaf(hf, 8.3333333e-3f, -0.16666667f));
-    const double c1 = fma(h, -0.5, wide(hf * hf * fmaf(hf, -1.3888889e-3f, 4.1666667e-2f)));
-    const double cr = fma(T.x, c1, fma(-T.y, sn, T.x)), ci = fma(T.y, c1, fma(T.x, sn, T.y));
+    // exp(i theta) - 1 as a double-float (2^-46 of it is 2^-55)
+    const dfr dl = dfr_split(fma(d, a.il, magic - n), 0);
+    const df th = df_mul({dl.hi, dl.lo}, {6.2831855f, -1.7484555e-7f});   // 2 pi
+    const df h = df_mul(th, th);
+    const df sn = df_fast_two_sum(th.hi, fmaf(th.hi * h.hi, fmaf(h.hi, 8.3333333e-3f, -0.16666667f), th.lo));
+    const df c1 = df_fast_two_sum(-0.5f * h.hi, fmaf(h.hi * h.hi, fmaf(h.hi, -1.3888889e-3f, 4.1666667e-2f),
+                                                     -0.5f * h.lo));
+    const dfc C = cmul(CTraits<dfc>::make(dfr_split(T.x, 0), dfr_split(T.y, 0)),
+                       CTraits<dfc>::make(dfr(c1.hi, c1.lo), dfr(sn.hi, sn.lo)));
+    const double cr = T.x + dfr_to_double(C.x(), 0), ci = T.y + dfr_to_double(C.y(), 0);
     const double y2 = y * y, P = y2 * y, Q = y2 * a.k;
     return {fma(P, cr, Q * ci), fma(P, ci, -(Q * cr))};
 }
