@@ -128,7 +128,6 @@ nuasm_status nuasm_batch_create(nuasm_batch_t* out, const nuasm_batch_item_t* it
             const nuasm_batch_item_t& it = items[i];
             nuasm_plan_s view = *it.plan;   // no per-stage events inside a graph
             view.prof = false;
-            view.batched = true;
             if (it.type == 1) ce = chain_type1(&view, it.in, it.out, q);
             else if (it.type == 2) ce = chain_type2(&view, it.in, it.out, q);
             else ce = chain_type3(&view, it.dst, it.in, it.out, q);

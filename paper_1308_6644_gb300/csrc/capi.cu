@@ -257,7 +257,6 @@ cudaError_t nuasm::chain_type3(nuasm_plan_s* P, const nuasm_plan_s* Q, const voi
         nuasm_plan_s view = *Q;          // destination records over the source plan's window
         view.d.win = P->d.win;
         view.prof = false;
-        view.batched = P->batched;
         StageScope sc(P, NUASM_STAGE_INTERP, st);
         if ((e = launch_interp(&view, v, st)) != cudaSuccess) return e;
     }

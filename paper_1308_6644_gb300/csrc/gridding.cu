@@ -1609,7 +1609,7 @@ cudaError_t interp_impl(const nuasm_plan_s* P, void* v, cudaStream_t st) {
     cudaError_t e = set_smem(interp_kernel<S, WMAX, EXACT>, sm);
     if (e != cudaSuccess) return e;
     const int grid = P->d.interp_items ? P->n_interp_items : P->g.ntiles;
-    e = launch_chained(launch_early(P), interp_kernel<S, WMAX, EXACT>, dim3(grid), dim3(kInterpThreads), sm, st,
+    e = launch_chained(launch_early(P, st), interp_kernel<S, WMAX, EXACT>, dim3(grid), dim3(kInterpThreads), sm, st,
                        static_cast<const typename RecOf<S>::type*>(P->d.rec), P->d.tile_off, P->d.tile_home,
                        P->d.tile_order, static_cast<const int4*>(P->d.interp_items), static_cast<const V*>(P->d.win),
                        static_cast<V*>(v), a, taps_arg<S>(P));

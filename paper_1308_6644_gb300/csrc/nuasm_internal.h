@@ -107,7 +107,6 @@ struct nuasm_plan_s {
     int64_t nrec = 0;
     bool has_w = false;
     bool f64 = false;
-    bool batched = false;       // a view recorded into a batch
     double rc = 0.0;            // z / (2 lambda)
     int texp[3] = {0, 0, 0};    // double-float FFT passes: power of two taken out of type t's tables
     int nonsep_mode = 0;        // ASM non-separable phase: 0 none, 1 plain, 2 double-float
@@ -252,10 +251,17 @@ inline bool fft_double_float(const nuasm_plan_s* P) { return fft_double_float(P-
 // 37.3).  At N' = 2048 the early CTAs cost as much as they hide (jittered points
 // 106 -> 97 us, graded ones 107 -> 113); from N' = 4096 on they must not run
 // early: the column passes there write with bulk tensor stores, which the early
-// kernel's wait does not cover (the next pass read stale values).  Batches
-// overlap whole planes instead (709 -> 727 us for 12 planes with early launches),
-// and FP64 chains gained 5% at N = 32 and 512 and lost as much at N = 128 and 256.
-inline bool launch_early(const nuasm_plan_s* P) { return !P->f64 && P->g.np <= 1024 && !P->batched; }
+// kernel's wait does not cover (the next pass read stale values).  Chains recorded
+// into a graph (batches too) don't: a replayed graph has smaller gaps, and early
+// launches in it cost more than they hide (solves replayed from a graph, without ->
+// with: N = 256 weighted type 1 24.7 -> 29.9 us, N = 256 type 2 19.0 -> 21.9, N = 512
+// type 1 43.0 -> 45.9, N = 32 15.4 -> 13.3; 12 planes in a batch 709 -> 727).  FP64
+// chains gained 5% at N = 32 and 512 and lost as much at N = 128 and 256.
+inline bool launch_early(const nuasm_plan_s* P, cudaStream_t st) {
+    cudaStreamCaptureStatus recording;
+    return !P->f64 && P->g.np <= 1024 && cudaStreamIsCapturing(st, &recording) == cudaSuccess &&
+           recording == cudaStreamCaptureStatusNone;
+}
 
 // The exponents of a solve's double-float data, behind bufB's elements: word 0
 // the solve's (types 1 and 3: set by the spreading; type 2: by the row pass),

@@ -1138,16 +1138,16 @@ cudaError_t launch_row(const nuasm_plan_s* P, int type, cudaStream_t st) {
     cudaError_t e;
     if (type == 1) {
         if ((e = set_smem(row_t1_kernel<V, LOGNP>, C1::smem())) != cudaSuccess) return e;
-        e = launch_chained(launch_early(P), row_t1_kernel<V, LOGNP>, dim3(C1::NP / C1::ROWS), dim3(C1::P), C1::smem(), st,
+        e = launch_chained(launch_early(P, st), row_t1_kernel<V, LOGNP>, dim3(C1::NP / C1::ROWS), dim3(C1::P), C1::smem(), st,
                            static_cast<const M*>(P->d.bufA), static_cast<M*>(P->d.bufB),
                            static_cast<const M*>(P->d.t1x), static_cast<const M*>(P->d.t1y), s, tw, a);
     } else if (type == 3) {
         if ((e = set_smem(row_t3_kernel<V, LOGNP>, C3::smem())) != cudaSuccess) return e;
-        e = launch_chained(launch_early(P), row_t3_kernel<V, LOGNP>, dim3(C3::NP / C3::ROWS), dim3(C3::P), C3::smem(), st, static_cast<M*>(P->d.bufA),
+        e = launch_chained(launch_early(P, st), row_t3_kernel<V, LOGNP>, dim3(C3::NP / C3::ROWS), dim3(C3::P), C3::smem(), st, static_cast<M*>(P->d.bufA),
                            static_cast<const M*>(P->d.t3x), static_cast<const M*>(P->d.t3y), s, tw, a);
     } else {
         if ((e = set_smem(row_t2_kernel<V, LOGNP>, C2::smem())) != cudaSuccess) return e;
-        e = launch_chained(launch_early(P), row_t2_kernel<V, LOGNP>, dim3(C2::NP / C2::ROWS), dim3(C2::P), C2::smem(), st,
+        e = launch_chained(launch_early(P, st), row_t2_kernel<V, LOGNP>, dim3(C2::NP / C2::ROWS), dim3(C2::P), C2::smem(), st,
                            static_cast<const M*>(P->d.bufB), static_cast<M*>(P->d.bufA),
                            static_cast<const M*>(P->d.t2x), static_cast<const M*>(P->d.t2y), s, tw, a);
     }
@@ -1173,7 +1173,7 @@ cudaError_t launch_col(const nuasm_plan_s* P, const void* src, void* dst, int nc
     if constexpr (MODE == COL_FWD) {   // first kernel of the type-2 chain
         col_kernel<V, LOGNP, MODE><<<grid, Cf::P, sm, st>>>(static_cast<const MS*>(src), static_cast<MD*>(dst), tw, a);
     } else {
-        e = launch_chained(launch_early(P), col_kernel<V, LOGNP, MODE>, grid, dim3(Cf::P), sm, st, static_cast<const MS*>(src),
+        e = launch_chained(launch_early(P, st), col_kernel<V, LOGNP, MODE>, grid, dim3(Cf::P), sm, st, static_cast<const MS*>(src),
                            static_cast<MD*>(dst), tw, a);
         if (e != cudaSuccess) return e;
     }
@@ -1196,7 +1196,7 @@ cudaError_t launch_col2(const nuasm_plan_s* P, const void* src, void* dst, int n
         col2_kernel<LOGNP, MODE><<<grid, block, Cf::SMEM, st>>>(static_cast<const float2*>(src),
                                                                 static_cast<float2*>(dst), tw, a);
     } else {
-        e = launch_chained(launch_early(P), col2_kernel<LOGNP, MODE>, grid, block, Cf::SMEM, st, static_cast<const float2*>(src),
+        e = launch_chained(launch_early(P, st), col2_kernel<LOGNP, MODE>, grid, block, Cf::SMEM, st, static_cast<const float2*>(src),
                            static_cast<float2*>(dst), tw, a);
         if (e != cudaSuccess) return e;
     }
@@ -1268,7 +1268,7 @@ cudaError_t launch_col_tma(const nuasm_plan_s* P, const void* src, void* dst, in
                                                                  static_cast<const float2*>(P->d.tw), a, nfull,
                                                                  nitems, nboxes, nz, P->d.err);
         } else {
-            e = launch_chained(launch_early(P), col_tma_kernel<LOGNP, MODE>, dim3(grid), dim3(Cf::P), sm, st, map, omap, omap_h,
+            e = launch_chained(launch_early(P, st), col_tma_kernel<LOGNP, MODE>, dim3(grid), dim3(Cf::P), sm, st, map, omap, omap_h,
                                static_cast<float2*>(dst), static_cast<const float2*>(P->d.tw), a, nfull, nitems,
                                nboxes, nz, P->d.err);
             if (e != cudaSuccess) return e;
