@@ -532,7 +532,7 @@ __global__ void __launch_bounds__(NT, NUASM_SPREAD_FIXED_MINB * 256 / NT) spread
     const int x0 = tx * T, y0 = ty * T;
     const float L = load[tile];
     const bool crowded = L > kMaxLoad;
-    for (int i = threadIdx.x; i < (crowded ? 4 : 2) * TT; i += NT) are[i] = 0;
+    for (int i = threadIdx.x; i < 2 * TT; i += NT) are[i] = 0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int half = T / 2;   // cells are folded and written in pairs
     // cells (gx, gy) and (gx + 1, gy) of the window: W, x0 and xx are even, so both lie in it or neither
@@ -629,10 +629,11 @@ __global__ void __launch_bounds__(NT, NUASM_SPREAD_FIXED_MINB * 256 / NT) spread
         q = fixed ? bound * pre * scale : 1.f;
     };
     int step = BATCH;
+    fetch(b, e);   // its loads do not wait for the tile's load
     if (!crowded) {
         unsigned top = 0;   // bits of the largest |re| or |im| (an infinity or a NaN tops every number)
         for (int i0 = b; i0 < e; i0 += BATCH) {
-            fetch(i0, e);
+            if (i0 != b) fetch(i0, e);
 #pragma unroll
             for (int k = 0; k < RPB; ++k)
                 top = max(top, max(__float_as_uint(val[k].x) & 0x7fffffffu, __float_as_uint(val[k].y) & 0x7fffffffu));
@@ -645,8 +646,9 @@ __global__ void __launch_bounds__(NT, NUASM_SPREAD_FIXED_MINB * 256 / NT) spread
         const float bound = __uint_as_float(top) * L;   // of every cell's sum
         empty = top == 0;
         if (!empty) set_quantum(bound, 1.00390625f / 2147483648.f);
-    } else if (T <= 32) {
-        step = BATCH / 2;   // folds are cheap on small tiles: batches of half the records, half the quantum
+    } else {
+        for (int i = threadIdx.x; i < 2 * TT; i += NT) tre[i] = 0.f;
+        if (T <= 32) step = BATCH / 2;   // folds are cheap on small tiles: batches of half the records, half the quantum
     }
     for (int i0 = empty ? e : b; i0 < e; i0 += step) {
         const int end = crowded ? min(e, i0 + step) : e;
