@@ -219,7 +219,10 @@ def kernel_of_stage(stage: str, info: dict, f64: bool) -> str:
     """Name of the kernel a stage launches for this geometry (as ncu lists it)."""
     lognp = int(np.log2(info["n_pad"]))
     v, s = ("double2", "double") if f64 else ("float2", "float")
-    rv = "dfc" if f64 and lognp >= 9 else v   # FP64 FFT passes from N' = 512 up: double-float
+    # FP64 FFT passes: double-float, below N' = 512 where the kernel's width (a built
+    # plan's tolerance from 1e-12 up) allows it
+    plan = "records" in info
+    rv = "dfc" if f64 and (lognp >= 9 or (plan and info.get("double_float"))) else v
     w = info["kernel_width"]
     if f64:
         tap = f"double, {w}, true" if w in (11, 13) else f"double, {8 if w <= 8 else (16 if w <= 16 else 26)}, false"
@@ -235,7 +238,7 @@ def kernel_of_stage(stage: str, info: dict, f64: bool) -> str:
         spread = f"spread_df_kernel<{w}>"
     elif f64:
         spread = f"spread_private_kernel<{tap}>" if tile <= 16 else f"spread_kernel<{tap}>"
-    elif tile <= 32:
+    elif tile <= 32 and not plan:
         spread = f"spread_private_kernel<{tap}>"
     else:
         spread = (f"spread_fixed_kernel<{w}, true, 2>" if 4 <= w <= 8 else
@@ -621,7 +624,7 @@ def run_ours(args):
                        "kernel": args.kernel, "tol": params.tol or (1e-12 if f64 else 1e-6),
                        "kernel_width": info["kernel_width"], "tile": info["tile"],
                        "precision": ("complex128 data; double-float (pairs of FP32) arithmetic in the gridding "
-                                     "and the FFT passes from N' = 512 up, FP64 elsewhere" if f64
+                                     "and the FFT passes, FP64 where the tolerance is below theirs" if f64
                                      else "complex64 + FP64-derived phase"),
                        "l2": "flushed (256 MB write) before every step", "plan_s": round(plan_s, 3),
                        "autotuned": tuned,

@@ -85,9 +85,11 @@ typedef enum {
                                      compensated (double-float) FP32 arithmetic */
     NUASM_PREC_F64 = 1            /* complex128 data; FP64 arithmetic, except that gridding at the
                                      kernel widths of the FP64 tolerances (see
-                                     nuasm_plan_info_t.double_float) and the FFT passes of planes
-                                     with N' >= 512 run in double-float arithmetic (pairs of FP32
-                                     values, about 47 significant bits); results within 1e-10
+                                     nuasm_plan_info_t.double_float) and the FFT passes (below N' =
+                                     512 at tolerances from 1e-12 up) run in double-float
+                                     arithmetic (pairs of FP32 values, about 47 significant bits,
+                                     at one power-of-two scale per solve: values below 2^-100 of
+                                     the largest input count as zero); results within 1e-10
                                      (rel-L2) of exact FP64 evaluation */
 } nuasm_prec;
 
