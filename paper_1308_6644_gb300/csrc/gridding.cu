@@ -495,9 +495,12 @@ __global__ void __launch_bounds__(256, sizeof(S) == 4 ? NUASM_SPREAD_MINB : 1) s
 #ifndef NUASM_SPREAD_FIXED_MINB
 #define NUASM_SPREAD_FIXED_MINB 4   // CTAs of 256 threads per SM the register budget is set for
 #endif
+// kernels wider than 8 taps hold more weights: 64 registers a thread spilled (Gaussian
+// w = 13, 4M clustered points, spreading about 930 us with four CTAs, 798 with three)
+constexpr int fixed_minb(int wmax) { return wmax <= 8 ? NUASM_SPREAD_FIXED_MINB : 3; }
 constexpr float kMaxLoad = 256.f;
 template <int WMAX, bool EXACT, int RPB, int NT>
-__global__ void __launch_bounds__(NT, NUASM_SPREAD_FIXED_MINB * 256 / NT) spread_fixed_kernel(const RecF* __restrict__ rec,
+__global__ void __launch_bounds__(NT, fixed_minb(WMAX) * 256 / NT) spread_fixed_kernel(const RecF* __restrict__ rec,
                                                                       const int* __restrict__ off,
                                                                       const double* __restrict__ wpt,
                                                                       const int4* __restrict__ order,
