@@ -466,14 +466,26 @@ __global__ void __launch_bounds__(256, sizeof(S) == 4 ? NUASM_SPREAD_MINB : 1) s
 // native.  A contribution v wx wy is rounded to a multiple of the quantum q and
 // added to int32 planes, q such that no cell's sum leaves the range:
 //  * the plan knows each tile's load L, the largest sum of wx wy over its
-//    records at one cell (tile_load_kernel), so with V the largest |re| or |im|
-//    of the CTA's values (weights included) q = V L 2^-31 (1 + 2^-8) serves all
-//    of them at once: one pass for V, one that adds, one write of the window
-//    (the 2^-8 is room for the roundings of up to 2^24 contributions);
-//  * where records crowd a few cells (L > kMaxLoad; the error of a cell is about
-//    L 1e-9 of its value, that of FP32 sums of the same records sqrt(L) 7e-8),
-//    they go in batches with q = S 2^-30, S = sum(|re| + |im|) of the batch, each
-//    folded into FP32 totals (tot += q acc) and cleared.
+//    records at one cell (tile_load_kernel).  With V the largest and S the sum of
+//    max(|re|, |im|) over the CTA's values (weights included), no cell exceeds B =
+//    min(V L, S), and q = B 2^-31 (1 + 2^-8) serves all of them at once: one pass
+//    for V and S, one that adds, one write of the window (the 2^-8 is room for the
+//    roundings of up to 2^24 contributions).  A contribution is off by up to q/2,
+//    so the CTA's error is 6e-10 B of the values' root mean square: small where V
+//    is not far above the mean.
+//  * where it is (a bright sample among faint ones: V L > max_load times the mean
+//    of max(|re|, |im|)) or records crowd a few cells (L > max_load, which is the
+//    same at best), the records go in batches, each with its own V, S and q: one
+//    sample of 1 among samples of 1e-3 in a tile of load 111 is off by 8e-8 (float
+//    sums of the same records: 1e-7; one quantum for all of them: 1.5e-5).  With
+//    max_load and the batch below the error is that of float sums to within a
+//    factor of two, or less, over loads of 5 to 280 and values of one magnitude,
+//    uniform, normal and log-normal ones and bright samples 10 to 10^4 above the
+//    rest, and no more than theirs up to loads of 60 (3e-8 to 1e-7).  Dense tiles
+//    that hold a bright sample take longer for it (4M even points at N = 1024 and
+//    2048: 202 -> 300 and 250 us), crowded ones than with FP32 totals in shared
+//    memory and q = sum(|re| + |im|) 2^-30 (800,000 points at N = 512 70 -> 85 us, 4M
+//    in a few tiles 18.9 -> 19.8 ms; off by 2e-7, not 4e-7).
 // Zero values are skipped; values so small that q would underflow (the skirts of
 // a Gaussian beam) are taken times 2^64 and back; values that are not finite add
 // with float atomics, so they propagate.
@@ -498,7 +510,10 @@ __global__ void __launch_bounds__(256, sizeof(S) == 4 ? NUASM_SPREAD_MINB : 1) s
 // kernels wider than 8 taps hold more weights: 64 registers a thread spilled (Gaussian
 // w = 13, 4M clustered points, spreading about 930 us with four CTAs, 798 with three)
 constexpr int fixed_minb(int wmax) { return wmax <= 8 ? NUASM_SPREAD_FIXED_MINB : 3; }
-constexpr float kMaxLoad = 256.f;
+// tiles of side 64: batches of 512 records (1e-7 to 3e-7 against 2e-7 to 8e-7 of the
+// 512-record batches of q = sum(|re| + |im|) 2^-30 that they had for every tile);
+// sides 16 and 32, whose planes fold in a fraction of the time: 256
+__host__ __device__ constexpr float max_load(int T) { return T > 32 ? 256.f : 128.f; }
 template <int WMAX, bool EXACT, int RPB, int NT>
 __global__ void __launch_bounds__(NT, fixed_minb(WMAX) * 256 / NT) spread_fixed_kernel(const RecF* __restrict__ rec,
                                                                       const int* __restrict__ off,
@@ -510,7 +525,7 @@ __global__ void __launch_bounds__(NT, fixed_minb(WMAX) * 256 / NT) spread_fixed_
                                                                       const KernelPoly kp,
                                                                       const int4* __restrict__ items) {
     extern __shared__ unsigned char smem_raw[];
-    __shared__ unsigned red[NT / 32];
+    __shared__ float2 red[NT / 32];
     int tile, b, e;
     bool chunked = false;
     if (items) {   // a chunk of a tile's records: several CTAs add into the tile (window cleared)
@@ -528,23 +543,21 @@ __global__ void __launch_bounds__(NT, fixed_minb(WMAX) * 256 / NT) spread_fixed_
     const int T = a.T, w = EXACT ? WMAX : a.w, TS = plane_stride(T, a.skew_of(tile)), TT = T * TS;
     int* are = reinterpret_cast<int*>(smem_raw);
     int* aim = are + TT;
-    float* tre = reinterpret_cast<float*>(aim + TT);   // totals: only where the plan has a crowded tile
-    float* tim = tre + TT;
     pdl_allow_next();
     const int ty = tile / a.ntx, tx = tile - ty * a.ntx;
     const int x0 = tx * T, y0 = ty * T;
     const float L = load[tile];
-    const bool crowded = L > kMaxLoad;
     for (int i = threadIdx.x; i < 2 * TT; i += NT) are[i] = 0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int half = T / 2;   // cells are folded and written in pairs
     // cells (gx, gy) and (gx + 1, gy) of the window: W, x0 and xx are even, so both lie in it or neither
+    bool add = chunked;   // or the CTA has stored its tile's cells (each thread its own) and adds to them from then on
     auto emit = [&](int gx, int gy, float4 v) {
         if (gy >= a.W || gx >= a.W ||
             !NUASM_IN_RANGE(gy * (long long)a.Wp + gx + 1, (long long)a.W * a.Wp, dbg::kSpreadWindow))
             return;
         float2* p = &win[size_t(gy) * a.Wp + gx];
-        if (!chunked) {
+        if (!add) {
             *reinterpret_cast<float4*>(p) = v;
         } else {
             if (v.x != 0.f || v.y != 0.f) {
@@ -622,102 +635,115 @@ __global__ void __launch_bounds__(NT, fixed_minb(WMAX) * 256 / NT) spread_fixed_
         }
     };
     constexpr int BATCH = RPB * NT;
-    // one quantum for all records (fixed, q), or one per batch
-    bool fixed = false, empty = false;
+    bool fixed = false;
     float q = 1.f, pre = 1.f, post = 1.f;   // the planes hold the values times pre in units of q; post = 1 / pre
-    auto set_quantum = [&](float bound, float scale) {
+    auto set_quantum = [&](float bound) {
         fixed = bound <= 3e38f;
         pre = fixed && bound < 1e-20f ? 18446744073709551616.f : 1.f;
         post = fixed && bound < 1e-20f ? 5.42101086242752217e-20f : 1.f;
-        q = fixed ? bound * pre * scale : 1.f;
+        q = fixed ? bound * pre * (1.00390625f / 2147483648.f) : 1.f;
     };
-    int step = BATCH;
-    fetch(b, e);   // its loads do not wait for the tile's load
-    if (!crowded) {
-        unsigned top = 0;   // bits of the largest |re| or |im| (an infinity or a NaN tops every number)
-        for (int i0 = b; i0 < e; i0 += BATCH) {
-            if (i0 != b) fetch(i0, e);
+    // the largest (x) and the sum (y) of max(|re|, |im|) over values: of the fetched
+    // records added to a thread's v, and of the CTA's threads (an infinity or a NaN,
+    // whose bits top every number's, goes into both)
+    auto measure = [&](float2 v) {
 #pragma unroll
-            for (int k = 0; k < RPB; ++k)
-                top = max(top, max(__float_as_uint(val[k].x) & 0x7fffffffu, __float_as_uint(val[k].y) & 0x7fffffffu));
+        for (int k = 0; k < RPB; ++k) {
+            const unsigned t = max(__float_as_uint(val[k].x) & 0x7fffffffu, __float_as_uint(val[k].y) & 0x7fffffffu);
+            v = make_float2(__uint_as_float(max(__float_as_uint(v.x), t)), v.y + __uint_as_float(t));
         }
-        top = __reduce_max_sync(0xffffffffu, top);
-        if (lane == 0) red[warp] = top;
-        __syncthreads();   // also orders the clearing above
+        return v;
+    };
+    auto over_cta = [&](float2 v) {
+        unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(v.x));
 #pragma unroll
-        for (int k = 0; k < NT / 32; ++k) top = max(top, red[k]);
-        const float bound = __uint_as_float(top) * L;   // of every cell's sum
-        empty = top == 0;
-        if (!empty) set_quantum(bound, 1.00390625f / 2147483648.f);
-    } else {
-        for (int i = threadIdx.x; i < 2 * TT; i += NT) tre[i] = 0.f;
-        if (T <= 32) step = BATCH / 2;   // folds are cheap on small tiles: batches of half the records, half the quantum
-    }
-    for (int i0 = empty ? e : b; i0 < e; i0 += step) {
-        const int end = crowded ? min(e, i0 + step) : e;
-        if (crowded || e - b > BATCH) fetch(i0, end);   // else the first pass left the records in registers
-        if (crowded) {
-            float part = 0.f;
-#pragma unroll
-            for (int k = 0; k < RPB; ++k) part += fabsf(val[k].x) + fabsf(val[k].y);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-            __syncthreads();   // the clearing above, or the previous batch's fold and its reads of red, are done
-            if (lane == 0) red[warp] = __float_as_uint(part);
-            __syncthreads();
-            float S = 0.f;
-#pragma unroll
-            for (int k = 0; k < NT / 32; ++k) S += __uint_as_float(red[k]);
-            if (S == 0.f) continue;   // every value of the batch is zero (uniform)
-            set_quantum(S, 1.f / 1073741824.f);
-        }
-        add_taps(i0, end, pre, 1.f / q, fixed);
-        if (!crowded) continue;
-        // fold the batch into the totals and clear the planes
+        for (int o = 16; o > 0; o >>= 1) v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+        if (lane == 0) red[warp] = make_float2(__uint_as_float(top), v.y);
         __syncthreads();
+        v.y = 0.f;
+#pragma unroll
+        for (int k = 0; k < NT / 32; ++k) {
+            top = max(top, __float_as_uint(red[k].x));
+            v.y += red[k].y;
+        }
+        v.x = __uint_as_float(top);
+        return v;
+    };
+    auto bound_of = [&](float2 v) { return v.y < v.x * L ? v.y : v.x * L; };   // of every cell's sum
+    // f(cell in the planes, window column and row) of the tile's pairs of cells: a thread's are its own
+    auto cells = [&](auto f) {
         for (int i = threadIdx.x; i < T * half; i += NT) {
-            const int yy = i / half, xx = 2 * (i - yy * half), j = yy * TS + xx;
-            int2* pr = reinterpret_cast<int2*>(&are[j]);
-            int2* pm = reinterpret_cast<int2*>(&aim[j]);
-            float2* pa = reinterpret_cast<float2*>(&tre[j]);
-            float2* pb = reinterpret_cast<float2*>(&tim[j]);
-            const int2 rr = *pr, mm = *pm;
-            const float2 tr = *pa, ti = *pb;
-            if (fixed) {
-                *pa = make_float2(fmaf(float(rr.x) * q, post, tr.x), fmaf(float(rr.y) * q, post, tr.y));
-                *pb = make_float2(fmaf(float(mm.x) * q, post, ti.x), fmaf(float(mm.y) * q, post, ti.y));
-            } else {
-                *pa = make_float2(tr.x + __int_as_float(rr.x), tr.y + __int_as_float(rr.y));
-                *pb = make_float2(ti.x + __int_as_float(mm.x), ti.y + __int_as_float(mm.y));
-            }
-            *pr = make_int2(0, 0);
-            *pm = make_int2(0, 0);
+            const int yy = i / half, xx = 2 * (i - yy * half);
+            f(yy * TS + xx, x0 + xx, y0 + yy);
+        }
+    };
+    auto sums = [&](int j) {
+        const int2 rr = *reinterpret_cast<const int2*>(&are[j]), mm = *reinterpret_cast<const int2*>(&aim[j]);
+        if (fixed)
+            return make_float4(float(rr.x) * q * post, float(mm.x) * q * post, float(rr.y) * q * post,
+                               float(mm.y) * q * post);
+        return make_float4(__int_as_float(rr.x), __int_as_float(mm.x), __int_as_float(rr.y), __int_as_float(mm.y));
+    };
+    const int n = e - b, batch = T > 32 ? 512 : 256;
+    bool one = n <= batch;   // one quantum for all records, or one per batch
+    fetch(b, e);   // its loads do not wait for the tile's load
+    if (one || L <= max_load(T)) {
+        float2 v = measure(make_float2(0.f, 0.f));
+        for (int i0 = b + BATCH; i0 < e; i0 += BATCH) {
+            fetch(i0, e);
+            v = measure(v);
+        }
+        v = over_cta(v);   // its barrier also orders the clearing above
+        one = one || v.x * L * float(n) <= max_load(T) * v.y;
+        if (v.x == 0.f) {   // every value is zero: the window gets the cleared planes
+            one = true;
+            e = b;
+        } else if (one) {
+            set_quantum(bound_of(v));
         }
     }
-    __syncthreads();
-    // the window's cells: the planes in units of q, the planes as floats, or the totals
-    const int* ore = crowded ? reinterpret_cast<const int*>(tre) : are;
-    const int* oim = crowded ? reinterpret_cast<const int*>(tim) : aim;
-    const bool ints = fixed && !crowded;
-    for (int i = threadIdx.x; i < T * half; i += NT) {
-        const int yy = i / half, xx = 2 * (i - yy * half), j = yy * TS + xx;
-        const int2 rr = *reinterpret_cast<const int2*>(&ore[j]), mm = *reinterpret_cast<const int2*>(&oim[j]);
-        float4 v = make_float4(__int_as_float(rr.x), __int_as_float(mm.x), __int_as_float(rr.y), __int_as_float(mm.y));
-        if (ints)
-            v = make_float4(float(rr.x) * q * post, float(mm.x) * q * post, float(rr.y) * q * post,
-                            float(mm.y) * q * post);
-        emit(x0 + xx, y0 + yy, v);
+    if (one) {
+        for (int i0 = b; i0 < e; i0 += BATCH) {
+            if (n > BATCH) fetch(i0, e);   // else the first pass left the records in registers
+            add_taps(i0, e, pre, 1.f / q, fixed);
+        }
+        __syncthreads();
+        cells([&](int j, int gx, int gy) { emit(gx, gy, sums(j)); });
+        return;
+    }
+    // Batches add up in the window's cells: totals in shared memory were no faster on
+    // tiles of side 32 (83 and 85 us, 800,000 points crowded at N = 512) and cost a
+    // resident CTA at side 64.  This loop beside the other costs the tiles of one
+    // quantum 1.5% at side 64.
+    fetch(b, min(e, b + batch));
+    for (int i0 = b; i0 < e; i0 += batch) {
+        const int end = min(e, i0 + batch);
+        __syncthreads();   // the clearing above, or the previous batch's, and its reads of red, are done
+        const float2 v = over_cta(measure(make_float2(0.f, 0.f)));
+        const bool some = v.x != 0.f;
+        fixed = false;
+        if (some) {
+            set_quantum(bound_of(v));
+            add_taps(i0, end, pre, 1.f / q, fixed);
+        }
+        fetch(end, min(e, end + batch));   // the next batch's loads run under this one's fold
+        if (!some && (add || end < e)) continue;   // zeros (but the window is written once)
+        __syncthreads();
+        cells([&](int j, int gx, int gy) {
+            emit(gx, gy, sums(j));
+            *reinterpret_cast<int2*>(&are[j]) = make_int2(0, 0);
+            *reinterpret_cast<int2*>(&aim[j]) = make_int2(0, 0);
+        });
+        add = true;
     }
 }
 
 // Plan time (FP32): each tile's load, the largest sum over its records of wx wy
-// at one cell, rounded up, and the largest of all tiles' (bits, in *most).  Sums
-// in units of 2^-14 fit int32 for 2^17 records at one cell; tiles with more
+// at one cell, rounded up.  Sums in units of 2^-14 fit int32 for 2^17 records at one cell; tiles with more
 // records take their count.
 template <int WMAX, bool EXACT>
 __global__ void __launch_bounds__(256) tile_load_kernel(const RecF* __restrict__ rec, const int* __restrict__ off,
-                                                        GridArgs a, const KernelPoly kp, float* __restrict__ load,
-                                                        unsigned* __restrict__ most) {
+                                                        GridArgs a, const KernelPoly kp, float* __restrict__ load) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ int red[8];
     const int tile = blockIdx.x, b = off[tile], e = off[tile + 1];
@@ -755,9 +781,7 @@ __global__ void __launch_bounds__(256) tile_load_kernel(const RecF* __restrict__
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int k = 1; k < 8; ++k) top = max(top, red[k]);
-        const float v = count ? 1.0001f * float(e - b) : 1.0001f * (float(top) / 16384.f);
-        load[tile] = v;
-        atomicMax(most, __float_as_uint(v));
+        load[tile] = count ? 1.0001f * float(e - b) : 1.0001f * (float(top) / 16384.f);
     }
 }
 
@@ -1567,8 +1591,7 @@ cudaError_t spread_impl(const nuasm_plan_s* P, const void* c, cudaStream_t st) {
     if constexpr (sizeof(S) == 4) {
         auto fixed = [&](auto threads) -> cudaError_t {
             constexpr int RPB = NUASM_SPREAD_FIXED_RPB, NT = decltype(threads)::value;
-            // int32 planes, and totals where the plan has a crowded tile
-            const size_t sm = size_t(P->max_load > kMaxLoad ? 4 : 2) * a.T * plane_stride(a.T, a.max_skew) * sizeof(float);
+            const size_t sm = size_t(2) * a.T * plane_stride(a.T, a.max_skew) * sizeof(int);
             cudaError_t e = set_smem(spread_fixed_kernel<WMAX, EXACT, RPB, NT>, sm);
             if (e != cudaSuccess) return e;
             spread_fixed_kernel<WMAX, EXACT, RPB, NT><<<grid, NT, sm, st>>>(
@@ -1708,13 +1731,10 @@ template <bool SPREAD> cudaError_t gridding(const nuasm_plan_s* P, const void* i
     }
 }
 
-// Fill the plan's tile loads (FP32) and their maximum.
+// Fill the plan's tile loads (FP32).
 cudaError_t fill_tile_load(nuasm_plan_s* P, cudaStream_t st) {
     if (P->f64) return cudaSuccess;
     const GridArgs a = grid_args(P);
-    unsigned* most = reinterpret_cast<unsigned*>(P->d.tile_load + P->g.ntiles);
-    cudaError_t e = cudaMemsetAsync(most, 0, sizeof(unsigned), st);
-    if (e != cudaSuccess) return e;
     auto run = [&](auto tag) -> cudaError_t {
         using Tg = decltype(tag);
         auto kernel = tile_load_kernel<Tg::W, Tg::X>;
@@ -1722,20 +1742,17 @@ cudaError_t fill_tile_load(nuasm_plan_s* P, cudaStream_t st) {
         cudaError_t err = set_smem(kernel, sm);
         if (err != cudaSuccess) return err;
         kernel<<<P->g.ntiles, 256, sm, st>>>(static_cast<const RecF*>(P->d.rec), P->d.tile_off, a, P->poly,
-                                             P->d.tile_load, most);
+                                             P->d.tile_load);
         return cudaGetLastError();
     };
     switch (P->g.w) {
-        case 4: e = run(GTag<float, 4, true>{}); break;
-        case 5: e = run(GTag<float, 5, true>{}); break;
-        case 6: e = run(GTag<float, 6, true>{}); break;
-        case 7: e = run(GTag<float, 7, true>{}); break;
-        case 8: e = run(GTag<float, 8, true>{}); break;
-        default: e = P->g.w <= 16 ? run(GTag<float, 16, false>{}) : run(GTag<float, kPolyMaxW, false>{});
+        case 4: return run(GTag<float, 4, true>{});
+        case 5: return run(GTag<float, 5, true>{});
+        case 6: return run(GTag<float, 6, true>{});
+        case 7: return run(GTag<float, 7, true>{});
+        case 8: return run(GTag<float, 8, true>{});
+        default: return P->g.w <= 16 ? run(GTag<float, 16, false>{}) : run(GTag<float, kPolyMaxW, false>{});
     }
-    if (e != cudaSuccess) return e;
-    e = cudaMemcpyAsync(&P->max_load, most, sizeof(float), cudaMemcpyDeviceToHost, st);
-    return e != cudaSuccess ? e : cudaStreamSynchronize(st);
 }
 
 }  // namespace
@@ -1773,8 +1790,8 @@ cudaError_t make_tile_order(nuasm_plan_s* P, cudaStream_t st) {
     std::stable_sort(order.begin(), order.end(),
                      [&](int a, int b) { return off[a + 1] - off[a] > off[b + 1] - off[b]; });
     P->max_tile_rec = off[order[0] + 1] - off[order[0]];
-    // the tiles with their record ranges, then their loads and the largest (fill_tile_load)
-    const size_t bytes = sizeof(int4) * size_t(nt) + sizeof(float) * (size_t(nt) + 1);
+    // the tiles with their record ranges, then their loads (fill_tile_load)
+    const size_t bytes = (sizeof(int4) + sizeof(float)) * size_t(nt);
     if ((e = xmalloc(reinterpret_cast<void**>(&P->d.tile_order), bytes)) != cudaSuccess) return e;
     P->d.tile_load = reinterpret_cast<float*>(P->d.tile_order + nt);
     P->device_bytes += int64_t(bytes);

@@ -116,7 +116,6 @@ struct nuasm_plan_s {
     int n_interp_items = 0;     // entries of d.interp_items
     int n_spread_items = 0;     // entries of d.spread_items
     int max_tile_rec = 0;       // records of the fullest tile
-    float max_load = 0.f;       // FP32: largest of d.tile_load
     nuasm::KernelPoly poly{};   // kernel taps as polynomials (F32 gridding)
     nuasm::KernelPoly64 poly64{};   // the same in FP64 (F64 gridding)
     nuasm::KernelPolyDF poly64df{};   // poly64 as float pairs (F64 gridding in double-float arithmetic)
