@@ -54,6 +54,7 @@ struct RsArgs {
     double norm;               // 1 / (2 pi), likewise
     unsigned rho2_max;         // FP64: high word of the rho^2 from which on (or from 2^40 turns) a pair takes
                                // the direct formulas
+    float near;                // FP32: distance per axis up to which the phase is below 2^22 - 1 half-turns
     int64_t m1, m2;
 };
 
@@ -91,10 +92,67 @@ __device__ __forceinline__ void cluster_sum(V* part, int count, StoreF store) {
 // instruction for the two.  The phase is rounded where the correctly rounded
 // operations round it (r, r + z, the quotient, the product with 1/lambda), then
 // reduced to half-turns by additions of 1.5 2^23, whose low bit is the sign of
-// the half-turn; sine and cosine are polynomials on [-1/4, 1/4] turn
-// (Chebyshev-node fits, 1.5e-7 at most in FP32).  43 FP32 operations and three
-// MUFU ones per pair of points; the FP32 pipe bounds it (78% of its rate at
-// 65536 x 65536).
+// the half-turn.  That holds below 2^22 half-turns (2^21 wavelengths, where an FP32
+// phase is down to half a turn); from there on only a pair's magnitude means
+// anything, and its phase is taken mod 2 first, so that the sine and cosine stay
+// within 1.  A warp asks once per 32 sources whether any may lie that far from the
+// CTA's points and takes the reduced loop if so.  Sine and cosine are polynomials
+// on [-1/4, 1/4] turn (Chebyshev-node fits, 1.5e-7 at most in FP32).  43 FP32
+// operations and three MUFU ones per pair of points; the FP32 pipe bounds it (78%
+// of its rate at 65536 x 65536).
+struct Consts32 { float2 z, z2, il2, zf2, zk, nzk; };   // each in both halves; phases in half-turns
+struct Sums32 { float2 rr, ii, im; };                   // of re re, im im and of the imaginary part
+// one source's share for a lane's two points
+template <bool FAR>
+__device__ __forceinline__ void rs_pair32(float4 s, float4 v, float2 px, float2 py, const Consts32& k, Sums32& sum) {
+    const float2 one = f2_dup(1.f), none = f2_dup(-1.f), half = f2_dup(0.5f), magic = f2_dup(12582912.f);
+    const float2 dx = sub2(px, make_float2(s.x, s.y)), dy = sub2(py, make_float2(s.z, s.w));
+    const float2 rho2 = fma2(dx, dx, mul2(dy, dy));
+    const float2 d2 = add2(rho2, k.z2);
+    // r = sqrt(d2) and d = rho^2 / (r + z), each an approximation and one
+    // step with the exact remainder (Markstein)
+    const float2 y = make_float2(rsqrt_fast(d2.x), rsqrt_fast(d2.y));
+    const float2 r0 = mul2(d2, y);
+    const float2 r = fma2(fma2(mul2(r0, none), r0, d2), mul2(y, half), r0);
+    const float2 t = add2(r, k.z);
+    const float2 rc = make_float2(rcp_fast(t.x), rcp_fast(t.y));
+    const float2 g = mul2(rho2, rc);
+    const float2 d = fma2(fma2(mul2(g, none), t, rho2), rc, g);
+    // half-turns: the nearest integer n and the rest
+    float2 ph = fma2(d, k.il2, k.zf2);
+    if (FAR) ph = make_float2(fmaf(-2.f, rintf(0.5f * ph.x), ph.x), fmaf(-2.f, rintf(0.5f * ph.y), ph.y));
+    const float2 kb = add2(ph, magic);
+    const float2 x = sub2(ph, sub2(kb, magic));
+    const float2 u = mul2(x, x);
+    float2 cs = fma2(f2_dup(-0.024395931512117386f), u, f2_dup(0.23493707180023193f));
+    cs = fma2(cs, u, f2_dup(-1.335211992263794f));
+    cs = fma2(cs, u, f2_dup(4.058709144592285f));
+    cs = fma2(cs, u, f2_dup(-4.934802055358887f));
+    cs = fma2(cs, u, one);
+    float2 sn = fma2(f2_dup(0.07765591144561768f), u, f2_dup(-0.5982903838157654f));
+    sn = fma2(sn, u, f2_dup(2.550077438354492f));
+    sn = fma2(sn, u, f2_dup(-5.167710304260254f));
+    sn = mul2(x, fma2(sn, u, f2_dup(3.1415927410125732f)));
+    // +- 1 / r^2, the sign (-1)^n
+    float2 w = make_float2(rcp_fast(d2.x), rcp_fast(d2.y));
+    w.x = __uint_as_float(__float_as_uint(w.x) ^ (__float_as_uint(kb.x) << 31));
+    w.y = __uint_as_float(__float_as_uint(w.y) ^ (__float_as_uint(kb.y) << 31));
+    // z/r^3 (1 - i k r)(cs + i sn) = (z/r^3 cs + z k/r^2 sn) + i (z/r^3 sn - z k/r^2 cs)
+    const float2 A = mul2(mul2(w, make_float2(fabsf(w.x), fabsf(w.y))), mul2(r, k.z));
+    const float2 kre = fma2(A, cs, mul2(mul2(w, k.zk), sn));
+    const float2 kim = fma2(A, sn, mul2(mul2(w, k.nzk), cs));
+    const float2 vr = make_float2(v.x, v.y), vi = make_float2(v.z, v.w);
+    sum.rr = fma2(vr, kre, sum.rr);
+    sum.ii = fma2(vi, kim, sum.ii);
+    sum.im = fma2(vr, kim, fma2(vi, kre, sum.im));
+}
+// (out of line: a second copy of the loop beside the first made that one 2% slower)
+__device__ __noinline__ Sums32 rs_far32(const float4* pos, const float4* val, int count, float2 px, float2 py,
+                                        Consts32 k, Sums32 sum) {
+#pragma unroll 1
+    for (int q = 0; q < count; ++q) rs_pair32<true>(pos[q], val[q], px, py, k, sum);
+    return sum;
+}
 constexpr int kPts32 = 64;
 __global__ void __launch_bounds__(kThreads, 3) rs_f32_kernel(const double* __restrict__ x1, const double* __restrict__ y1,
                                                           const float2* __restrict__ c, const double* __restrict__ area,
@@ -106,18 +164,24 @@ __global__ void __launch_bounds__(kThreads, 3) rs_f32_kernel(const double* __res
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int rank = int(blockIdx.x) % split;
     const int64_t p0 = int64_t(blockIdx.x / split) * kPts32;
-    auto coord = [&](const double* v, double o, int64_t i) { return i < a.m2 ? float((v[i] + o) * a.scale) : 0.f; };
+    // (lanes without a point of their own take the last one, which keeps them near the others)
+    auto coord = [&](const double* v, double o, int64_t i) { return float((v[min(i, a.m2 - 1)] + o) * a.scale); };
     const float2 px = make_float2(coord(x2, a.ox, p0 + lane), coord(x2, a.ox, p0 + 32 + lane));
     const float2 py = make_float2(coord(y2, a.oy, p0 + lane), coord(y2, a.oy, p0 + 32 + lane));
-    const float2 z = f2_dup(float(a.z)), z2 = f2_dup(float(a.z) * float(a.z));
-    const float2 il2 = f2_dup(float(2.0 * a.il)), zf2 = f2_dup(float(2.0 * a.zfrac));   // phases in half-turns
-    const float2 zk = f2_dup(float(a.z * a.k)), nzk = f2_dup(-float(a.z * a.k));
-    const float2 one = f2_dup(1.f), none = f2_dup(-1.f), half = f2_dup(0.5f), magic = f2_dup(12582912.f);
-    const float2 zero = make_float2(0.f, 0.f);
-    float2 rr = zero, ii = zero, im = zero;   // sums of re re, im im and of the imaginary part
+    const float z = float(a.z), zk = float(a.z * a.k);
+    const Consts32 k{f2_dup(z), f2_dup(z * z), f2_dup(float(2.0 * a.il)), f2_dup(float(2.0 * a.zfrac)), f2_dup(zk),
+                     f2_dup(-zk)};
+    Sums32 sum{make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+    // the points lie within `reach` of the first one per axis (bits of magnitudes: a NaN tops all),
+    // sources within `near` of it are near all of them
+    const float cx = __shfl_sync(0xffffffffu, px.x, 0), cy = __shfl_sync(0xffffffffu, py.x, 0);
+    auto off = [](float v, float c) { return __float_as_uint(v - c) & 0x7fffffffu; };
+    const float reach = __uint_as_float(__reduce_max_sync(
+        0xffffffffu, max(max(off(px.x, cx), off(px.y, cx)), max(off(py.x, cy), off(py.y, cy)))));
+    const float near = a.near - reach;
     for (int64_t base = int64_t(rank) * kTile; base < a.m1; base += int64_t(split) * kTile) {
         const int64_t j = base + threadIdx.x;
-        float4 ps = make_float4(0.f, 0.f, 0.f, 0.f), vs = ps;
+        float4 ps = make_float4(cx, cx, cy, cy), vs = make_float4(0.f, 0.f, 0.f, 0.f);
         if (j < a.m1) {
             const float2 v = c[j];
             const float w = float(area[j]), sx = float(x1[j] * a.scale), sy = float(y1[j] * a.scale);
@@ -127,53 +191,19 @@ __global__ void __launch_bounds__(kThreads, 3) rs_f32_kernel(const double* __res
         __syncthreads();
         pos[threadIdx.x] = ps;
         val[threadIdx.x] = vs;
+        // (a warp's sources are those that its lanes loaded)
+        const bool far = !__all_sync(0xffffffffu, fabsf(ps.x - cx) <= near && fabsf(ps.z - cy) <= near);
         __syncthreads();
         const int q0 = warp * 32, q1 = int(min(int64_t(q0 + 32), a.m1 - base));
-#pragma unroll 2
-        for (int q = q0; q < q1; ++q) {
-            const float4 s = pos[q], v = val[q];
-            const float2 dx = sub2(px, make_float2(s.x, s.y)), dy = sub2(py, make_float2(s.z, s.w));
-            const float2 rho2 = fma2(dx, dx, mul2(dy, dy));
-            const float2 d2 = add2(rho2, z2);
-            // r = sqrt(d2) and d = rho^2 / (r + z), each an approximation and one
-            // step with the exact remainder (Markstein)
-            const float2 y = make_float2(rsqrt_fast(d2.x), rsqrt_fast(d2.y));
-            const float2 r0 = mul2(d2, y);
-            const float2 r = fma2(fma2(mul2(r0, none), r0, d2), mul2(y, half), r0);
-            const float2 t = add2(r, z);
-            const float2 rc = make_float2(rcp_fast(t.x), rcp_fast(t.y));
-            const float2 g = mul2(rho2, rc);
-            const float2 d = fma2(fma2(mul2(g, none), t, rho2), rc, g);
-            // half-turns: the nearest integer n and the rest
-            const float2 ph = fma2(d, il2, zf2);
-            const float2 kb = add2(ph, magic);
-            const float2 x = sub2(ph, sub2(kb, magic));
-            const float2 u = mul2(x, x);
-            float2 cs = fma2(f2_dup(-0.024395931512117386f), u, f2_dup(0.23493707180023193f));
-            cs = fma2(cs, u, f2_dup(-1.335211992263794f));
-            cs = fma2(cs, u, f2_dup(4.058709144592285f));
-            cs = fma2(cs, u, f2_dup(-4.934802055358887f));
-            cs = fma2(cs, u, one);
-            float2 sn = fma2(f2_dup(0.07765591144561768f), u, f2_dup(-0.5982903838157654f));
-            sn = fma2(sn, u, f2_dup(2.550077438354492f));
-            sn = fma2(sn, u, f2_dup(-5.167710304260254f));
-            sn = mul2(x, fma2(sn, u, f2_dup(3.1415927410125732f)));
-            // +- 1 / r^2, the sign (-1)^n
-            float2 w = make_float2(rcp_fast(d2.x), rcp_fast(d2.y));
-            w.x = __uint_as_float(__float_as_uint(w.x) ^ (__float_as_uint(kb.x) << 31));
-            w.y = __uint_as_float(__float_as_uint(w.y) ^ (__float_as_uint(kb.y) << 31));
-            // z/r^3 (1 - i k r)(cs + i sn) = (z/r^3 cs + z k/r^2 sn) + i (z/r^3 sn - z k/r^2 cs)
-            const float2 A = mul2(mul2(w, make_float2(fabsf(w.x), fabsf(w.y))), mul2(r, z));
-            const float2 kre = fma2(A, cs, mul2(mul2(w, zk), sn));
-            const float2 kim = fma2(A, sn, mul2(mul2(w, nzk), cs));
-            const float2 vr = make_float2(v.x, v.y), vi = make_float2(v.z, v.w);
-            rr = fma2(vr, kre, rr);
-            ii = fma2(vi, kim, ii);
-            im = fma2(vr, kim, fma2(vi, kre, im));
+        if (far) {
+            sum = rs_far32(pos + q0, val + q0, q1 - q0, px, py, k, sum);
+            continue;
         }
+#pragma unroll 4
+        for (int q = q0; q < q1; ++q) rs_pair32<false>(pos[q], val[q], px, py, k, sum);
     }
-    acc[warp][lane] = make_float2(rr.x - ii.x, im.x);
-    acc[warp][32 + lane] = make_float2(rr.y - ii.y, im.y);
+    acc[warp][lane] = make_float2(sum.rr.x - sum.ii.x, sum.im.x);
+    acc[warp][32 + lane] = make_float2(sum.rr.y - sum.ii.y, sum.im.y);
     __syncthreads();
     if (threadIdx.x < kPts32) {
         float2 t = acc[0][threadIdx.x];
@@ -411,6 +441,9 @@ extern "C" nuasm_status nuasm_rs_direct(const nuasm_params_t* p, int64_t m1, con
     uint64_t limbits;
     std::memcpy(&limbits, &lim, sizeof(limbits));
     a.rho2_max = unsigned(limbits >> 32);
+    // |2 (d / lambda + zfrac)| < 2^22 - 1 up to d (2^-16 below it for FP32's roundings); rho^2 = d (d + 2 z)
+    const double d = (4194302.0 - 64.0) / (2.0 * a.il);
+    a.near = float(std::fmin(std::sqrt(0.5 * d) * std::sqrt(d + 2.0 * a.z), 1e19));
     a.m1 = m1;
     a.m2 = m2;
     const bool f64 = p->prec == NUASM_PREC_F64;
