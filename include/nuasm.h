@@ -125,8 +125,10 @@ typedef struct {
     int32_t interp_chunk;  /* type-2 interpolation: 0 = the library's rule (tiles of side 16 and 32
                               that hold far more than their share are split); N >= 64 = a tile with
                               more than N home records is split into chunks of at most N
-                              (rounded up to a multiple of 32), one CTA each.  Results are the
-                              same bit for bit; values 1..63 or < 0 return NUASM_EINVAL. */
+                              (rounded up to a multiple of 32), one CTA each, so one CTA per
+                              tile with any N from the number of points up (INT32_MAX too).
+                              Results are the same bit for bit; values 1..63 or < 0 return
+                              NUASM_EINVAL. */
     int32_t spread_chunk;  /* type-1 spreading, for the kernels that can split a tile (FP64, and
                               FP32 tiles of side <= 32): 0 = the library's rule (a tile with
                               more records than the larger of 128 (FP64) / 1024 (FP32) and an

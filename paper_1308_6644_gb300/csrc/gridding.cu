@@ -1858,7 +1858,8 @@ cudaError_t make_tile_order(nuasm_plan_s* P, cudaStream_t st) {
             if (b == e2) continue;   // no home records: nothing to interpolate
             // chunks start on a multiple of 32 records from the tile start: the record order's
             // bank classes repeat every 32 records, so each warp keeps its distinct classes
-            const int pieces = (e2 - b + ch - 1) / ch, step = (((e2 - b + pieces - 1) / pieces) + 31) & ~31;
+            // (ch may be any int, so no sum with it)
+            const int pieces = (e2 - b - 1) / ch + 1, step = (((e2 - b + pieces - 1) / pieces) + 31) & ~31;
             for (int s = b; s < e2; s += step) items.push_back(make_int4(t, s, std::min(e2, s + step), 0));
         }
         std::stable_sort(items.begin(), items.end(), [](const int4& a, const int4& b) { return a.z - a.y > b.z - b.y; });
