@@ -739,11 +739,14 @@ __global__ void __launch_bounds__(NT, fixed_minb(WMAX) * 256 / NT) spread_fixed_
 }
 
 // Plan time (FP32): each tile's load, the largest sum over its records of wx wy
-// at one cell, rounded up.  Sums in units of 2^-14 fit int32 for 2^17 records at one cell; tiles with more
+// at one cell, rounded up, and in *clash (where it is not null) whether any warp of
+// spread_private_kernel would take two records of one first-tap cell together.
+// Sums in units of 2^-14 fit int32 for 2^17 records at one cell; tiles with more
 // records take their count.
 template <int WMAX, bool EXACT>
 __global__ void __launch_bounds__(256) tile_load_kernel(const RecF* __restrict__ rec, const int* __restrict__ off,
-                                                        GridArgs a, const KernelPoly kp, float* __restrict__ load) {
+                                                        GridArgs a, const KernelPoly kp, float* __restrict__ load,
+                                                        int* __restrict__ clash) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ int red[8];
     const int tile = blockIdx.x, b = off[tile], e = off[tile + 1];
@@ -754,9 +757,19 @@ __global__ void __launch_bounds__(256) tile_load_kernel(const RecF* __restrict__
     for (int i = threadIdx.x; i < TT; i += 256) sum[i] = 0;
     __syncthreads();
     const bool count = e - b > 100000;
-    for (int i = b + threadIdx.x; i < e && !count; i += 256) {
-        if (!NUASM_IN_RANGE(i, a.nrec, dbg::kSpreadRec)) continue;
-        const RecF r = rec[i];
+    bool met = count;
+    const int lane = threadIdx.x & 31;
+    for (int i0 = b + int(threadIdx.x) - lane; i0 < e && !count; i0 += 256) {
+        const int i = i0 + lane;
+        const bool live = i < e && NUASM_IN_RANGE(i, a.nrec, dbg::kSpreadRec);
+        RecF r{};
+        if (live) r = rec[i];
+        if (clash) {
+            const unsigned key = live ? r.cell : 0xffffffffu - unsigned(lane);
+            const unsigned peers = __match_any_sync(0xffffffffu, key);   // every lane of the warp, every time
+            met |= __popc(peers) > 1;
+        }
+        if (!live) continue;
         const int lx = int(r.cell & 0xffffu) - x0, ly = int(r.cell >> 16) - y0;
         float wx[WMAX], wy[WMAX];
         tap_weights<WMAX>(r.fx, kp, wx);
@@ -774,10 +787,11 @@ __global__ void __launch_bounds__(256) tile_load_kernel(const RecF* __restrict__
         }
     }
     __syncthreads();
+    if (clash && met) *clash = 1;
     int top = 0;
     for (int i = threadIdx.x; i < TT; i += 256) top = max(top, sum[i]);
     top = __reduce_max_sync(0xffffffffu, top);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = top;
+    if (lane == 0) red[threadIdx.x >> 5] = top;
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int k = 1; k < 8; ++k) top = max(top, red[k]);
@@ -1588,15 +1602,36 @@ cudaError_t spread_impl(const nuasm_plan_s* P, const void* c, cudaStream_t st) {
         cudaError_t e = clear();
         if (e != cudaSuccess) return e;
     }
+    const auto* rec = static_cast<const typename RecOf<S>::type*>(P->d.rec);
+    const V* src = static_cast<const V*>(c);
+    V* win = static_cast<V*>(P->d.win);
+    auto private_copies = [&]() -> cudaError_t {
+        const size_t sm = size_t(8) * a.T * plane_stride(a.T, a.max_skew) * sizeof(V);
+        cudaError_t e = set_smem(spread_private_kernel<S, WMAX, EXACT>, sm);
+        if (e != cudaSuccess) return e;
+        spread_private_kernel<S, WMAX, EXACT><<<grid, 256, sm, st>>>(rec, P->d.tile_off, P->d.wpt, P->d.tile_order, src,
+                                                                     win, a, taps_arg<S>(P), items, expo);
+        return cudaGetLastError();
+    };
     if constexpr (sizeof(S) == 4) {
+        // Warp-private copies where the order of the points keeps records of one cell
+        // apart (lattices, a pitch per quadrant) and the tiles fill the chip at most
+        // twice over or are dense: no reduction over the CTA, no conversions, no
+        // atomics.  Against int32 sums, us: quadrant pitches N = 64 and 128 8.7 and 9.0 /
+        // 11.9 and 12.0, N = 256 (1089 tiles, up to 256 records) 13.4 / 14.6; lattices N =
+        // 64 8.6 / 9.5, 128 8.5 / 9.9, 256 of 484 records a tile 23.4 / 24.6, but of 121
+        // 14.6 / 12.7, and side 32 33.7 / 23.1.  Jittered points, whose records meet in
+        // every warp: N = 64 18.5 / 9.7, 256 27.4 / 12.7.
+        if constexpr (EXACT)
+            if (P->distinct_cells && (P->g.ntiles <= 2 * 152 || P->max_tile_rec > 128)) return private_copies();
         auto fixed = [&](auto threads) -> cudaError_t {
             constexpr int RPB = NUASM_SPREAD_FIXED_RPB, NT = decltype(threads)::value;
             const size_t sm = size_t(2) * a.T * plane_stride(a.T, a.max_skew) * sizeof(int);
             cudaError_t e = set_smem(spread_fixed_kernel<WMAX, EXACT, RPB, NT>, sm);
             if (e != cudaSuccess) return e;
-            spread_fixed_kernel<WMAX, EXACT, RPB, NT><<<grid, NT, sm, st>>>(
-                static_cast<const RecF*>(P->d.rec), P->d.tile_off, P->d.wpt, P->d.tile_order, P->d.tile_load,
-                static_cast<const float2*>(c), static_cast<float2*>(P->d.win), a, taps_arg<S>(P), items);
+            spread_fixed_kernel<WMAX, EXACT, RPB, NT><<<grid, NT, sm, st>>>(rec, P->d.tile_off, P->d.wpt,
+                                                                            P->d.tile_order, P->d.tile_load, src, win,
+                                                                            a, taps_arg<S>(P), items);
             return cudaGetLastError();
         };
         // tiles of side 16 with at most two records a thread in the fullest (kept
@@ -1606,22 +1641,13 @@ cudaError_t spread_impl(const nuasm_plan_s* P, const void* c, cudaStream_t st) {
         if (a.T <= 16 && P->max_tile_rec <= 256) return fixed(std::integral_constant<int, 128>{});
         return fixed(std::integral_constant<int, 256>{});
     } else {
-        if (a.T <= 16) {
-            const size_t sm = size_t(8) * a.T * plane_stride(a.T, a.max_skew) * sizeof(V);
-            cudaError_t e = set_smem(spread_private_kernel<S, WMAX, EXACT>, sm);
-            if (e != cudaSuccess) return e;
-            spread_private_kernel<S, WMAX, EXACT><<<grid, 256, sm, st>>>(
-                static_cast<const typename RecOf<S>::type*>(P->d.rec), P->d.tile_off, P->d.wpt, P->d.tile_order,
-                static_cast<const V*>(c), static_cast<V*>(P->d.win), a, taps_arg<S>(P), items, expo);
-            return cudaGetLastError();
-        }
-    const size_t sm = size_t(2) * a.T * plane_stride(a.T, a.max_skew) * sizeof(S);
-    cudaError_t e = set_smem(spread_kernel<S, WMAX, EXACT>, sm);
-    if (e != cudaSuccess) return e;
-    spread_kernel<S, WMAX, EXACT><<<grid, 256, sm, st>>>(
-        static_cast<const typename RecOf<S>::type*>(P->d.rec), P->d.tile_off, P->d.wpt, P->d.tile_order,
-        static_cast<const V*>(c), static_cast<V*>(P->d.win), a, taps_arg<S>(P), items, expo);
-    return cudaGetLastError();
+        if (a.T <= 16) return private_copies();
+        const size_t sm = size_t(2) * a.T * plane_stride(a.T, a.max_skew) * sizeof(S);
+        cudaError_t e = set_smem(spread_kernel<S, WMAX, EXACT>, sm);
+        if (e != cudaSuccess) return e;
+        spread_kernel<S, WMAX, EXACT><<<grid, 256, sm, st>>>(rec, P->d.tile_off, P->d.wpt, P->d.tile_order, src, win, a,
+                                                             taps_arg<S>(P), items, expo);
+        return cudaGetLastError();
     }
 }
 
@@ -1731,10 +1757,17 @@ template <bool SPREAD> cudaError_t gridding(const nuasm_plan_s* P, const void* i
     }
 }
 
-// Fill the plan's tile loads (FP32).
+// Fill the plan's tile loads (FP32) and, on tiles of side 16, find out whether its
+// order keeps records of one cell apart in spreading.
 cudaError_t fill_tile_load(nuasm_plan_s* P, cudaStream_t st) {
     if (P->f64) return cudaSuccess;
     const GridArgs a = grid_args(P);
+    int* clash = nullptr;
+    if (P->g.T == 16 && !P->d.spread_items) {
+        clash = reinterpret_cast<int*>(P->d.tile_load + P->g.ntiles);
+        const cudaError_t err = cudaMemsetAsync(clash, 0, sizeof(int), st);
+        if (err != cudaSuccess) return err;
+    }
     auto run = [&](auto tag) -> cudaError_t {
         using Tg = decltype(tag);
         auto kernel = tile_load_kernel<Tg::W, Tg::X>;
@@ -1742,17 +1775,24 @@ cudaError_t fill_tile_load(nuasm_plan_s* P, cudaStream_t st) {
         cudaError_t err = set_smem(kernel, sm);
         if (err != cudaSuccess) return err;
         kernel<<<P->g.ntiles, 256, sm, st>>>(static_cast<const RecF*>(P->d.rec), P->d.tile_off, a, P->poly,
-                                             P->d.tile_load);
+                                             P->d.tile_load, clash);
         return cudaGetLastError();
     };
+    cudaError_t e;
     switch (P->g.w) {
-        case 4: return run(GTag<float, 4, true>{});
-        case 5: return run(GTag<float, 5, true>{});
-        case 6: return run(GTag<float, 6, true>{});
-        case 7: return run(GTag<float, 7, true>{});
-        case 8: return run(GTag<float, 8, true>{});
-        default: return P->g.w <= 16 ? run(GTag<float, 16, false>{}) : run(GTag<float, kPolyMaxW, false>{});
+        case 4: e = run(GTag<float, 4, true>{}); break;
+        case 5: e = run(GTag<float, 5, true>{}); break;
+        case 6: e = run(GTag<float, 6, true>{}); break;
+        case 7: e = run(GTag<float, 7, true>{}); break;
+        case 8: e = run(GTag<float, 8, true>{}); break;
+        default: e = P->g.w <= 16 ? run(GTag<float, 16, false>{}) : run(GTag<float, kPolyMaxW, false>{});
     }
+    if (e != cudaSuccess || !clash) return e;
+    int met = 1;
+    e = cudaMemcpyAsync(&met, clash, sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (e != cudaSuccess || (e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
+    P->distinct_cells = met == 0;
+    return cudaSuccess;
 }
 
 }  // namespace
@@ -1790,8 +1830,8 @@ cudaError_t make_tile_order(nuasm_plan_s* P, cudaStream_t st) {
     std::stable_sort(order.begin(), order.end(),
                      [&](int a, int b) { return off[a + 1] - off[a] > off[b + 1] - off[b]; });
     P->max_tile_rec = off[order[0] + 1] - off[order[0]];
-    // the tiles with their record ranges, then their loads (fill_tile_load)
-    const size_t bytes = (sizeof(int4) + sizeof(float)) * size_t(nt);
+    // the tiles with their record ranges, then their loads and a word (fill_tile_load)
+    const size_t bytes = (sizeof(int4) + sizeof(float)) * size_t(nt) + sizeof(int);
     if ((e = xmalloc(reinterpret_cast<void**>(&P->d.tile_order), bytes)) != cudaSuccess) return e;
     P->d.tile_load = reinterpret_cast<float*>(P->d.tile_order + nt);
     P->device_bytes += int64_t(bytes);

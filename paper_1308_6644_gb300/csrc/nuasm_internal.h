@@ -116,6 +116,7 @@ struct nuasm_plan_s {
     int n_interp_items = 0;     // entries of d.interp_items
     int n_spread_items = 0;     // entries of d.spread_items
     int max_tile_rec = 0;       // records of the fullest tile
+    bool distinct_cells = false;    // FP32, side 16: no 32 records that a warp spreads together share a first-tap cell
     nuasm::KernelPoly poly{};   // kernel taps as polynomials (F32 gridding)
     nuasm::KernelPoly64 poly64{};   // the same in FP64 (F64 gridding)
     nuasm::KernelPolyDF poly64df{};   // poly64 as float pairs (F64 gridding in double-float arithmetic)
