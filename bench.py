@@ -216,13 +216,15 @@ def stage_flops(info: dict, m: int, type_: int = 2, f64: bool = False) -> dict:
 
 
 def kernel_of_stage(stage: str, info: dict, f64: bool) -> str:
-    """Name of the kernel a stage launches for this geometry (as ncu lists it)."""
+    """Name of the kernel a stage launches for this geometry (as ncu lists it).
+
+    A built plan's info ("records") with its tolerance ("tol") names what the
+    library launches; a bare geometry the kernels of an FP64 plan below 1e-12 and
+    of ordered points."""
     lognp = int(np.log2(info["n_pad"]))
     v, s = ("double2", "double") if f64 else ("float2", "float")
-    # FP64 FFT passes: double-float, below N' = 512 where the kernel's width (a built
-    # plan's tolerance from 1e-12 up) allows it
     plan = "records" in info
-    rv = "dfc" if f64 and (lognp >= 9 or (plan and info.get("double_float"))) else v
+    rv = "dfc" if f64 and (lognp >= 9 or info.get("tol", 0.0) >= 1e-12) else v   # FP64 FFT passes: double-float
     w = info["kernel_width"]
     if f64:
         tap = f"double, {w}, true" if w in (11, 13) else f"double, {8 if w <= 8 else (16 if w <= 16 else 26)}, false"
@@ -230,6 +232,7 @@ def kernel_of_stage(stage: str, info: dict, f64: bool) -> str:
         tap = f"float, {w}, true" if 4 <= w <= 8 else f"float, {16 if w <= 16 else 26}, false"
     tma = not f64 and 512 <= info["n_pad"] <= 4096          # folded column passes
     tma_wide = not f64 and info["n_pad"] == 4096              # unfolded ones too
+    col = f"col2_kernel<{lognp}, " if not f64 and lognp == 13 else f"col_kernel<{rv}, {lognp}, "   # pairs of columns
     tile = info.get("tile", 64)
     interp = f"interp_kernel<{tap}>"
     if f64 and info.get("double_float"):
@@ -241,15 +244,21 @@ def kernel_of_stage(stage: str, info: dict, f64: bool) -> str:
     elif tile <= 32 and not plan:
         spread = f"spread_private_kernel<{tap}>"
     else:
-        spread = (f"spread_fixed_kernel<{w}, true, 2>" if 4 <= w <= 8 else
-                  f"spread_fixed_kernel<{16 if w <= 16 else 26}, false, 2>")
-    return {"col_fwd": f"col_tma_kernel<{lognp}, 2>" if tma_wide else f"col_kernel<{rv}, {lognp}, 2>",
+        spread = (f"spread_fixed_kernel<{w}, true, 2" if 4 <= w <= 8 else
+                  f"spread_fixed_kernel<{16 if w <= 16 else 26}, false, 2")
+        if not plan:
+            spread += ">"
+        elif tile > 16:
+            spread += ", 256>"
+        else:   # 128 threads where the fullest tile has up to 256 records; warp-private copies for ordered points
+            spread = f"{spread}, 128>, {spread}, 256> or spread_private_kernel<{tap}>"
+    return {"col_fwd": f"col_tma_kernel<{lognp}, 2>" if tma_wide else f"{col}2>",
             "row_t2": f"row_t2_kernel<{rv}, {lognp}>",
-            "col_inv_fold": f"col_tma_kernel<{lognp}, 3>" if tma else f"col_kernel<{rv}, {lognp}, 3>",
+            "col_inv_fold": f"col_tma_kernel<{lognp}, 3>" if tma else f"{col}3>",
             "interp": interp, "spread": spread,
-            "col_fwd_fold": f"col_tma_kernel<{lognp}, 0>" if tma else f"col_kernel<{rv}, {lognp}, 0>",
+            "col_fwd_fold": f"col_tma_kernel<{lognp}, 0>" if tma else f"{col}0>",
             "row_t1": f"row_t1_kernel<{rv}, {lognp}>",
-            "col_inv": f"col_tma_kernel<{lognp}, 1>" if tma_wide else f"col_kernel<{rv}, {lognp}, 1>"}[stage]
+            "col_inv": f"col_tma_kernel<{lognp}, 1>" if tma_wide else f"{col}1>"}[stage]
 
 
 _FFT_SOURCES = ["passes.cuh", "fft_engine.cuh", "tma.cuh", "dfloat.cuh"]
@@ -456,7 +465,7 @@ def run_ours(args):
     t_plan0 = time.perf_counter()
     plan = P.nuasm_plan(params, x, y, wts, stream=stream)
     plan_s = time.perf_counter() - t_plan0
-    info = plan.info()
+    info = dict(plan.info(), tol=params.tol or (1e-12 if f64 else 1e-6))
     n_out = wl.n * wl.n if wl.type == 1 else wl.m
     inp = torch.from_numpy(np.ascontiguousarray(np.asarray(wl.values).astype(cdt).reshape(-1))).to(dev)
     out = torch.empty(n_out, dtype=tdt, device=dev)
