@@ -396,7 +396,7 @@ nuasm_status nuasm::plan_create(nuasm_plan_s** out, const nuasm_params_t* p, int
             if ((e = dalloc(P, &P->d.etab, ne * eb)) != cudaSuccess) return bail(cuda_status(e));
             if ((e = build_etab(P, st)) != cudaSuccess) return bail(cuda_status(e));
             if (NUASM_ETAB2 && !P->f64 && g.np <= 4096) {
-                // type 2's row pass stages T2x E rows (merged row engines: N' <= 4096 in FP32)
+                // rows of T2x E, which type 2's row pass stages up to N' = 4096
                 const size_t n2 = size_t(g.np / 2 + 1) * g.np;
                 if ((e = dalloc(P, &P->d.etab2, n2 * eb)) != cudaSuccess) return bail(cuda_status(e));
                 if ((e = build_etab2(P, st)) != cudaSuccess) return bail(cuda_status(e));

@@ -29,7 +29,9 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src)
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// `early` asks for it (launch_early in nuasm_internal.h).
+// A launch that may start before the stream's previous kernel has finished where
+// `early` says so (launch_early in nuasm_internal.h): the kernel then waits with
+// pdl_wait before it touches what the previous one writes.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_chained(bool early, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                            Args&&... args) {
@@ -42,7 +44,7 @@ cudaError_t launch_chained(bool early, void (*kernel)(KArgs...), dim3 grid, dim3
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-        cfg.numAttrs = early ? 1 : 0;
+    cfg.numAttrs = early ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 

@@ -55,8 +55,12 @@ template <int DIR> __device__ __forceinline__ dfc cadd_i(dfc a, dfc b) {
     const float2 e = add2(sub2(a.h, add2(s, nb)), fma2(bh, sg, nb));
     return dfc_renorm(s, add2(e, fma2(bl, sg, a.l)));
 }
-// a r for a real constant r (the product and its error in scalar FMAs: the
-// packed fma of a, r and the packed product of a and -r came back as zero)
+// a r for a real constant r.  The product and its error are scalar, which is no
+// slower (row and column passes of the N = 2048 plane: the same 3.73 ms a solve with
+// packed ones).  In a packed form the fma's addend has to be the product with its
+// sign flipped: CUDA 13.0's assembler takes fma2(a, R, mul2(a, -R)), two exact
+// operations on a and a constant, for zero (checked on 8192 values, alone in a
+// kernel: off by 1.5e-8; fma2(a, R, -mul2(a, R)) and every scalar mix: 2e-15).
 __device__ __forceinline__ dfc cscale(dfc a, dfr r) {
     const float2 p = make_float2(a.h.x * r.hi, a.h.y * r.hi);
     float2 e = make_float2(fmaf(a.h.x, r.hi, -p.x), fmaf(a.h.y, r.hi, -p.y));

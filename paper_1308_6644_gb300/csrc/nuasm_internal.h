@@ -73,7 +73,7 @@ struct PlanDevice {
     void* etab = nullptr;       // ASM non-separable factor E(|kx|, |ky|): N'/2 + 1 rows of etab_pitch
                                 // entries in the plan precision (null: evaluated per mode)
     void* etab2 = nullptr;      // type 2's T2x(kx) E(|kx|, |ky|): N'/2 + 1 rows of N' entries (FP32 plans
-                                // with merged row engines; null: row_t2 uses etab and T2x)
+                                // up to N' = 4096; null: row_t2 uses etab and T2x)
     void* rec = nullptr;        // binned point records
     double* wpt = nullptr;      // optional per-point weights, in point order
     int* tile_off = nullptr;    // ntiles + 1 offsets into rec
@@ -241,8 +241,11 @@ inline size_t ws_bufB_elems(const Geometry& g) { return size_t(g.np) * g.n + kEx
 // FP64 plans run their FFT passes in double-float arithmetic (passes.cuh): the
 // mode-side arrays bufA and bufB, the transfer-function tables and the twiddles
 // hold pairs of floats (dfc), the window and the caller's arrays FP64.  Its
-// error, about 2e-14, hides behind the gridding's at tolerances down to 1e-12;
-// plans below N' = 512 with a smaller one keep FP64 passes.
+// error, about 2e-14, hides behind the gridding's at tolerances down to 1e-12 (types
+// 1 to 3, N = 32 to 512, tolerances 1e-6, 1e-10 and 1e-12, jittered, clustered and
+// graded points: within 0.7% of FP64 passes' with the ES kernel, either way by up to
+// 6% with the Gaussian's 1e-12); plans below N' = 512 with a smaller one keep FP64
+// passes.
 inline bool fft_double_float(bool f64, int np, double tol) { return f64 && (np >= 512 || tol >= 1e-12); }
 inline bool fft_double_float(const nuasm_plan_s* P) { return fft_double_float(P->f64, P->g.np, P->p.tol); }
 // Whether a solve's kernels after the first launch before the previous one has
@@ -252,11 +255,12 @@ inline bool fft_double_float(const nuasm_plan_s* P) { return fft_double_float(P-
 // 106 -> 97 us, graded ones 107 -> 113); from N' = 4096 on they must not run
 // early: the column passes there write with bulk tensor stores, which the early
 // kernel's wait does not cover (the next pass read stale values).  Chains recorded
-// into a graph (batches too) don't: a replayed graph has smaller gaps, and early
-// launches in it cost more than they hide (solves replayed from a graph, without ->
-// with: N = 256 weighted type 1 24.7 -> 29.9 us, N = 256 type 2 19.0 -> 21.9, N = 512
-// type 1 43.0 -> 45.9, N = 32 15.4 -> 13.3; 12 planes in a batch 709 -> 727).  FP64
-// chains gained 5% at N = 32 and 512 and lost as much at N = 128 and 256.
+// into a graph (batches too) don't: a replayed graph has smaller gaps, and from N =
+// 128 up early launches in it cost more than they hide (solves replayed from a graph,
+// without -> with: N = 256 weighted type 1 24.7 -> 29.9 us, N = 256 type 2 19.0 -> 21.9,
+// N = 512 type 1 43.0 -> 45.9; 12 planes in a batch 709 -> 727).  N = 32 would gain (type
+// 1 18.3 -> 17.8 us, type 2 15.4 -> 13.3) but has no rule of its own.  FP64 chains gained
+// 5% at N = 32 and 512 and lost as much at N = 128 and 256.
 inline bool launch_early(const nuasm_plan_s* P, cudaStream_t st) {
     cudaStreamCaptureStatus recording;
     return !P->f64 && P->g.np <= 1024 && cudaStreamIsCapturing(st, &recording) == cudaSuccess &&

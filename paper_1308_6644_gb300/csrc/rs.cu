@@ -21,7 +21,8 @@
 // 0.18 ms; FP64 16384 x 16384 83.6 -> 13.5 ms, 5001 x 1001 25.5 -> 0.39 ms.
 //
 // Lengths are scaled by the power of two that takes z into [1, 2), so the FP32
-// seeds below neither overflow nor meet subnormals for any unit of length.
+// seeds below neither overflow nor meet subnormals for any unit of length.  (The
+// FP32 kernel's result takes the scaling back as a float: z from 2^-63 to 2^63.)
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
